@@ -86,9 +86,13 @@ int build_plan(const specext_attn_desc* d, AttnPlan* out) {
   p.Hq = d->n_q_heads; p.Hkv = d->n_kv_heads; p.G = G; p.D = d->head_dim;
   p.L = d->prefix_len; p.T = d->n_tree; p.C = d->chunk_size;
   p.rows = G * p.T;
-  // (a tree of more than 64 nodes with head_dim 128 always takes 256-row blocks: the one-CTA kernel keeps
-  // one mask word per node there)
-  p.RB = (p.rows > 128 || (p.D == 128 && p.T > 64)) ? 256 : 128;
+  // Kernel: pairs of CTAs on 256-row blocks for head_dim 128 and more than 128 stacked rows; otherwise one CTA on
+  // 128-row blocks (want != 0 only in the test library).
+  const int want = tuning_kernel();
+  const bool pair = p.D == 128 && p.rows > 128 && want != 2;
+  p.kernel = want == 1 ? 1 : (pair ? 3 : 2);
+  p.RB = pair ? 256 : 128;
+  p.q_rows = p.kernel == 2 && p.D == 128 && p.rows <= 64 ? 64 : 128;
   p.n_rblk = (p.rows + p.RB - 1) / p.RB;
   p.NP = p.Hkv * p.n_rblk;
   p.TPH = (p.L + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS;
@@ -97,10 +101,6 @@ int build_plan(const specext_attn_desc* d, AttnPlan* out) {
   if (U > (1ll << 30)) return SPECEXT_ERR_UNSUPPORTED;
   p.U = (int)U;
   const int min_units = tuning_min_units();
-  const int want = tuning_kernel();
-  const bool pair_ok = p.D == 128 && p.RB == 256;       // what the paired-CTA kernel is built for
-  p.kernel = want == 1 ? 1 : ((want == 0 || want == 3) && pair_ok ? 3 : 2);   // want != 0 only in the test library
-  if (p.kernel == 2 && p.D == 128 && p.T > 64) return SPECEXT_ERR_UNSUPPORTED;  // (only reachable by a test override)
   if (p.kernel == 3) {
     // one worker = a cluster of two CTAs; every problem gets the same number of workers when possible
     const int n_workers = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
@@ -225,7 +225,7 @@ int run_attn(const specext_attn_desc* desc, const void* Q, const void* K_prefix,
 #ifdef SPECEXT_TESTING
   if (p.kernel == 1) e = spx_launch_attn_simt(a, st, &n); else
 #endif
-  e = p.kernel == 3 ? spx_launch_attn_tc2(a, st, &n) : spx_launch_attn_tc(a, st, &n);
+  e = p.kernel == 3 ? spx_launch_attn_tc2(a, st, &n) : spx_launch_verify(a, st, &n);
   if (e == cudaSuccess) e = spx_launch_merge(a, st, &n);
   g_launches.fetch_add(n);
   if (e != cudaSuccess) {

@@ -96,8 +96,8 @@ cudaError_t spx_opt_in_smem(Kernel* kernel, int bytes, SpxOncePerDevice* once) {
 #ifdef SPECEXT_TESTING
 cudaError_t spx_launch_attn_simt(const AttnArgs& a, cudaStream_t st, int* n_launches);   // cross-check kernel, test library only
 #endif
-cudaError_t spx_launch_attn_tc(const AttnArgs& a, cudaStream_t st, int* n_launches);
 cudaError_t spx_launch_attn_tc2(const AttnArgs& a, cudaStream_t st, int* n_launches);
+cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launches);
 cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches);
 
 #endif  // SPECEXT_COMMON_CUH_

@@ -1,0 +1,410 @@
+// Hybrid Tree Attention with one CTA per worker, on the pipeline of core.cuh: split-over-KV partial attention of the
+// stacked (query head x tree node) rows of one KV head, in row blocks of 128, against 128-key tiles of the prefix and the
+// tree.  Taken for head_dim 64 and for at most 128 stacked rows: targets without grouped heads, single-token steps, draft
+// models.  (More rows with head_dim 128 go to the pairs of attn_tc2.cu.)
+//
+// A worker owns a range of (problem, key tile) units; the part of the range inside one problem is a segment and ends with
+// one partial result (unnormalised O, reference maximum, row sum) in the workspace.
+//
+// What bounds it: memory.  A K/V tile of 64 KB is 3.0 K cycles of an SM's share of the copy rate, a softmax warpgroup
+// needs ~3.3 K for a tile and two alternate.  Measured (us per call, replayed; before: two row tiles of one CTA, whose
+// second softmax warpgroup had nothing to do here and whose S, P and PV of a tile formed one chain):
+//   32 heads of their own, 60 nodes, 8K prefix    40.3 -> 30.5 (scored 62.5 -> 35.1)   4.4 TB/s of K/V; 16K 64.9 -> 50.5
+//   32 query / 8 KV heads, one node, 16K prefix   27.9 -> 20.0 (scored 37.5 -> 22.7)   128K 113.8 -> 88.8 = 6.0 TB/s
+//   12 heads x 64, 8 nodes, 4K prefix             15.6 -> 11.8
+//
+// Warps: 0-7 softmax (two warpgroups), 8 TMA producer of K and V, 9 issuer of the S MMAs, 10 of the PV MMAs, 11 ancestor
+// masks of the tree and TMA producer of Q.  Every wait is bounded; an expired wait raises SPECEXT_ERR_TIMEOUT, and all
+// threads reach the final barrier before tensor memory is freed.
+//
+// The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory allocation and the
+// start-up barrier run while the kernel before it in the stream finishes; global memory is touched only after
+// griddepcontrol.wait.
+#include "common.cuh"
+#include "core.cuh"
+#include "tmap.h"
+
+using namespace core;
+
+namespace {
+
+struct VerifyMaps {
+  CUtensorMap q, kp, vp, kt, vt;
+};
+
+// The segments of a worker's unit range, in order.
+template <bool DEVLEN>
+struct VerifyWork {
+  const AttnPlan& p;
+  int u, hi, tph_eff;
+  int prob, tile_lo, n;
+  SpxSeg sg;
+  __device__ __forceinline__ VerifyWork(const AttnPlan& plan, int lo, int hi_, int tph) : p(plan), u(lo), hi(hi_), tph_eff(tph) {}
+  // next segment, an empty one (no tile of it exists at the device-side length) included
+  __device__ __forceinline__ bool next_any() {
+    if (u >= hi) return false;
+    prob = u / p.UPP;
+    tile_lo = u - prob * p.UPP;
+    const int n_units = min(p.UPP - tile_lo, hi - u);
+    u += n_units;
+    n = n_units;
+    if (DEVLEN) {
+      sg = spx_segment(p, tile_lo, n_units, tph_eff);
+      n = sg.n;
+    }
+    return true;
+  }
+  __device__ __forceinline__ bool next() {
+    while (next_any())
+      if (!DEVLEN || n > 0) return true;
+    return false;
+  }
+  __device__ __forceinline__ int tile(int j) const { return DEVLEN ? spx_seg_tile(p, sg, tile_lo, j) : tile_lo + j; }
+};
+
+// SCORE: 0 no chunk sums; otherwise the class of the chunk size, so that each variant carries only the code it runs:
+// 1 chunks of 32 keys, 2 chunks of 64 or 128 keys, 3 chunks of fewer than 32 keys.
+// DEVLEN: the prefix length is read from device memory (a.L_dev) and may be shorter than the planned capacity p.L; the
+// instantiation without it carries none of that code.
+template <int D, int SCORE, bool DEVLEN>
+__global__ void __launch_bounds__(kThreads, 1)
+verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ VerifyMaps maps) {
+  using G = Geo<1, D>;
+  const AttnPlan& p = a.plan;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                         ~static_cast<uintptr_t>(1023));
+  Ctrl* ctl = reinterpret_cast<Ctrl*>(base + G::kCtrlOffset);
+  volatile int* abort_flag = &ctl->abort_flag;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const G geo(p.q_rows);
+
+  setup_begin<1>(ctl, warp, lane);
+  // The kernel after this one (the merge) may be set up while this one runs; this one touches global memory only once
+  // the kernel before it has completed (its set-up so far has used none).
+  pdl_launch_dependents();
+  pdl_wait();
+
+  const int worker = blockIdx.x;
+  const int unit_lo = spx_unit_start(p, worker), unit_hi = spx_unit_start(p, worker + 1);
+  if (warp == kProducerWarp && lane == 0 && unit_lo < unit_hi && !DEVLEN) {
+    // The first K/V tile can only be loaded once the barriers are known to exist; until then it is pulled into L2.
+    const int prob = unit_lo / p.UPP, tile = unit_lo - prob * p.UPP, g = prob / p.n_rblk;
+    const bool is_tree = tile == p.TPH;
+    const int key0 = is_tree ? 0 : tile * SPX_TILE_KEYS;
+    for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.kt : &maps.kp, 64 * ds, g, key0);
+    for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * ds, g, key0);
+  }
+  setup_wait<1>();
+
+  const int L_eff = DEVLEN ? spx_prefix_len(a) : p.L;
+  const int tph_eff = DEVLEN ? (L_eff + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS : p.TPH;
+  VerifyWork<DEVLEN> work(p, unit_lo, unit_hi, tph_eff);
+  bool ok = true;
+
+  if (warp == kProducerWarp) {
+    // ================================ TMA producer of K and V ================================
+    setmaxnreg_dec<kRegsOther>();
+    if (lane == 0) {
+      const uint64_t stream_once = policy_evict_first();
+      const uint32_t kfull0 = smem_u32(&ctl->k_full[0]), vfull0 = smem_u32(&ctl->v_full[0]);
+      unsigned char* kring = base + geo.k_off;
+      unsigned char* vring = base + geo.v_off;
+      int kst = 0, vst = 0, n_done = 0;
+      uint32_t kph = 1, vph = 1, n_rag = 0;
+      while (ok && work.next()) {
+        const int g = work.prob / p.n_rblk;
+        for (int j = 0; j < work.n && ok; ++j) {
+          const int tile = work.tile(j);
+          const bool is_tree = tile == p.TPH;
+          const int key0 = is_tree ? 0 : tile * SPX_TILE_KEYS;
+          // Start-up: only two tiles are requested until the first S MMA has consumed K tile 0.  A full ring requested
+          // at once by every SM sits in the memory system's queues in no particular order, and tile 0 would arrive
+          // last as often as first.
+          if (n_done == 2) ok = wait_c(&ctl->k_empty[0], 0, abort_flag);
+          if (ok) ok = wait_c(&ctl->k_empty[kst], kph, abort_flag);
+          if (!ok) break;
+          {
+            const uint32_t bar = kfull0 + kst * 8, dst = smem_u32(kring + kst * G::kKStage);
+            const CUtensorMap* m = is_tree ? &maps.kt : &maps.kp;
+            arrive_expect_tx_cluster(bar, G::kKStage);
+#pragma unroll
+            for (int ds = 0; ds < G::kBlocks; ++ds) {
+              // (no eviction hint with a device-side length: a compact cache is read again at the next draft step)
+              if (DEVLEN) tma_load<1>(dst + ds * G::kKBlk, m, bar, 64 * ds, g, key0);
+              else tma_load_hint<1>(dst + ds * G::kKBlk, m, bar, 64 * ds, g, key0, stream_once);
+            }
+          }
+          if (++kst == geo.nk) {
+            kst = 0;
+            kph ^= 1;
+          }
+          ok = wait_c(&ctl->v_empty[vst], vph, abort_flag);
+          if (!ok) break;
+          {
+            const uint32_t bar = vfull0 + vst * 8;
+            unsigned char* dst = vring + vst * G::kVStage;
+            const CUtensorMap* m = is_tree ? &maps.vt : &maps.vp;
+            const int nk = is_tree ? SPX_TILE_KEYS : L_eff - tile * SPX_TILE_KEYS;
+            if (DEVLEN && nk < SPX_TILE_KEYS) {
+              // Device-side length: the tensor map spans the whole capacity, so the rows of this tile past the length
+              // hold whatever the cache holds (their probabilities are zero, but zero times a NaN is a NaN).  The tile
+              // lands on a barrier of its own, its tail rows are cleared (a row of a block is 128 bytes whatever the
+              // swizzle), and only then is the stage handed to the MMA issuer.
+              mbar_arrive_expect_tx(&ctl->v_rag, G::kVStage);
+              for (int ds = 0; ds < G::kBlocks; ++ds) tma_load_3d(dst + ds * G::kVBlk, m, &ctl->v_rag, 64 * ds, g, key0);
+              ok = mbar_wait(&ctl->v_rag, n_rag & 1, abort_flag);
+              if (!ok) break;
+              ++n_rag;
+              for (int ds = 0; ds < G::kBlocks; ++ds) {
+                uint4* tail = reinterpret_cast<uint4*>(dst + ds * G::kVBlk + nk * 128);
+                for (int i = 0; i < (SPX_TILE_KEYS - nk) * 8; ++i) tail[i] = make_uint4(0u, 0u, 0u, 0u);
+              }
+              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+              mbar_arrive(&ctl->v_full[vst]);
+            } else {
+              arrive_expect_tx_cluster(bar, G::kVStage);
+#pragma unroll
+              for (int ds = 0; ds < G::kBlocks; ++ds) {
+                const uint32_t d = smem_u32(dst + ds * G::kVBlk);
+                if (DEVLEN) tma_load<1>(d, m, bar, 64 * ds, g, key0);
+                else tma_load_hint<1>(d, m, bar, 64 * ds, g, key0, stream_once);
+              }
+            }
+          }
+          if (++vst == geo.nv) {
+            vst = 0;
+            vph ^= 1;
+          }
+          ++n_done;
+        }
+      }
+    }
+  } else if (warp == kMmaWarp) {
+    setmaxnreg_dec<kRegsOther>();
+    if (lane == 0) ok = issue_s<1, D>(ctl, base, geo, work, abort_flag);
+  } else if (warp == kPvWarp) {
+    setmaxnreg_dec<kRegsOther>();
+    if (lane == 0) ok = issue_pv<1, D>(ctl, base, geo, work, abort_flag);
+  } else if (warp == kTreeWarp) {
+    // ================================ ancestor masks, TMA producer of Q =======================
+    setmaxnreg_dec<kRegsOther>();
+    // boxes of 64 elements x G heads x q_rows/G nodes: exactly the stacked rows (G is a power of two), rows past the
+    // tree zero-filled
+    const uint32_t q_bar = smem_u32(&ctl->q_full);
+    auto load_q = [&]() {
+      const int g = work.prob / p.n_rblk, rblk = work.prob - g * p.n_rblk;
+      arrive_expect_tx_cluster(q_bar, geo.q_blk * G::kBlocks);
+#pragma unroll
+      for (int ds = 0; ds < G::kBlocks; ++ds)
+        tma_load<1>(smem_u32(base + ds * geo.q_blk), &maps.q, q_bar, 64 * ds, g * p.G, rblk * p.RB / p.G);
+    };
+    if (lane == 0 && work.next()) load_q();              // the first segment's; later ones below
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < kSpxMaxTree / 32; ++q) ctl->parent[lane + 32 * q] = lane + 32 * q < p.T ? a.parent[lane + 32 * q] : -1;
+    __syncwarp();
+    bool bad = false;
+#pragma unroll 1
+    for (int q = 0; q < kSpxMaxTree / 32; ++q) {
+      const int t = lane + 32 * q;
+      SpxMask128 m = {0ull, 0ull};
+      if (t < p.T) m = spx_walk_up(ctl->parent, p.T, t, bad);
+      ctl->anc[t][0] = m.lo;
+      ctl->anc[t][1] = m.hi;
+    }
+    if (bad && blockIdx.x == 0) spx_raise(a.status, SPECEXT_ERR_BAD_TREE);
+    warp_arrive(&ctl->anc_ready, lane);
+    if (lane == 0) {
+      for (uint32_t seg = 0; ok && work.next(); ++seg) {
+        ok = wait_c(&ctl->q_empty, seg & 1, abort_flag);
+        if (ok) load_q();
+      }
+    }
+  } else {
+    // ================================ softmax warps ===========================================
+    setmaxnreg_inc<kRegsSoftmax>();
+    const int quarter = warp & 3;
+    RowCtx rc;
+    rc.ctl = ctl;
+    rc.w = warp >> 2;
+    rc.lane = lane;
+    rc.row_t = quarter * 32 + lane;
+    rc.lane_tmem = ctl->tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+    rc.s_free = smem_u32(&ctl->s_free[rc.w]);
+    rc.p_full = smem_u32(&ctl->p_full[rc.w]);
+    rc.scale2 = p.scale2;
+    rc.abort_flag = abort_flag;
+    const int rr = rc.row_t;                             // row inside the row block
+    uint32_t t0 = 0, seg = 0;                            // tiles and segments before the current segment
+    bool anc_seen = false;
+    while (ok && work.next_any()) {
+      const int prob = work.prob, g = prob / p.n_rblk, rblk = prob - g * p.n_rblk, n = work.n;
+      const int r = rblk * p.RB + rr;
+      const bool valid = r < p.rows;
+      const bool warp_valid = r - lane < p.rows;
+      const int slot = worker + prob;
+      float* po = a.ws + p.off_part_o + (long long)slot * (D / 4) * p.RB * 4;
+      // this warpgroup's half of the output columns, in groups of 16
+      constexpr int kGroups = D / 16 / kWG;
+      const int c_lo = rc.w * kGroups;
+      if (DEVLEN && n == 0) {
+        // No tile of this run exists at the device-side length: its slot gets the neutral partial (weight zero in
+        // the merge), and no barrier of the pipeline is touched.
+        if (valid) {
+#pragma unroll 4
+          for (int q4 = c_lo * 4; q4 < (c_lo + kGroups) * 4; ++q4)
+            *reinterpret_cast<float4*>(po + ((long long)q4 * p.RB + rr) * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (rc.w == 0) {
+            a.ws[p.off_part_m + (long long)slot * p.RB + rr] = -1e30f;      // finite: see the merge
+            a.ws[p.off_part_l + (long long)slot * p.RB + rr] = 0.f;
+          }
+        }
+        continue;
+      }
+      const int t_node = valid ? r / p.G : 0;
+      float m_loc = -INFINITY, l = 0.f;                  // l is relative to m_loc
+      for (int j = (rc.w ^ t0) & 1; j < n && ok; j += kWG) {
+        if (!warp_valid) {
+          ok = skip_tile(rc, t0 + j);
+          continue;
+        }
+        const int tile = work.tile(j);
+        const bool is_tree = tile == p.TPH;
+        const int nkeys = is_tree ? p.T : min(SPX_TILE_KEYS, L_eff - tile * SPX_TILE_KEYS);
+        if (is_tree && !anc_seen) {
+          ok = mbar_wait(&ctl->anc_ready, 0, abort_flag);
+          if (!ok) break;
+          anc_seen = true;
+        }
+        float cg[4];                                     // sums of the tile's four groups of 32 keys
+        float* mass = nullptr;
+        long long rowbase = 0;
+        if (SCORE != 0 && !is_tree) {
+          rowbase = ((long long)prob * p.TPH + tile) * p.RB + rr;
+          mass = a.ws + p.off_mass + rowbase * p.CPT;
+        }
+        ok = softmax_tile<D>(
+            rc, t0 + j, j == 0, is_tree || nkeys < SPX_TILE_KEYS,
+            [&](unsigned long long& lo, unsigned long long& hi) {
+              if (is_tree) {               // this node and its ancestors (a padding row sees key 0)
+                lo = valid ? ctl->anc[t_node][0] : 1ull;
+                hi = valid ? ctl->anc[t_node][1] : 0ull;
+              } else {
+                lo = nkeys >= 64 ? ~0ull : ((1ull << nkeys) - 1ull);
+                hi = nkeys <= 64 ? 0ull : ((1ull << (nkeys - 64)) - 1ull);
+              }
+            },
+            [&](int c, const uint32_t (&v)[32], float sum) {
+              if (SCORE == 1 || SCORE == 2) {
+                cg[c] = sum;
+              } else if (SCORE == 3 && mass) {
+                float acc = 0.f;
+#pragma unroll
+                for (int k = 0; k < 32; ++k) {
+                  acc += __uint_as_float(v[k]);
+                  if (((k + 1) & (p.C - 1)) == 0) {
+                    mass[(c * 32 + k) / p.C] = acc;
+                    acc = 0.f;
+                  }
+                }
+              }
+            },
+            m_loc, l);
+        if (SCORE != 0 && ok && mass) {
+          if (SCORE == 1) {
+            *reinterpret_cast<float4*>(mass) = make_float4(cg[0], cg[1], cg[2], cg[3]);
+          } else if (SCORE == 2) {
+            if (p.C == 64)
+              *reinterpret_cast<float2*>(mass) = make_float2(cg[0] + cg[1], cg[2] + cg[3]);
+            else
+              *mass = (cg[0] + cg[1]) + (cg[2] + cg[3]);
+          }
+          a.ws[p.off_mref + rowbase] = m_loc;
+        }
+      }
+      if (!ok) break;
+
+      // ---- end of the segment: unnormalised O, reference maximum and row sum to the partial slot ----
+      float m_fin, l_tot;
+      ok = segment_end(rc, t0 + n - 1, seg, m_loc, l, m_fin, l_tot);
+      if (!ok) break;
+      if (warp_valid) {
+#pragma unroll
+        for (int c = 0; c < kGroups; ++c) {
+          uint32_t v[16];
+          tmem_ld16(rc.lane_tmem + kColO + (c_lo + c) * 16, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4) {
+            const float4 x = make_float4(__uint_as_float(v[q4 * 4]), __uint_as_float(v[q4 * 4 + 1]),
+                                         __uint_as_float(v[q4 * 4 + 2]), __uint_as_float(v[q4 * 4 + 3]));
+            if (valid) *reinterpret_cast<float4*>(po + ((long long)((c_lo + c) * 4 + q4) * p.RB + rr) * 4) = x;
+          }
+        }
+      }
+      if (rc.w == 0 && valid) {                          // rows past the last stacked row are never read
+        a.ws[p.off_part_m + (long long)slot * p.RB + rr] = m_fin;
+        a.ws[p.off_part_l + (long long)slot * p.RB + rr] = l_tot;
+      }
+      tc_fence_before();
+      warp_arrive(&ctl->o_free, lane);
+      t0 += n;
+      ++seg;
+    }
+  }
+
+  if (!ok && lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+  finish<1>(ctl, warp);
+}
+
+template <int D, int SCORE, bool DEVLEN>
+cudaError_t launch(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
+  static SpxOncePerDevice once;
+  constexpr int smem = smem_bytes<1, D>();
+  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN>, smem, &once);
+  if (ec != cudaSuccess) return ec;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.plan.n_cta);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, verify_kernel<D, SCORE, DEVLEN>, a, maps);
+}
+
+template <int D>
+cudaError_t launch_class(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
+  const AttnPlan& p = a.plan;
+  if (a.L_dev) return launch<D, 0, true>(a, maps, st);       // never with chunk sums
+  if (!p.want_score) return launch<D, 0, false>(a, maps, st);
+  return p.C == 32 ? launch<D, 1, false>(a, maps, st)
+         : p.C > 32 ? launch<D, 2, false>(a, maps, st)
+                    : launch<D, 3, false>(a, maps, st);
+}
+
+}  // namespace
+
+// Row blocks of 128 (plan.RB); plan.n_cta counts CTAs.
+cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launches) {
+  const AttnPlan& p = a.plan;
+  VerifyMaps maps;
+  bool ok = spx_encode_map(&maps.kt, a.Kt, p.D, p.Hkv, a.tkv_sh, p.T, a.tkv_st, 1, SPX_TILE_KEYS);
+  ok = ok && spx_encode_map(&maps.vt, a.Vt, p.D, p.Hkv, a.tkv_sh, p.T, a.tkv_st, 1, SPX_TILE_KEYS);
+  if (p.L > 0) {
+    ok = ok && spx_encode_map(&maps.kp, a.Kp, p.D, p.Hkv, a.kv_sh, p.L, a.kv_sl, 1, SPX_TILE_KEYS);
+    ok = ok && spx_encode_map(&maps.vp, a.Vp, p.D, p.Hkv, a.kv_sh, p.L, a.kv_sl, 1, SPX_TILE_KEYS);
+  } else {
+    maps.kp = maps.kt;
+    maps.vp = maps.vt;
+  }
+  ok = ok && spx_encode_map(&maps.q, a.Q, p.D, p.Hq, a.q_sh, p.T, a.q_st, p.G, p.q_rows / p.G);
+  if (!ok) return cudaErrorInvalidValue;
+  const cudaError_t e = p.D == 128 ? launch_class<128>(a, maps, st) : launch_class<64>(a, maps, st);
+  *n_launches += 1;
+  return e;
+}

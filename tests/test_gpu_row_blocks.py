@@ -1,0 +1,24 @@
+"""The one-CTA verification kernel at the edges of its row blocks and segments, against the oracle (tolerances of
+test_gpu_parity: bf16 inputs and probabilities, fp32 sums)."""
+import pytest
+
+from tests.test_gpu_parity import check_attn, make_hp
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,L", [
+    (2, 2, 128, 63, 300),      # 64-row form of Q, one row short
+    (2, 2, 128, 64, 256),      # 64-row form, full
+    (2, 2, 128, 65, 129),      # 128-row form, tree of more than 64 nodes
+    (2, 2, 128, 128, 127),     # 128-row form, full
+    (8, 2, 128, 8, 1),         # 32 rows: one warp works, one key
+    (4, 1, 64, 33, 640),       # head_dim 64: a second row block with 4 rows
+    (4, 1, 64, 128, 131),      # head_dim 64: four row blocks
+    (256, 256, 128, 3, 40),    # more problems than CTAs: several segments per worker, each of one tile or two
+    (160, 160, 64, 5, 515),    # the same with head_dim 64 and segments of an odd and an even number of tiles
+])
+def test_one_cta_row_blocks(cuda_device, Hq, Hkv, D, T, L):
+    w = synth.Workload("rows", Hq, Hkv, D, L, T, 32, 4, "uniform", "needle", seed=Hq + T + L)
+    check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, 32)
