@@ -11,10 +11,9 @@ cudaError_t spx_launch_gather(const void* dK, const void* dV, int n_layers, int 
                               long long s_layer, long long s_l, long long s_h, const int32_t* idx,
                               const int32_t* n_selected, int max_selected, void* K_out, void* V_out,
                               int32_t* n_tokens_out, int32_t* status, cudaStream_t st);
-cudaError_t spx_launch_prefill_tc2(const void* Q, const void* K, const void* V, void* O, float* lse, int L, int Hq,
-                                   int Hkv, float scale2, long long q_st, long long q_sh, long long kv_sl,
-                                   long long kv_sh, long long o_st, long long o_sh, int n_sm, int32_t* status,
-                                   cudaStream_t st);
+cudaError_t spx_launch_prefill(const void* Q, const void* K, const void* V, void* O, float* lse, int L, int Hq, int Hkv,
+                               float scale2, long long q_st, long long q_sh, long long kv_sl, long long kv_sh,
+                               long long o_st, long long o_sh, int n_sm, int32_t* status, cudaStream_t st);
 bool spx_select_gather_fusable(int NC, int k);
 cudaError_t spx_launch_select_gather(const float* score_row, int k, int n_sink, int n_recent, const void* dK,
                                      const void* dV, int n_layers,
@@ -273,11 +272,10 @@ int specext_prefill_attn(const specext_attn_desc* desc, const void* Q, const voi
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(O) || (reinterpret_cast<uintptr_t>(lse) & 3u) != 0)
     return SPECEXT_ERR_INVALID_ARG;
   const float scale = desc->softmax_scale > 0.f ? desc->softmax_scale : 1.0f / std::sqrt((float)desc->head_dim);
-  const cudaError_t e = spx_launch_prefill_tc2(Q, K, V, O, lse, desc->prefix_len, desc->n_q_heads, desc->n_kv_heads,
-                                               scale * 1.44269504088896340736f, desc->q_stride_t, desc->q_stride_h,
-                                               desc->kv_stride_l, desc->kv_stride_h, desc->o_stride_t,
-                                               desc->o_stride_h, sm_count(), device_status,
-                                               static_cast<cudaStream_t>(cuda_stream));
+  const cudaError_t e = spx_launch_prefill(Q, K, V, O, lse, desc->prefix_len, desc->n_q_heads, desc->n_kv_heads,
+                                           scale * 1.44269504088896340736f, desc->q_stride_t, desc->q_stride_h,
+                                           desc->kv_stride_l, desc->kv_stride_h, desc->o_stride_t, desc->o_stride_h,
+                                           sm_count(), device_status, static_cast<cudaStream_t>(cuda_stream));
   g_launches.fetch_add(1);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();

@@ -1,8 +1,9 @@
-"""The one-CTA verification kernel at the edges of its row blocks and segments, against the oracle (tolerances of
-test_gpu_parity: bf16 inputs and probabilities, fp32 sums)."""
+"""The one-CTA verification kernel at the edges of its row blocks and segments, and prefill with many query heads per KV
+head, against the oracle (tolerances of test_gpu_parity: bf16 inputs and probabilities, fp32 sums)."""
 import pytest
 
 from tests.test_gpu_parity import check_attn, make_hp
+from tests.test_gpu_prefill import _compare, _inputs, _run
 from workloads import synth
 
 pytestmark = pytest.mark.gpu
@@ -22,3 +23,12 @@ pytestmark = pytest.mark.gpu
 def test_one_cta_row_blocks(cuda_device, Hq, Hkv, D, T, L):
     w = synth.Workload("rows", Hq, Hkv, D, L, T, 32, 4, "uniform", "needle", seed=Hq + T + L)
     check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, 32)
+
+
+@pytest.mark.parametrize("G", [64, 128, 256])
+def test_prefill_wide_groups(cuda_device, G):
+    """Blocks of 4, 2 and 1 tokens: more problems than clusters, and (G = 256) one token's heads on two CTAs."""
+    L = 131
+    Q, K, V = _inputs(L, G, 1, seed=G)
+    O, lse = _run(cuda_device, Q, K, V)
+    _compare(O, lse, Q, K, V, [0, 1, 2, 3, 4, 63, 64, 126, 127, 128, 129, 130], f"prefill-small-G{G}")
