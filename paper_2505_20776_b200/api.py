@@ -1,14 +1,15 @@
-"""Thin ctypes binding of the C ABI declared in include/specext.h.
+"""Thin binding of the C ABI declared in include/specext.h.
 
 The functions here carry the same names as the C entry points and only marshal arguments
-(device pointers, strides, the current CUDA stream); every step of the path runs in the library's
-kernels.  There is no CPU fallback: if the shared library is missing or a tensor is not on a CUDA
+(device pointers, strides, the current CUDA stream; the calls of a decoding step through the extension
+module built from csrc/binding.cpp, the others through ctypes); every step of the path runs in the
+library's kernels.  There is no CPU fallback: if the shared library is missing or a tensor is not on a CUDA
 device the call raises.
 """
 from __future__ import annotations
 
 import ctypes
-import math
+import importlib.util
 import os
 from typing import Optional, Tuple
 
@@ -40,6 +41,8 @@ class AttnDesc(ctypes.Structure):
 
 
 _LIB: Optional[ctypes.CDLL] = None
+_BINDING = None
+_ENTRIES = ("verify_attn", "draft_attn", "prefill_attn", "select_gather")     # called through the extension module
 
 
 def bind(path: str) -> ctypes.CDLL:
@@ -70,7 +73,22 @@ def bind(path: str) -> ctypes.CDLL:
     L.specext_status_string.argtypes = [ctypes.c_int]
     L.specext_launch_count.restype = i64
     L.specext_launch_count.argtypes = []
+    L.entry = {n: ctypes.cast(getattr(L, "specext_" + n), vp).value for n in _ENTRIES}
     return L
+
+
+def _binding():
+    """The extension module (built in-tree by build.py); raises if it is not there."""
+    global _BINDING
+    if _BINDING is None:
+        path = _build.BINDING_PATH
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: run `python -m paper_2505_20776_b200.build`")
+        spec = importlib.util.spec_from_file_location(__package__ + "._binding", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _BINDING = module
+    return _BINDING
 
 
 def lib() -> ctypes.CDLL:
@@ -95,7 +113,7 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return _binding().current_stream()
 
 
 def _check(code: int, where: str) -> None:
@@ -103,27 +121,12 @@ def _check(code: int, where: str) -> None:
         raise SpecextError(code, where)
 
 
-def _bf16_3d(t: torch.Tensor, name: str) -> None:
-    if t.dtype != torch.bfloat16 or t.dim() != 3 or t.stride(2) != 1:
-        raise ValueError(f"{name} must be a bf16 [.][heads][head_dim] tensor with contiguous head_dim")
-
-
 def make_attn_desc(Q: torch.Tensor, K_prefix: torch.Tensor, K_tree: torch.Tensor, O: torch.Tensor,
                    prefix_len: int, chunk_size: int, softmax_scale: float = 0.0,
                    want_chunk_score: bool = False) -> AttnDesc:
     """Fills a specext_attn_desc from tensor shapes and strides (V tensors share K's strides)."""
-    for t, n in ((Q, "Q"), (K_prefix, "K_prefix"), (K_tree, "K_tree"), (O, "O")):
-        _bf16_3d(t, n)
-    T, Hq, D = Q.shape
     d = AttnDesc()
-    d.n_q_heads, d.n_kv_heads, d.head_dim = Hq, K_tree.shape[1], D
-    d.prefix_len, d.n_tree, d.chunk_size = int(prefix_len), T, int(chunk_size)
-    d.softmax_scale = float(softmax_scale)
-    d.want_chunk_score = 1 if want_chunk_score else 0
-    d.q_stride_t, d.q_stride_h = Q.stride(0), Q.stride(1)
-    d.kv_stride_l, d.kv_stride_h = K_prefix.stride(0), K_prefix.stride(1)
-    d.tkv_stride_t, d.tkv_stride_h = K_tree.stride(0), K_tree.stride(1)
-    d.o_stride_t, d.o_stride_h = O.stride(0), O.stride(1)
+    _binding().fill_desc(d, Q, K_prefix, K_tree, O, int(prefix_len), int(chunk_size), softmax_scale, want_chunk_score)
     return d
 
 
@@ -136,17 +139,10 @@ def specext_verify_attn(desc: AttnDesc, Q: torch.Tensor, K_prefix: torch.Tensor,
                         lse: torch.Tensor, chunk_score: Optional[torch.Tensor], workspace: torch.Tensor,
                         device_status: torch.Tensor) -> None:
     """Enqueues one verification attention call on the current stream (see include/specext.h)."""
-    if V_prefix.stride() != K_prefix.stride() or V_tree.stride() != K_tree.stride():
-        raise ValueError("V tensors must have the strides of the matching K tensors")
-    if parent.dtype != torch.int32 or lse.dtype != torch.float32 or device_status.dtype != torch.int32:
-        raise ValueError("parent/device_status must be int32 and lse fp32")
-    if chunk_score is not None and chunk_score.dtype != torch.float32:
-        raise ValueError("chunk_score must be fp32")
-    rc = lib().specext_verify_attn(ctypes.byref(desc), _ptr(Q), _ptr(K_prefix), _ptr(V_prefix), _ptr(K_tree),
-                                   _ptr(V_tree), _ptr(parent), _ptr(O), _ptr(lse), _ptr(chunk_score),
-                                   _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                   _ptr(device_status), _stream())
-    _check(rc, "specext_verify_attn")
+    rc = (_BINDING or _binding()).verify_attn((_LIB or lib()).entry["verify_attn"], desc, Q, K_prefix, V_prefix, K_tree,
+                                              V_tree, parent, O, lse, chunk_score, workspace, device_status)
+    if rc:
+        raise SpecextError(rc, "specext_verify_attn")
 
 
 def specext_draft_attn(desc: AttnDesc, Q: torch.Tensor, K_cache: torch.Tensor, V_cache: torch.Tensor,
@@ -154,38 +150,18 @@ def specext_draft_attn(desc: AttnDesc, Q: torch.Tensor, K_cache: torch.Tensor, V
                        O: torch.Tensor, lse: torch.Tensor, workspace: torch.Tensor,
                        device_status: torch.Tensor) -> None:
     """Enqueues the draft model's attention over a compact cache whose length is an int32 on the device."""
-    if V_cache.stride() != K_cache.stride() or V_tree.stride() != K_tree.stride():
-        raise ValueError("V tensors must have the strides of the matching K tensors")
-    if (parent.dtype != torch.int32 or lse.dtype != torch.float32 or device_status.dtype != torch.int32 or
-            n_tokens.dtype != torch.int32):
-        raise ValueError("parent/device_status/n_tokens must be int32 and lse fp32")
-    rc = lib().specext_draft_attn(ctypes.byref(desc), _ptr(Q), _ptr(K_cache), _ptr(V_cache), _ptr(n_tokens),
-                                  _ptr(K_tree), _ptr(V_tree), _ptr(parent), _ptr(O), _ptr(lse), _ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _ptr(device_status), _stream())
-    _check(rc, "specext_draft_attn")
+    rc = (_BINDING or _binding()).draft_attn((_LIB or lib()).entry["draft_attn"], desc, Q, K_cache, V_cache, n_tokens,
+                                             K_tree, V_tree, parent, O, lse, workspace, device_status)
+    if rc:
+        raise SpecextError(rc, "specext_draft_attn")
 
 
 def specext_prefill_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, O: torch.Tensor, lse: torch.Tensor,
                          device_status: torch.Tensor, softmax_scale: float = 0.0) -> None:
     """Enqueues the prefill (causal self-attention) of a prompt: Q, O [L][Hq][128], K, V [L][Hkv][128], lse [Hq][L]."""
-    for t, n in ((Q, "Q"), (K, "K"), (V, "V"), (O, "O")):
-        _bf16_3d(t, n)
-    if K.stride() != V.stride() or lse.dtype != torch.float32 or device_status.dtype != torch.int32:
-        raise ValueError("K and V must share strides; lse must be fp32 and device_status int32")
-    L, Hq, D = Q.shape
-    if K.shape[0] < L or O.shape != Q.shape or lse.numel() < Hq * L or not lse.is_contiguous():
-        raise ValueError("shapes: K, V [>=L][Hkv][D], O like Q, lse contiguous [Hq][L]")
-    d = AttnDesc()
-    d.n_q_heads, d.n_kv_heads, d.head_dim = Hq, K.shape[1], D
-    d.prefix_len, d.n_tree, d.chunk_size = L, 1, 32
-    d.softmax_scale, d.want_chunk_score = float(softmax_scale), 0
-    d.q_stride_t, d.q_stride_h = Q.stride(0), Q.stride(1)
-    d.kv_stride_l, d.kv_stride_h = K.stride(0), K.stride(1)
-    d.tkv_stride_t, d.tkv_stride_h = K.stride(0), K.stride(1)
-    d.o_stride_t, d.o_stride_h = O.stride(0), O.stride(1)
-    rc = lib().specext_prefill_attn(ctypes.byref(d), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(lse),
-                                    _ptr(device_status), _stream())
-    _check(rc, "specext_prefill_attn")
+    rc = _binding().prefill_attn(lib().entry["prefill_attn"], Q, K, V, O, lse, device_status, softmax_scale)
+    if rc:
+        raise SpecextError(rc, "specext_prefill_attn")
 
 
 STATIC_SCRATCH_BYTES = 32 << 20
@@ -253,29 +229,23 @@ def specext_select_gather(chunk_score: torch.Tensor, row: int, prefix_len: int, 
                           n_tokens_out: torch.Tensor, device_status: torch.Tensor, n_sink_chunks: int = 0,
                           n_recent_chunks: int = 0) -> None:
     """Enqueues SelectChunks + UpdateDraftCache as one call (one kernel launch for the usual sizes)."""
-    if chunk_score.dtype != torch.float32 or chunk_score.dim() != 2 or not chunk_score.is_contiguous():
+    if chunk_score.dim() != 2:
         raise ValueError("chunk_score must be a contiguous fp32 [n_tree][n_chunks] tensor")
-    if idx.dtype != torch.int32 or n_selected.dtype != torch.int32:
-        raise ValueError("idx and n_selected must be int32")
-    for t in (draft_K, draft_V):
-        if t.dtype != torch.bfloat16 or t.dim() != 4 or t.stride(3) != 1:
-            raise ValueError("draft K/V must be bf16 [layers][tokens][heads][dim]")
-    if draft_K.stride() != draft_V.stride():
-        raise ValueError("draft K and V must share strides")
     n_tree, n_chunks = chunk_score.shape
-    nl, _, H, D = draft_K.shape
-    need = nl * k * chunk_size * H * D
-    if idx.numel() < min(k, n_chunks):
-        raise ValueError("idx is too small")
-    if not (K_out.is_contiguous() and V_out.is_contiguous()) or K_out.numel() < need or V_out.numel() < need:
-        raise ValueError("K_out/V_out must be contiguous and hold [layers][k*C][H][D]")
-    rc = lib().specext_select_gather(_ptr(chunk_score), n_tree, n_chunks, int(row), int(prefix_len),
-                                     int(chunk_size), int(k), int(n_sink_chunks), int(n_recent_chunks),
-                                     _ptr(draft_K), _ptr(draft_V), nl, H, D,
-                                     draft_K.stride(0), draft_K.stride(1), draft_K.stride(2), _ptr(idx),
-                                     _ptr(n_selected), _ptr(K_out), _ptr(V_out), _ptr(n_tokens_out),
-                                     _ptr(device_status), _stream())
-    _check(rc, "specext_select_gather")
+    select_gather_flat(chunk_score, n_tree, n_chunks, row, prefix_len, chunk_size, k, draft_K, draft_V, idx, n_selected,
+                       K_out, V_out, n_tokens_out, device_status, n_sink_chunks, n_recent_chunks)
+
+
+def select_gather_flat(chunk_score: torch.Tensor, n_tree: int, n_chunks: int, row: int, prefix_len: int, chunk_size: int,
+                       k: int, draft_K: torch.Tensor, draft_V: torch.Tensor, idx: torch.Tensor,
+                       n_selected: torch.Tensor, K_out: torch.Tensor, V_out: torch.Tensor, n_tokens_out: torch.Tensor,
+                       device_status: torch.Tensor, n_sink_chunks: int = 0, n_recent_chunks: int = 0) -> None:
+    """specext_select_gather with the scores as the first n_tree x n_chunks values of a contiguous buffer."""
+    rc = _binding().select_gather(lib().entry["select_gather"], chunk_score, n_tree, n_chunks, int(row), int(prefix_len),
+                                  int(chunk_size), int(k), int(n_sink_chunks), int(n_recent_chunks), draft_K, draft_V,
+                                  idx, n_selected, K_out, V_out, n_tokens_out, device_status)
+    if rc:
+        raise SpecextError(rc, "specext_select_gather")
 
 
 def specext_read_status(device_status: torch.Tensor) -> int:

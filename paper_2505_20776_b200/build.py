@@ -2,17 +2,20 @@
 
 libspecext.so is the product.  libspecext_testing.so is the same code compiled with -DSPECEXT_TESTING
 plus the CUDA-core cross-check kernel and a few test hooks (csrc/testing.h); only the tests load it.
+_binding.so is the Python extension module that marshals the calls of a decoding step (csrc/binding.cpp).
 """
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB_PATH = os.path.join(HERE, "libspecext.so")
+BINDING_PATH = os.path.join(HERE, "_binding.so")
 TESTING_LIB_PATH = os.path.join(HERE, "libspecext_testing.so")
 SOURCES = ["api.cu", "attn_tc2.cu", "verify.cu", "prefill.cu", "merge.cu", "retrieval.cu"]
 TESTING_SOURCES = SOURCES + ["attn_simt.cu", "testing.cu"]
@@ -23,17 +26,29 @@ def nvcc_path() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
-def _stale(lib: str) -> bool:
+def _stale(lib: str, deps) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
-    deps.append(os.path.join(os.path.dirname(HERE), "include", "specext.h"))
+    deps = list(deps) + [os.path.join(os.path.dirname(HERE), "include", "specext.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _cuda_deps():
+    return [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")]
+
+
 def needs_build() -> bool:
-    return _stale(LIB_PATH)
+    return _stale(LIB_PATH, _cuda_deps())
+
+
+def _run(cmd, lib: str, verbose: bool) -> str:
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError(f"{os.path.basename(cmd[0])} failed building {os.path.basename(lib)}")
+    return lib
 
 
 def _compile(lib: str, sources, defines, verbose: bool) -> str:
@@ -42,16 +57,28 @@ def _compile(lib: str, sources, defines, verbose: bool) -> str:
     if verbose:
         cmd += ["-Xptxas", "-v"]
     cmd += [os.path.join(CSRC, s) for s in sources]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-    if res.returncode != 0:
-        raise RuntimeError(f"nvcc failed building {os.path.basename(lib)}")
-    return lib
+    return _run(cmd, lib, verbose)
+
+
+def build_binding(force: bool = False, verbose: bool = False) -> str:
+    """Builds the extension module against the installed torch and returns its path."""
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and not _stale(BINDING_PATH, [src]):
+        return BINDING_PATH
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(nvcc_path())) if os.path.isabs(nvcc_path()) else "/usr/local/cuda"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-o", BINDING_PATH, src,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(root, "include"),
+           "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"), "-I" + os.path.join(cuda, "include"),
+           "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    return _run(cmd, BINDING_PATH, verbose)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Builds libspecext.so next to this file and returns its path."""
+    """Builds libspecext.so (and the extension module) next to this file and returns its path."""
+    build_binding(force, verbose)
     if not force and not needs_build():
         return LIB_PATH
     return _compile(LIB_PATH, SOURCES, [], verbose)
@@ -59,7 +86,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def build_testing(force: bool = False, verbose: bool = False) -> str:
     """Builds the test library (cross-check kernel and test hooks) and returns its path."""
-    if not force and not _stale(TESTING_LIB_PATH):
+    if not force and not _stale(TESTING_LIB_PATH, _cuda_deps()):
         return TESTING_LIB_PATH
     return _compile(TESTING_LIB_PATH, TESTING_SOURCES, ["-DSPECEXT_TESTING"], verbose)
 

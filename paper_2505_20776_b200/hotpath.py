@@ -37,7 +37,6 @@ class HotPath:
         self.K_compact = self._alloc(shape, torch.bfloat16).zero_()
         self.V_compact = self._alloc(shape, torch.bfloat16).zero_()
         self._ws = self._alloc((0,), torch.uint8)
-        self._desc_cache: Dict[tuple, api.AttnDesc] = {}
 
     # -- helpers -------------------------------------------------------------------------------
     def _alloc(self, shape, dtype) -> torch.Tensor:
@@ -53,17 +52,13 @@ class HotPath:
         return self._score_flat[: self.T * nc].view(self.T, nc)
 
     def _desc(self, t: Dict[str, torch.Tensor], prefix_len: int, want_score: bool) -> api.AttnDesc:
-        key = (prefix_len, want_score, t["Q"].stride(), t["K_prefix"].stride(), t["K_tree"].stride())
-        d = self._desc_cache.get(key)
-        if d is None:
-            d = api.make_attn_desc(t["Q"], t["K_prefix"], t["K_tree"], self.O, prefix_len, self.C, self.scale,
-                                   want_score)
-            need = api.specext_verify_attn_workspace(d)
-            if need == 0:
-                raise api.SpecextError(2, "specext_verify_attn_workspace")
-            if self._ws.numel() < need:
-                self._ws = self._alloc((need,), torch.uint8)
-            self._desc_cache[key] = d
+        # made anew for every call (half a microsecond): the prefix grows with every step
+        d = api.make_attn_desc(t["Q"], t["K_prefix"], t["K_tree"], self.O, prefix_len, self.C, self.scale, want_score)
+        need = api.specext_verify_attn_workspace(d)
+        if need == 0:
+            raise api.SpecextError(2, "specext_verify_attn_workspace")
+        if self._ws.numel() < need:
+            self._ws = self._alloc((need,), torch.uint8)
         return d
 
     # -- the three steps -----------------------------------------------------------------------
@@ -72,7 +67,7 @@ class HotPath:
         if prefix_len > self.max_prefix:
             raise ValueError("prefix_len exceeds max_prefix")
         d = self._desc(t, prefix_len, want_score)
-        cs = self.chunk_score(prefix_len) if want_score else None
+        cs = self._score_flat if want_score else None
         api.specext_verify_attn(d, t["Q"], t["K_prefix"], t["V_prefix"], t["K_tree"], t["V_tree"], parent,
                                 self.O, self.lse, cs, self._ws, self.status)
 
@@ -87,9 +82,9 @@ class HotPath:
     def select_gather(self, row: int, prefix_len: int, draft_K: torch.Tensor, draft_V: torch.Tensor,
                       n_sink_chunks: int = 0, n_recent_chunks: int = 0) -> None:
         """SelectChunks + UpdateDraftCache as one library call."""
-        api.specext_select_gather(self.chunk_score(prefix_len), row, prefix_len, self.C, self.k, draft_K, draft_V,
-                                  self.idx, self.n_selected, self.K_compact, self.V_compact, self.n_tokens,
-                                  self.status, n_sink_chunks, n_recent_chunks)
+        api.select_gather_flat(self._score_flat, self.T, self.n_chunks(prefix_len), row, prefix_len, self.C, self.k,
+                               draft_K, draft_V, self.idx, self.n_selected, self.K_compact, self.V_compact,
+                               self.n_tokens, self.status, n_sink_chunks, n_recent_chunks)
 
     def read_status(self) -> int:
         return api.specext_read_status(self.status)
