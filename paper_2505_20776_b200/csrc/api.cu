@@ -19,7 +19,7 @@ cudaError_t spx_launch_select_gather(const float* score_row, int k, int n_sink, 
                                      const void* dV, int n_layers,
                                      int H, int D, int L, int C, long long s_layer, long long s_l, long long s_h,
                                      int32_t* idx, int32_t* n_selected, void* K_out, void* V_out,
-                                     int32_t* n_tokens_out, int32_t* status, cudaStream_t st);
+                                     int32_t* n_tokens_out, int n_sm, int32_t* status, cudaStream_t st);
 
 // Scratch of the entry point that takes no workspace.  Part of the library image: resident on every
 // device that loads the library until the process exits.  Device code may name it directly; host
@@ -392,7 +392,7 @@ int specext_select_gather(const float* chunk_score, int32_t n_tree, int32_t n_ch
                                                  n_recent_chunks, draft_K, draft_V,
                                                  n_layers, n_kv_heads, head_dim, prefix_len, chunk_size,
                                                  stride_layer, stride_l, stride_h, idx, n_selected, K_out, V_out,
-                                                 n_tokens_out, device_status, st);
+                                                 n_tokens_out, sm_count(), device_status, st);
   g_launches.fetch_add(1);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();

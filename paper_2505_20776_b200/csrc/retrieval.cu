@@ -1,22 +1,24 @@
 // SelectChunks and UpdateDraftCache kernels.
 //
-// select_kernel (one CTA): the ranking key of chunk c is score[c] / len_c, a non-negative fp32
-// whose bit pattern orders like the value.  A most-significant-digit radix select (4 passes of
-// 8 bits, warp-aggregated shared-memory histograms) finds the k-th largest key exactly; every
-// chunk with a larger key is kept, and of the chunks equal to it the lowest-indexed are kept
-// until k are chosen.  A block-wide ballot/popcount scan in index order then emits the kept
-// chunks in ascending order, which also implements the tie rule.
+// The ranking key of chunk c is score[c] / len_c, a non-negative fp32 whose bit pattern orders like the value.  A block
+// reads every key once, into registers (thread t holds the keys of consecutive chunks), finds the k-th largest by a
+// most-significant-digit radix select (at most 4 passes of 8 bits over shared-memory histograms) and emits the kept
+// chunks in ascending order after one block-wide scan: a chunk with a larger key is kept, and of the chunks equal to the
+// k-th the lowest-indexed are kept until k are chosen.
 //
-// gather_kernel: 16-byte vector copy of the kept chunks of the draft K and V into the compact cache.
+// What bounds it: latency.  One block barrier per radix pass (every warp scans the histogram for itself) and two for the
+// emission; the copy that follows has all its loads in flight at once.  select_gather_kernel, us per call replayed alone
+// (draft cache in L2), against the form with two barriers per pass, one emission round per 256 chunks and the selection
+// repeated by 256 to 512 blocks: 128 chunks 5.5 -> 5.6, 512 chunks 6.5 -> 5.1, 4096 chunks 29.7 -> 10.2, two layers of
+// 12 x 64 heads and 257 chunks 7.9 -> 6.2.
 #include "common.cuh"
 #include "sm100.cuh"
 
 namespace {
 
-constexpr int kSelThreads = 1024;
-constexpr int kFusedThreads = 256;
+constexpr int kSelThreads = 512;
 constexpr int kFusedMaxK = 1024;           // selected indices a fused block keeps in shared memory
-constexpr int kFusedMaxChunks = 8192;      // above this every block repeating the selection costs more than a launch
+constexpr int kFusedMaxChunks = 8192;      // 16 keys a thread; above this the repeated selection costs more than a launch
 
 // Shape of one selection: chunk count, prefix length, chunk size, and the forced chunks (the first n_sink
 // and the last n_recent chunks are kept whatever their score; 0 and 0 = the plain top-k).
@@ -33,122 +35,105 @@ __device__ __forceinline__ uint32_t chunk_key(const float* __restrict__ score, i
   return __float_as_uint(x);
 }
 
-constexpr int kKeyCache = 2048;            // ranking keys kept in shared memory (more chunks: recomputed per pass)
-
 template <int NT>
 struct SelectSmem {
-  uint32_t hist[4][256];                   // one histogram per radix pass: cleared once, no barrier in between
-  uint32_t s_prefix[4], s_need[4];
-  uint32_t warp_eq[2][NT / 32], warp_keep[2][NT / 32];     // per batch of NT chunks, double-buffered
-  uint32_t keys[kKeyCache];
+  uint32_t hist[4][256];                   // one histogram per radix pass: cleared once
+  uint32_t warp_tot[NT / 32];
 };
 
-// Selection by one block of NT threads: writes the keff = min(k, NC) kept chunk indices, ascending,
-// to idx_out (global or shared memory).  Every thread of the block must call it.  Two block barriers per
-// radix pass and two per batch of NT chunks in the emission.
-template <int NT>
+// Selection by one block of NT threads over NC <= NT * IPT chunks: writes the keff = min(k, NC) kept chunk indices,
+// ascending, to idx_out (global or shared memory).  Every thread of the block must call it.
+template <int NT, int IPT>
 __device__ __forceinline__ void select_block(SelectSmem<NT>& sm, const float* __restrict__ score, const SelShape& sh,
                                              int keff, int32_t* idx_out) {
-  const int NC = sh.NC;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = NT / 32;
-  // one load and one division per chunk when the keys fit in shared memory
-  const bool cached = NC <= kKeyCache;
-  if (cached)
-    for (int c = tid; c < NC; c += NT) sm.keys[c] = chunk_key(score, c, sh);
-  auto key_of = [&](int c) -> uint32_t { return cached ? sm.keys[c] : chunk_key(score, c, sh); };
+  const int c0 = tid * IPT;
+  uint32_t key[IPT];
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) key[i] = c0 + i < sh.NC ? chunk_key(score, c0 + i, sh) : 0u;
   for (int i = tid; i < 4 * 256; i += NT) (&sm.hist[0][0])[i] = 0;
   __syncthreads();
 
   // ---- radix select of the keff-th largest key --------------------------------------------
-  uint32_t prefix = 0, need = keff;        // `need` keys still to take among those matching prefix
+  uint32_t prefix = 0, mask = 0, need = keff;        // `need` keys still to take among those matching prefix
+  bool all = false;                                  // every key that matches prefix is kept
 #pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {
+  for (int pass = 0; pass < 4 && !all; ++pass) {
     const int shift = 24 - 8 * pass;
-    const uint32_t himask = pass == 0 ? 0u : (0xFFFFFFFFu << (shift + 8));
-    for (int c = tid; c < NC; c += NT) {
-      const uint32_t key = key_of(c);
-      if ((key & himask) == prefix) atomicAdd(&sm.hist[pass][(key >> shift) & 255u], 1u);
-    }
+#pragma unroll
+    for (int i = 0; i < IPT; ++i)
+      if (c0 + i < sh.NC && (key[i] & mask) == prefix) atomicAdd(&sm.hist[pass][(key[i] >> shift) & 255u], 1u);
     __syncthreads();
-    if (warp == 0) {
-      // bins from high to low: lane owns bins 255-8*lane .. 248-8*lane
-      uint32_t local[8], tot = 0;
+    // bins from high to low: lane owns bins 255-8*lane .. 248-8*lane
+    const uint4 h0 = *reinterpret_cast<const uint4*>(&sm.hist[pass][248 - 8 * lane]);
+    const uint4 h1 = *reinterpret_cast<const uint4*>(&sm.hist[pass][252 - 8 * lane]);
+    const uint32_t local[8] = {h1.w, h1.z, h1.y, h1.x, h0.w, h0.z, h0.y, h0.x};
+    const uint32_t tot = ((local[0] + local[1]) + (local[2] + local[3])) + ((local[4] + local[5]) + (local[6] + local[7]));
+    uint32_t incl = tot;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        local[i] = sm.hist[pass][255 - (lane * 8 + i)];
-        tot += local[i];
-      }
-      uint32_t incl = tot;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      uint32_t before = incl - tot;       // keys in strictly higher bins than this lane's
-      if (before < need && need <= incl) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (before < need && need <= before + local[i]) {
-            sm.s_prefix[pass] = prefix | ((uint32_t)(255 - (lane * 8 + i)) << shift);
-            sm.s_need[pass] = need - before;
-          }
-          before += local[i];
-        }
-      }
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
     }
-    __syncthreads();
-    prefix = sm.s_prefix[pass];
-    need = sm.s_need[pass];
+    // the lane whose bins hold the need-th key (one of them always does: need <= the number of matching keys)
+    const int src = __ffs(__ballot_sync(0xffffffffu, need <= incl)) - 1;
+    uint32_t before = incl - tot, bin = 0, left = 0, cnt = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (before < need && need <= before + local[i]) {
+        bin = 255 - (lane * 8 + i);
+        left = need - before;
+        cnt = local[i];
+      }
+      before += local[i];
+    }
+    bin = __shfl_sync(0xffffffffu, bin, src);
+    left = __shfl_sync(0xffffffffu, left, src);
+    cnt = __shfl_sync(0xffffffffu, cnt, src);
+    prefix |= bin << shift;
+    mask |= 255u << shift;
+    need = left;
+    all = left == cnt;
   }
-  const uint32_t theta = prefix;           // the keff-th largest key
-  const uint32_t need_eq = need;           // how many keys equal to theta are kept (lowest indices)
+  // now: a key above prefix (in the digits looked at) is kept, and `need` of those that match it
 
   // ---- emit in ascending index order --------------------------------------------------------
-  uint32_t carry_eq = 0, carry_keep = 0;   // totals of the batches before this one (the same in every thread)
-  int buf = 0;
-  for (int base = 0; base < NC; base += NT, buf ^= 1) {
-    const int c = base + tid;
-    uint32_t key = 0;
-    const bool in = c < NC;
-    if (in) key = key_of(c);
-    const bool eq = in && key == theta;
-    const bool gt = in && key > theta;
-    const uint32_t beq = __ballot_sync(0xffffffffu, eq);
-    if (lane == 0) sm.warp_eq[buf][warp] = __popc(beq);
-    __syncthreads();
-    uint32_t eq_before = carry_eq + __popc(beq & ((1u << lane) - 1u)), eq_all = 0;
+  uint32_t mine = 0;                                 // keys above | keys that match << 16
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      const uint32_t x = sm.warp_eq[buf][w];
-      eq_all += x;
-      if (w < warp) eq_before += x;
-    }
-    const bool keep = gt || (eq && eq_before < need_eq);
-    const uint32_t bk = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) sm.warp_keep[buf][warp] = __popc(bk);
-    __syncthreads();
-    uint32_t pos = carry_keep + __popc(bk & ((1u << lane) - 1u)), keep_all = 0;
+  for (int i = 0; i < IPT; ++i)
+    if (c0 + i < sh.NC) mine += (key[i] & mask) > prefix ? 1u : ((key[i] & mask) == prefix ? 0x10000u : 0u);
+  uint32_t incl = mine;
 #pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      const uint32_t x = sm.warp_keep[buf][w];
-      keep_all += x;
-      if (w < warp) pos += x;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) sm.warp_tot[warp] = incl;
+  __syncthreads();
+  uint32_t before = incl - mine;                     // (a count before a thread is below 65536: the two halves stay apart)
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w)
+    if (w < warp) before += sm.warp_tot[w];
+  uint32_t gt = before & 0xffffu, eq = before >> 16;
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    if (c0 + i < sh.NC) {
+      const uint32_t kv = key[i] & mask;
+      if (kv > prefix || (kv == prefix && eq < need)) idx_out[gt + min(eq, need)] = c0 + i;
+      gt += kv > prefix;
+      eq += kv == prefix;
     }
-    if (keep && pos < (uint32_t)keff) idx_out[pos] = c;
-    carry_eq += eq_all;
-    carry_keep += keep_all;
   }
 }
 
-template <int NT>
+template <int NT, int IPT>
 __global__ void __launch_bounds__(NT) select_kernel(const float* __restrict__ score, const SelShape sh, int k,
                                                     int32_t* __restrict__ idx, int32_t* __restrict__ n_selected) {
-  __shared__ SelectSmem<NT> sm;
+  __shared__ __align__(16) SelectSmem<NT> sm;
   sm100::pdl_launch_dependents();
   sm100::pdl_wait();                       // the scores are complete
   const int keff = min(k, sh.NC);
-  select_block<NT>(sm, score, sh, keff, idx);
+  select_block<NT, IPT>(sm, score, sh, keff, idx);
   if (threadIdx.x == 0) *n_selected = keff;
 }
 
@@ -241,32 +226,83 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
   gather_part(g, i, c, part, layer, which);
 }
 
-// SelectChunks and UpdateDraftCache in one launch: every block repeats the (deterministic) selection
-// in its own shared memory and then copies its share of the kept chunks, so no block waits for
-// another; block (0, 0, 0) also writes idx, n_selected and n_tokens.
-__global__ void __launch_bounds__(kFusedThreads) select_gather_kernel(const __grid_constant__ GatherArgs g) {
-  __shared__ SelectSmem<kFusedThreads> sm;
+// Copies the kept chunks in segments of 64 16-byte vectors, dealt to the warps of the grid; a warp has four segments (eight
+// loads a lane) in flight.  Where a segment lies is worked out once for the warp: per vector, the integer divisions took
+// longer than the copy.
+__device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32_t* s_idx, int keff) {
+  const int vpr = g.D / 8, vpt = g.H * vpr, vpc = g.C * vpt;       // vectors per head row, token, chunk
+  const uint32_t spc = (uint32_t)(vpc + 63) / 64;                  // segments per chunk
+  const uint32_t n_seg = 2u * g.n_layers * keff * spc;
+  const bool contiguous = g.s_h == g.D && g.s_l == (long long)g.H * g.D;
+  const int lane = threadIdx.x & 31;
+  const uint32_t n_warps = gridDim.x * (blockDim.x / 32);
+  // warps of different blocks next to each other in the line, so that a short line keeps every SM busy
+  const uint32_t first = (threadIdx.x / 32) * gridDim.x + blockIdx.x;
+  for (uint32_t s0 = first; s0 < n_seg; s0 += 4 * n_warps) {
+    uint4 x[4][2];
+    uint4* dst[4];
+    int lim[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t s = s0 + q * n_warps;
+      lim[q] = 0;
+      if (s < n_seg) {
+        const uint32_t chunk = s / spc, w0 = (s - chunk * spc) * 64;
+        const uint32_t part = chunk / (uint32_t)keff, i = chunk - part * keff;
+        const uint32_t which = part / (uint32_t)g.n_layers, layer = part - which * g.n_layers;
+        const int c = s_idx[i];
+        if (c >= 0 && c < g.NC) lim[q] = min(g.C, g.L - c * g.C) * vpt - (int)w0;     // vectors of the chunk from here on
+        const __nv_bfloat16* base = g.src[which] + (long long)layer * g.s_layer + (long long)c * g.C * g.s_l;
+        dst[q] = reinterpret_cast<uint4*>(g.dst[which]) + ((long long)layer * g.max_selected + i) * vpc + w0 + lane;
+        if (contiguous) {
+          const uint4* src = reinterpret_cast<const uint4*>(base) + w0 + lane;
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            if (lane + 32 * e < lim[q]) x[q][e] = __ldg(src + 32 * e);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int w = (int)w0 + lane + 32 * e, o = w / vpt, r = w - o * vpt, h = r / vpr;
+            if (lane + 32 * e < lim[q])
+              x[q][e] = __ldg(reinterpret_cast<const uint4*>(base + (long long)o * g.s_l + (long long)h * g.s_h + (r - h * vpr) * 8));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        if (lane + 32 * e < lim[q]) dst[q][32 * e] = x[q][e];
+  }
+}
+
+// SelectChunks and UpdateDraftCache in one launch: every block repeats the (deterministic) selection in its own shared
+// memory and then copies its share of the kept chunks, so no block waits for another; block 0 also writes idx,
+// n_selected and n_tokens.  At most two blocks per SM: with one the call alone is 1.0 us shorter (the
+// selections of two blocks share an SM's pipes), but behind a verification call, with the draft cache in DRAM, 0.4 to 1.1 us
+// longer (4K: 23.9 against 23.3 us for call and retrieval; 8K, two-layer draft: 42.2 against 41.1).
+template <int IPT>
+__global__ void __launch_bounds__(kSelThreads) select_gather_kernel(const __grid_constant__ GatherArgs g) {
+  __shared__ __align__(16) SelectSmem<kSelThreads> sm;
   __shared__ int32_t s_idx[kFusedMaxK];
-  const int i = blockIdx.x / g.sub;
-  const int part = blockIdx.x - i * g.sub;
-  const int layer = blockIdx.y;
-  const int which = blockIdx.z;
   sm100::pdl_launch_dependents();
-  sm100::pdl_wait();                                 // the scores are complete
   const int keff = min(g.k, g.NC);
-  if (i >= keff) return;                             // uniform for the block
+  // (an index stays -1 only when the scores change while they are ranked; the copy skips it)
+  for (int j = threadIdx.x; j < keff; j += kSelThreads) s_idx[j] = -1;
   const SelShape sh = {g.NC, g.L, g.C, g.n_sink, g.n_recent};
-  select_block<kFusedThreads>(sm, g.score, sh, keff, s_idx);
+  sm100::pdl_wait();                                 // the scores are complete
+  select_block<kSelThreads, IPT>(sm, g.score, sh, keff, s_idx);
   __syncthreads();
-  if (blockIdx.x == 0 && layer == 0 && which == 0) {
-    for (int j = threadIdx.x; j < keff; j += kFusedThreads) g.idx_out[j] = s_idx[j];
+  gather_segments(g, s_idx, keff);
+  if (blockIdx.x == 0) {
+    for (int j = threadIdx.x; j < keff; j += kSelThreads) g.idx_out[j] = s_idx[j];
     if (threadIdx.x == 0) {
       *g.n_selected_out = keff;
       const int last = s_idx[keff - 1];
       *g.n_tokens_out = (keff - 1) * g.C + min(g.C, g.L - last * g.C);
     }
   }
-  gather_part(g, i, s_idx[i], part, layer, which);
 }
 
 cudaError_t launch_pdl(const void* kernel, dim3 grid, dim3 block, void** args, cudaStream_t st) {
@@ -311,10 +347,11 @@ cudaError_t spx_launch_select(const float* score_row, int NC, int L, int C, int 
                               int32_t* idx, int32_t* n_selected, cudaStream_t st) {
   SelShape sh = {NC, L, C, n_sink, n_recent};
   void* args[] = {&score_row, &sh, &k, &idx, &n_selected};
-  // few chunks: a small block, whose barriers are cheap; many: the widest one
-  if (NC <= 2048)
-    return launch_pdl(reinterpret_cast<const void*>(select_kernel<kFusedThreads>), dim3(1), dim3(kFusedThreads), args, st);
-  return launch_pdl(reinterpret_cast<const void*>(select_kernel<kSelThreads>), dim3(1), dim3(kSelThreads), args, st);
+  const void* kernel = NC <= 512    ? reinterpret_cast<const void*>(select_kernel<512, 1>)
+                       : NC <= 2048 ? reinterpret_cast<const void*>(select_kernel<512, 4>)
+                       : NC <= 8192 ? reinterpret_cast<const void*>(select_kernel<512, 16>)
+                                    : reinterpret_cast<const void*>(select_kernel<1024, 64>);
+  return launch_pdl(kernel, dim3(1), dim3(NC <= 8192 ? 512 : 1024), args, st);
 }
 
 cudaError_t spx_launch_gather(const void* dK, const void* dV, int n_layers, int H, int D, int L, int C,
@@ -338,7 +375,7 @@ cudaError_t spx_launch_select_gather(const float* score_row, int k, int n_sink, 
                                      const void* dV, int n_layers,
                                      int H, int D, int L, int C, long long s_layer, long long s_l, long long s_h,
                                      int32_t* idx, int32_t* n_selected, void* K_out, void* V_out,
-                                     int32_t* n_tokens_out, int32_t* status, cudaStream_t st) {
+                                     int32_t* n_tokens_out, int n_sm, int32_t* status, cudaStream_t st) {
   GatherArgs g;
   fill_gather_args(g, dK, dV, n_layers, H, D, L, C, s_layer, s_l, s_h, k, K_out, V_out, n_tokens_out, status);
   g.score = score_row;
@@ -349,6 +386,11 @@ cudaError_t spx_launch_select_gather(const float* score_row, int k, int n_sink, 
   g.n_recent = n_recent;
   void* args[] = {&g};
   const int keff = k < g.NC ? k : g.NC;
-  return launch_pdl(reinterpret_cast<const void*>(select_gather_kernel), dim3(keff * g.sub, n_layers, 2),
-                    dim3(kFusedThreads), args, st);
+  const long long segments = 2ll * n_layers * keff * (((long long)C * H * (D / 8) + 63) / 64);
+  const long long blocks = (segments + kSelThreads / 32 - 1) / (kSelThreads / 32);
+  const void* kernel = g.NC <= kSelThreads       ? reinterpret_cast<const void*>(select_gather_kernel<1>)
+                       : g.NC <= 4 * kSelThreads ? reinterpret_cast<const void*>(select_gather_kernel<4>)
+                       : g.NC <= 8 * kSelThreads ? reinterpret_cast<const void*>(select_gather_kernel<8>)
+                                                 : reinterpret_cast<const void*>(select_gather_kernel<16>);
+  return launch_pdl(kernel, dim3((unsigned)(blocks < 2 * n_sm ? blocks : 2 * n_sm)), dim3(kSelThreads), args, st);
 }

@@ -1,0 +1,40 @@
+"""specext_select_gather at the edges of its chunk-count classes, exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import specext_oracle as orc
+from paper_2505_20776_b200 import api
+from tests.guards import GuardedAlloc
+from tests.util import bf16_bits
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("L,C,k", [(511, 1, 7), (512, 1, 512), (513, 1, 512), (2048, 1, 1), (2049, 1, 1024), (4096, 1, 64),
+                                   (4097, 1, 33), (8192, 1, 1000), (8193, 1, 40), (65536, 1, 300), (20001, 3, 50)])
+@pytest.mark.parametrize("ties", [False, True])
+def test_select_gather_chunk_counts(cuda_device, L, C, k, ties):
+    """Chunk counts around what a thread holds (1, 4, 8, 16, 64 keys), with all keys distinct and with few distinct values
+    (ties at the k-th key): indices, count and copied cache are exact.  Strided draft cache, two layers."""
+    dev = cuda_device
+    NC = -(-L // C)
+    rng = np.random.default_rng(L + k)
+    row = rng.integers(0, 5, NC).astype(np.float32) if ties else rng.permutation(NC).astype(np.float32) + 1
+    scores = torch.from_numpy(np.stack([np.zeros(NC, np.float32), row])).to(dev)
+    g = GuardedAlloc(dev)
+    idx, ns, nt = (g.alloc((n,), torch.int32).fill_(-1) for n in (k, 1, 1))
+    status = g.alloc((1,), torch.int32).zero_()
+    big = torch.arange(2 * L * 3 * 16, dtype=torch.int32, device=dev).to(torch.int16).view(torch.bfloat16).view(2, L, 3, 16)
+    dK, dV = big[:, :, 1:, :8], big[:, :, :2, 8:]                 # 2 heads x 8 of wider rows
+    K, V = (g.alloc((2, k * C, 2, 8), torch.bfloat16).zero_() for _ in range(2))
+    api.specext_select_gather(scores, 1, L, C, k, dK, dV, idx, ns, K, V, nt, status)
+    assert api.specext_read_status(status) == 0
+    g.check()
+    want = orc.select_chunks(row, L, C, k, key_dtype=np.float32)
+    assert int(ns.item()) == len(want)
+    np.testing.assert_array_equal(idx[:len(want)].cpu().numpy(), want)
+    for out, src in ((K, dK), (V, dV)):
+        ref, _, n = orc.gather_kv(bf16_bits(src), bf16_bits(src), want, L, C)
+        assert int(nt.item()) == n
+        np.testing.assert_array_equal(bf16_bits(out)[:, :n], ref)
