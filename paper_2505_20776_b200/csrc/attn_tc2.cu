@@ -664,8 +664,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
             mass = a.ws + p.off_mass + rowbase * p.CPT;
             a.ws[p.off_mref + rowbase] = m_new;
           }
-          float csum = 0.f;
-          float cg[4] = {0.f, 0.f, 0.f, 0.f};      // chunk size 32: the tile's four chunk sums, stored as one float4
+          float cg[4] = {0.f, 0.f, 0.f, 0.f};      // the sums of the tile's four groups of 32 keys, stored in one piece
           uint32_t pk0[16], pk1[16], pk2[16], pk3[16];
           auto exp_chunk = [&](uint32_t (&v)[32], uint32_t (&pk)[16], int c) {
             // two elements per fma and per add (packed fp32 pairs); the exponential itself is per element
@@ -692,14 +691,8 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
             const float gs = (gs0 + gs1) + (gs2 + gs3);
             l += gs;
             if (score) {
-              if (SCORE == 1) {
+              if (SCORE == 1 || SCORE == 2) {
                 cg[c] = gs;
-              } else if (SCORE == 2) {
-                csum += gs;
-                if ((((c + 1) * 32) & (p.C - 1)) == 0) {
-                  mass[((c + 1) * 32) / p.C - 1] = csum;
-                  csum = 0.f;
-                }
               } else {
                 float acc = 0.f;
 #pragma unroll
@@ -720,6 +713,12 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
           exp_chunk(s2, pk2, 2);
           exp_chunk(s3, pk3, 3);
           if (SCORE == 1 && score) *reinterpret_cast<float4*>(mass) = make_float4(cg[0], cg[1], cg[2], cg[3]);
+          if (SCORE == 2 && score) {
+            if (p.C == 64)
+              *reinterpret_cast<float2*>(mass) = make_float2(cg[0] + cg[1], cg[2] + cg[3]);
+            else
+              *mass = (cg[0] + cg[1]) + (cg[2] + cg[3]);
+          }
           // the P buffer is shared by all tiles: the PV of the previous tile must have read it
           ok = wait_prev_pv();
           if (!ok) break;

@@ -114,69 +114,85 @@ __global__ void __launch_bounds__(256) merge_kernel(const __grid_constant__ Attn
   *reinterpret_cast<uint4*>(out) = pk;
 }
 
-// Block = 64 tree nodes x kScoreSlices slices of the KV heads, for one key tile and one group of VW
-// chunks of the tile.  Consecutive threads are consecutive nodes, whose G stacked rows lie next to
-// each other in the per-row arrays, so a warp reads whole lines; the VW chunk sums of a row are one
-// vector load.  A slice sums its KV heads in a fixed order and the slices are added in a fixed
-// order, so the result does not depend on the run.
-constexpr int kScoreSlices = 8;
+// Block = the rows of one row block x S slices of the KV heads, for one key tile and one group of VW chunks of it: a thread
+// adds up its row over the KV heads of its slice, so that every load of a warp is one contiguous piece and the loads of
+// four heads are in flight at once; the G rows of a node and the slices are added through shared memory.  All sums have
+// a fixed order, so the result does not depend on the run.
+// What bounds it: reading the chunk sums (20 bytes per row and tile of 32-key chunks) from L2, and latency when there are
+// few tiles: 2.8 us of a 4K call, 3.2 at 16K, 7.7 at 128K (42 MB, 5.5 TB/s).  A scored call against the form with one node
+// per thread, whose loads were strided and waited for one another: 4K 17.2 -> 16.4 us, 16K 28.5 -> 26.8, 64 query heads
+// with chunks of 64 53.9 -> 43.5 (there together with the one-piece store of the chunk sums in attn_tc2.cu).
+constexpr int kScoreThreads = 512;
 
 template <int VW>
-__global__ void __launch_bounds__(64 * kScoreSlices) score_kernel(const __grid_constant__ AttnArgs a) {
+__global__ void __launch_bounds__(kScoreThreads) score_kernel(const __grid_constant__ AttnArgs a) {
   const AttnPlan& p = a.plan;
-  __shared__ float part[kScoreSlices][64][VW];
+  __shared__ __align__(16) float part[kScoreThreads][VW];
   sm100::pdl_launch_dependents();
-  sm100::pdl_wait();                               // lse and the chunk sums are complete
-  const int t = blockIdx.z * 64 + threadIdx.x, slice = threadIdx.y;       // 64 tree nodes per block
-  const int tile = blockIdx.x;
+  const int rr = threadIdx.x, slice = threadIdx.y, n_slices = blockDim.y;
+  const int tile = blockIdx.x, rblk = blockIdx.z;
   const int c0 = blockIdx.y * VW;                  // first chunk of the group inside the tile
+  const int r = rblk * p.RB + rr;
+  const int t = r / p.G, i = r - t * p.G;
   float acc[VW];
 #pragma unroll
   for (int k = 0; k < VW; ++k) acc[k] = 0.f;
-  if (t < p.T) {
-    for (int g = slice; g < p.Hkv; g += kScoreSlices) {
-      for (int i = 0; i < p.G; ++i) {
-        const int r = t * p.G + i;
-        const int rblk = r / p.RB, rr = r - rblk * p.RB;
-        const int prob = g * p.n_rblk + rblk;
-        const long long base = ((long long)prob * p.TPH + tile) * p.RB + rr;
-        const float lse2 = a.lse[(long long)(g * p.G + i) * p.T + t] * kLog2e;
-        const float f = exp2f(a.ws[p.off_mref + base] - lse2);
-        const float* m = a.ws + p.off_mass + base * p.CPT + c0;
-        if (VW == 4) {
-          const float4 v = *reinterpret_cast<const float4*>(m);
-          acc[0] = fmaf(v.x, f, acc[0]);
-          acc[1 % VW] = fmaf(v.y, f, acc[1 % VW]);
-          acc[2 % VW] = fmaf(v.z, f, acc[2 % VW]);
-          acc[3 % VW] = fmaf(v.w, f, acc[3 % VW]);
-        } else {
+  sm100::pdl_wait();                               // lse and the chunk sums are complete
+  if (r < p.rows) {
+    for (int g0 = slice; g0 < p.Hkv; g0 += 4 * n_slices) {
+      float m[4][VW], ref[4], lse[4];
 #pragma unroll
-          for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[k], f, acc[k]);
+      for (int q = 0; q < 4; ++q) {
+        const int g = g0 + q * n_slices;
+        if (g < p.Hkv) {
+          const long long base = ((long long)(g * p.n_rblk + rblk) * p.TPH + tile) * p.RB + rr;
+          const float* src = a.ws + p.off_mass + base * p.CPT + c0;
+          if (VW == 4) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+            m[q][0] = v.x; m[q][1 % VW] = v.y; m[q][2 % VW] = v.z; m[q][3 % VW] = v.w;
+          } else if (VW == 2) {
+            const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
+            m[q][0] = v.x; m[q][1 % VW] = v.y;
+          } else {
+            m[q][0] = __ldcg(src);
+          }
+          ref[q] = __ldcg(a.ws + p.off_mref + base);
+          lse[q] = __ldcg(a.lse + (long long)(g * p.G + i) * p.T + t);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (g0 + q * n_slices < p.Hkv) {
+          const float f = exp2f(ref[q] - lse[q] * kLog2e);
+#pragma unroll
+          for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[q][k], f, acc[k]);
         }
       }
     }
   }
 #pragma unroll
-  for (int k = 0; k < VW; ++k) part[slice][threadIdx.x][k] = acc[k];
+  for (int k = 0; k < VW; ++k) part[slice * p.RB + rr][k] = acc[k];
   __syncthreads();
-  if (slice == 0 && t < p.T) {
-    const float inv = 1.f / (float)p.Hq;
-#pragma unroll
-    for (int k = 0; k < VW; ++k) {
+  const int nodes = p.RB / p.G;                    // nodes of a row block
+  const float inv = 1.f / (float)p.Hq;
+  for (int o = slice * p.RB + rr; o < nodes * VW; o += n_slices * p.RB) {
+    const int tt = o / VW, k = o - tt * VW;
+    const int node = rblk * nodes + tt, c = tile * p.CPT + c0 + k;
+    if (node < p.T && c < p.NC) {
       float sum = 0.f;
-#pragma unroll
-      for (int q = 0; q < kScoreSlices; ++q) sum += part[q][threadIdx.x][k];
-      const int c = tile * p.CPT + c0 + k;
-      if (c < p.NC) a.chunk_score[(long long)t * p.NC + c] = sum * inv;
+      for (int s = 0; s < n_slices; ++s)
+        for (int j = 0; j < p.G; ++j) sum += part[s * p.RB + tt * p.G + j][k];
+      a.chunk_score[(long long)node * p.NC + c] = sum * inv;
     }
   }
 }
 
 template <int VW>
-cudaError_t launch_score(const AttnArgs& a, dim3 grid, cudaStream_t st) {
+cudaError_t launch_score(const AttnArgs& a, cudaStream_t st) {
+  const AttnPlan& p = a.plan;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(64, kScoreSlices);
+  cfg.gridDim = dim3(p.TPH, p.CPT / VW, p.n_rblk);
+  cfg.blockDim = dim3(p.RB, kScoreThreads / p.RB);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -214,13 +230,7 @@ cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches
   *n_launches += 1;
   if (e != cudaSuccess) return e;
   if (p.want_score && p.NC > 0) {
-    if (p.CPT >= 4) {
-      e = launch_score<4>(a, dim3(p.TPH, p.CPT / 4, (p.T + 63) / 64), st);
-    } else if (p.CPT == 2) {
-      e = launch_score<2>(a, dim3(p.TPH, 1, (p.T + 63) / 64), st);
-    } else {
-      e = launch_score<1>(a, dim3(p.TPH, 1, (p.T + 63) / 64), st);
-    }
+    e = p.CPT >= 4 ? launch_score<4>(a, st) : p.CPT == 2 ? launch_score<2>(a, st) : launch_score<1>(a, st);
     *n_launches += 1;
   }
   return e;
