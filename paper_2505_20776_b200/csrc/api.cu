@@ -65,42 +65,26 @@ int sm_count() {
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-int build_plan(const specext_attn_desc* d, AttnPlan* out) {
-  if (!d) return SPECEXT_ERR_INVALID_ARG;
-  if (d->n_q_heads < 1 || d->n_kv_heads < 1 || d->n_q_heads % d->n_kv_heads != 0) return SPECEXT_ERR_INVALID_ARG;
-  if (d->prefix_len < 0 || d->prefix_len > (1 << 24)) return SPECEXT_ERR_INVALID_ARG;
-  if (d->n_tree < 1 || d->n_tree > kSpxMaxTree) return SPECEXT_ERR_UNSUPPORTED;
-  if (d->head_dim != 64 && d->head_dim != 128) return SPECEXT_ERR_UNSUPPORTED;
-  if (!is_pow2(d->chunk_size) || d->chunk_size > 128) return SPECEXT_ERR_UNSUPPORTED;
-  const int G = d->n_q_heads / d->n_kv_heads;
-  if (!is_pow2(G) || G > 64) return SPECEXT_ERR_UNSUPPORTED;
-  if (!(d->softmax_scale >= 0.f) || !std::isfinite(d->softmax_scale)) return SPECEXT_ERR_INVALID_ARG;
-  const long long strides[8] = {d->q_stride_t, d->q_stride_h, d->kv_stride_l, d->kv_stride_h,
-                                d->tkv_stride_t, d->tkv_stride_h, d->o_stride_t, d->o_stride_h};
-  for (long long s : strides)
-    if (s < d->head_dim || (s & 7) != 0) return SPECEXT_ERR_INVALID_ARG;
-
-  AttnPlan p;
-  std::memset(&p, 0, sizeof(p));
-  p.Hq = d->n_q_heads; p.Hkv = d->n_kv_heads; p.G = G; p.D = d->head_dim;
-  p.L = d->prefix_len; p.T = d->n_tree; p.C = d->chunk_size;
-  p.rows = G * p.T;
-  // Kernel: pairs of CTAs on 256-row blocks for head_dim 128 and more than 128 stacked rows; otherwise one CTA on
-  // 128-row blocks (want != 0 only in the test library).
-  const int want = tuning_kernel();
-  const bool pair = p.D == 128 && p.rows > 128 && want != 2;
-  p.kernel = want == 1 ? 1 : (pair ? 3 : 2);
-  p.RB = pair ? 256 : 128;
-  p.q_rows = p.kernel == 2 && p.D == 128 && p.rows <= 64 ? 64 : 128;
+// Row blocks, workers and workspace of one kernel (plan.kernel); cluster > 0: its workers merge in clusters of that size.
+int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
+  AttnPlan& p = *plan;
+  p.kernel = kernel;
+  p.cluster = cluster;
+  p.RB = row_block;
+  p.q_rows = kernel == 2 && p.D == 128 && p.rows <= 64 ? 64 : 128;
   p.n_rblk = (p.rows + p.RB - 1) / p.RB;
   p.NP = p.Hkv * p.n_rblk;
-  p.TPH = (p.L + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS;
-  p.UPP = p.TPH + 1;
   const long long U = (long long)p.NP * p.UPP;
   if (U > (1ll << 30)) return SPECEXT_ERR_UNSUPPORTED;
   p.U = (int)U;
   const int min_units = tuning_min_units();
-  if (p.kernel == 3) {
+  if (cluster > 0) {
+    p.cpp = cluster;
+    p.n_cta = p.NP * p.cpp;
+    p.q = p.UPP / p.cpp;
+    p.rem = p.UPP % p.cpp;
+    p.max_segs = p.cpp;
+  } else if (p.kernel == 3) {
     // one worker = a cluster of two CTAs; every problem gets the same number of workers when possible
     const int n_workers = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
     if (p.NP <= n_workers) {
@@ -130,12 +114,7 @@ int build_plan(const specext_attn_desc* d, AttnPlan* out) {
     p.max_segs = (p.UPP + p.q - 1) / p.q + 1;
   }
   if (p.max_segs > p.n_cta) p.max_segs = p.n_cta;
-  p.n_slots = p.n_cta + p.NP - 1;
-  p.CPT = SPX_TILE_KEYS / p.C;
-  p.NC = (p.L + p.C - 1) / p.C;
-  p.want_score = d->want_chunk_score != 0;
-  const float scale = d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / std::sqrt((float)p.D);
-  p.scale2 = scale * 1.44269504088896340736f;
+  p.n_slots = p.cluster > 0 ? 1 : p.n_cta + p.NP - 1;           // (a cluster merges in shared memory)
   long long off = 0;
   p.off_part_o = off; off += (long long)p.n_slots * p.D * p.RB;
   p.off_part_m = off; off += (long long)p.n_slots * p.RB;
@@ -145,6 +124,86 @@ int build_plan(const specext_attn_desc* d, AttnPlan* out) {
     p.off_mref = off; off += (long long)p.NP * p.TPH * p.RB;
   }
   p.total_floats = off;
+  return SPECEXT_OK;
+}
+
+// Size of the cluster whose CTAs share the key tiles of a problem and merge among themselves, or 0 for workers that leave
+// partial results to the merge kernel.
+int cluster_size(const AttnPlan& p, bool pair) {
+  const long long np = (long long)p.Hkv * ((p.rows + 127) / 128);
+  int dev = -1, size = 0;
+  if (np > sm_count() / 2) return 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  // the largest clusters of which one per problem is resident at once
+  for (int s = 8; s >= 2 && size == 0; --s)
+    if (s <= p.UPP && np * s <= sm_count() && np <= spx_verify_max_clusters(dev, s)) size = s;
+  if (size == 0) return 0;
+  const int tiles = (p.UPP + size - 1) / size;
+  int split;
+  if (pair) {
+    const long long np2 = (long long)p.Hkv * ((p.rows + 255) / 256), workers = sm_count() / 2;
+    split = (int)(np2 <= workers ? (p.UPP + workers / np2 - 1) / (workers / np2) : (np2 * p.UPP + workers - 1) / workers);
+  } else {
+    split = (int)((np * p.UPP + sm_count() - 1) / sm_count());
+  }
+  // What merging in the cluster saves (4 us with the second launch) against the tiles it adds; the pairs, whose CTAs fetch
+  // half of every K/V tile, win again when the tiles are many.  us per call, split / cluster (32 query / 8 KV heads unless said):
+  //   60 nodes: 1K 10.9 / 10.6, 2K 11.6 / 11.5 (3 tiles against 2), 4K 13.4 / 14.4 (5 against 4)
+  //   60 nodes, 64 query heads: 1K 13.4 / 11.4, 4K 18.3 / 16.8 (9 against 9), 16K 36.6 / 38.4 (33 against 33)
+  //   60 nodes, 32 KV heads: 1K 13.5 / 10.9, 8K 31.6 / 29.3 (17 against 15), 32K 91.3 / 88.9 (65 against 56)
+  //   1 node: 2K 10.8 / 8.5, 8K 15.8 / 14.8 (9 against 4), 16K 20.4 / 22.5 (17 against 7)
+  //   12 x 64 heads: 4K 11.7 / 9.7 (5 against 3);  60 nodes, 32 x 64 query / 8 KV heads, 16K: 24.0 / 24.5 (19 against 14)
+  const int most = pair ? (tiles <= 16 ? (split > 3 ? split : 3) : 0)
+                        : split + (p.D == 64 ? 3 : split > 30 ? split / 6 : 5);
+  if (tiles > most) return 0;
+  while (size > 2 && (p.UPP + size - 2) / (size - 1) == tiles) --size;     // no more CTAs than the tile count needs
+  return size;
+}
+
+int build_plan(const specext_attn_desc* d, AttnPlan* out) {
+  if (!d) return SPECEXT_ERR_INVALID_ARG;
+  if (d->n_q_heads < 1 || d->n_kv_heads < 1 || d->n_q_heads % d->n_kv_heads != 0) return SPECEXT_ERR_INVALID_ARG;
+  if (d->prefix_len < 0 || d->prefix_len > (1 << 24)) return SPECEXT_ERR_INVALID_ARG;
+  if (d->n_tree < 1 || d->n_tree > kSpxMaxTree) return SPECEXT_ERR_UNSUPPORTED;
+  if (d->head_dim != 64 && d->head_dim != 128) return SPECEXT_ERR_UNSUPPORTED;
+  if (!is_pow2(d->chunk_size) || d->chunk_size > 128) return SPECEXT_ERR_UNSUPPORTED;
+  const int G = d->n_q_heads / d->n_kv_heads;
+  if (!is_pow2(G) || G > 64) return SPECEXT_ERR_UNSUPPORTED;
+  if (!(d->softmax_scale >= 0.f) || !std::isfinite(d->softmax_scale)) return SPECEXT_ERR_INVALID_ARG;
+  const long long strides[8] = {d->q_stride_t, d->q_stride_h, d->kv_stride_l, d->kv_stride_h,
+                                d->tkv_stride_t, d->tkv_stride_h, d->o_stride_t, d->o_stride_h};
+  for (long long s : strides)
+    if (s < d->head_dim || (s & 7) != 0) return SPECEXT_ERR_INVALID_ARG;
+
+  AttnPlan p;
+  std::memset(&p, 0, sizeof(p));
+  p.Hq = d->n_q_heads; p.Hkv = d->n_kv_heads; p.G = G; p.D = d->head_dim;
+  p.L = d->prefix_len; p.T = d->n_tree; p.C = d->chunk_size;
+  p.rows = G * p.T;
+  p.TPH = (p.L + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS;
+  p.UPP = p.TPH + 1;
+  p.CPT = SPX_TILE_KEYS / p.C;
+  p.NC = (p.L + p.C - 1) / p.C;
+  p.want_score = d->want_chunk_score != 0;
+  const float scale = d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / std::sqrt((float)p.D);
+  p.scale2 = scale * 1.44269504088896340736f;
+  // Kernel: pairs of CTAs on 256-row blocks for head_dim 128 and more than 128 stacked rows; otherwise one CTA on
+  // 128-row blocks (want != 0 only in the test library).
+  const int want = tuning_kernel();
+  const bool pair = p.D == 128 && p.rows > 128 && want != 2;
+  int rc = lay_out(&p, want == 1 ? 1 : (pair ? 3 : 2), pair ? 256 : 128, 0);
+  if (rc != SPECEXT_OK) return rc;
+  const int size = want == 0 && tuning_min_units() == 1 ? cluster_size(p, pair) : 0;
+  if (size > 0) {
+    // (the workspace keeps its size: it does not depend on what clusters the device holds)
+    const long long split_floats = p.total_floats;
+    rc = lay_out(&p, 2, 128, size);
+    if (rc != SPECEXT_OK) return rc;
+    if (p.total_floats < split_floats) p.total_floats = split_floats;
+  }
   *out = p;
   return SPECEXT_OK;
 }

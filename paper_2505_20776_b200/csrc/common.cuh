@@ -98,6 +98,7 @@ cudaError_t spx_launch_attn_simt(const AttnArgs& a, cudaStream_t st, int* n_laun
 #endif
 cudaError_t spx_launch_attn_tc2(const AttnArgs& a, cudaStream_t st, int* n_launches);
 cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launches);
+int spx_verify_max_clusters(int dev, int size);
 cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches);
 
 #endif  // SPECEXT_COMMON_CUH_

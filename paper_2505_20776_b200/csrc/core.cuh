@@ -132,10 +132,10 @@ __device__ __forceinline__ void tma_load_hint(uint32_t dst, const CUtensorMap* m
 }
 
 // ---- set-up and end of a CTA ---------------------------------------------------------------------------
-// Barriers by the producer warp, tensor memory by the MMA warp; the cluster barrier (block barrier) that publishes them
-// is completed by setup_wait, so that what needs neither can run in between.
+// Barriers by the producer warp, tensor memory by the MMA warp, and the cluster barrier (block barrier) that publishes
+// them.  None of it touches global memory: it runs ahead of the dependency wait, under the kernel before.
 template <int PAIR>
-__device__ __forceinline__ void setup_begin(Ctrl* ctl, int warp, int lane) {
+__device__ __forceinline__ void setup(Ctrl* ctl, int warp, int lane) {
   if (warp == kProducerWarp) {
     if (lane < kMaxStages) {
       mbar_init(&ctl->k_full[lane], PAIR);
@@ -173,11 +173,12 @@ __device__ __forceinline__ void setup_begin(Ctrl* ctl, int warp, int lane) {
     }
   }
   tc_fence_before();
-  if constexpr (PAIR == 2) cluster_arrive();
-}
-template <int PAIR>
-__device__ __forceinline__ void setup_wait() {
-  if constexpr (PAIR == 2) cluster_wait(); else __syncthreads();
+  if constexpr (PAIR == 2) {
+    cluster_arrive();
+    cluster_wait();
+  } else {
+    __syncthreads();
+  }
   tc_fence_after();
 }
 // The peer may still signal this CTA's barriers or read its halves, and tensor memory is freed by one warp for all:

@@ -205,19 +205,20 @@ cudaError_t launch_score(const AttnArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches) {
+namespace {
+
+// Launched so that its blocks may be resident (waiting) before the attention kernel has finished.
+// Blocks become resident wherever an SM has room, so without a limit the SMs that the attention
+// kernel leaves first would take eight blocks each and a fraction of the SMs would do all the work:
+// an (unused) dynamic shared-memory request caps residency at one block per SM (measured: 1.1 us
+// per call faster than two per SM, which in turn was 2 us faster than no cap).
+cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st) {
   const AttnPlan& p = a.plan;
-  const dim3 grid(p.NP * (p.RB / 32), p.D / 64);
-  // Launched so that its blocks may be resident (waiting) before the attention kernel has finished.
-  // Blocks become resident wherever an SM has room, so without a limit the SMs that the attention
-  // kernel leaves first would take eight blocks each and a fraction of the SMs would do all the work:
-  // an (unused) dynamic shared-memory request caps residency at one block per SM (measured: 1.1 us
-  // per call faster than two per SM, which in turn was 2 us faster than no cap).
   static SpxOncePerDevice once;
   const cudaError_t ec = spx_opt_in_smem(merge_kernel, kMergeSmemCap, &once);
   if (ec != cudaSuccess) return ec;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
+  cfg.gridDim = dim3(p.NP * (p.RB / 32), p.D / 64);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = kMergeSmemCap;
   cfg.stream = st;
@@ -226,9 +227,21 @@ cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, merge_kernel, a);
-  *n_launches += 1;
-  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, merge_kernel, a);
+}
+
+}  // namespace
+
+// What follows the attention kernel: the merge of the partial results (unless its clusters have merged them), then the
+// chunk scores.
+cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches) {
+  const AttnPlan& p = a.plan;
+  cudaError_t e = cudaSuccess;
+  if (p.cluster == 0) {
+    e = launch_merge(a, st);
+    *n_launches += 1;
+    if (e != cudaSuccess) return e;
+  }
   if (p.want_score && p.NC > 0) {
     e = p.CPT >= 4 ? launch_score<4>(a, st) : p.CPT == 2 ? launch_score<2>(a, st) : launch_score<1>(a, st);
     *n_launches += 1;

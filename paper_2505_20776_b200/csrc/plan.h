@@ -39,6 +39,7 @@ struct AttnPlan {
   int U;           // total units
   int n_cta;       // workers of the attention kernel (<= U)
   int kernel;      // 1 CUDA-core kernel, 2 one-CTA tensor-core kernel, 3 paired-CTA tensor-core kernel
+  int cluster;     // > 0: the cpp workers of a problem are one cluster of this many CTAs and merge among themselves
   int cpp;         // workers per problem, or 0 when the line of units is cut without regard to problems
   int q, rem;      // cpp > 0: UPP = q*cpp + rem;  cpp == 0: U = q*n_cta + rem
   int n_slots;     // n_cta + NP - 1 partial slots

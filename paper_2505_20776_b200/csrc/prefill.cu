@@ -73,12 +73,16 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const G geo(128);
 
-  setup_begin<2>(ctl, warp, lane);
-  pdl_launch_dependents();
-  pdl_wait();
+  if (warp == kProducerWarp && lane == 0) {
+    prefetch_tensormap(&maps.q);
+    prefetch_tensormap(&maps.k);
+    prefetch_tensormap(&maps.v);
+  }
+  setup<2>(ctl, warp, lane);
   const uint32_t rank = cluster_rank();
   PrefillWork work(a, blockIdx.x >> 1);
-  setup_wait<2>();
+  pdl_launch_dependents();
+  pdl_wait();
   bool ok = true;
 
   if (warp == kProducerWarp) {

@@ -9,9 +9,12 @@
 // What bounds it: memory.  A K/V tile of 64 KB is 3.0 K cycles of an SM's share of the copy rate, a softmax warpgroup
 // needs ~3.3 K for a tile and two alternate.  Measured (us per call, replayed; before: two row tiles of one CTA, whose
 // second softmax warpgroup had nothing to do here and whose S, P and PV of a tile formed one chain):
-//   32 heads of their own, 60 nodes, 8K prefix    40.3 -> 30.5 (scored 62.5 -> 35.1)   4.4 TB/s of K/V; 16K 64.9 -> 50.5
-//   32 query / 8 KV heads, one node, 16K prefix   27.9 -> 20.0 (scored 37.5 -> 22.7)   128K 113.8 -> 88.8 = 6.0 TB/s
-//   12 heads x 64, 8 nodes, 4K prefix             15.6 -> 11.8
+//   32 heads of their own, 60 nodes, 8K prefix    40.3 -> 27.3   4.9 TB/s of K/V; 16K 64.9 -> 46.5
+//   32 query / 8 KV heads, one node, 16K prefix   27.9 -> 19.3   128K 113.8 -> 87.5 = 6.1 TB/s
+//   12 heads x 64, 8 nodes, 4K prefix             15.6 -> 9.6
+//
+// FUSED: the workers of a problem form one cluster and merge their results through each other's shared memory, so that the
+// call is one kernel: no partials in memory, no second launch waiting for the slowest block of the first.
 //
 // Warps: 0-7 softmax (two warpgroups), 8 TMA producer of K and V, 9 issuer of the S MMAs, 10 of the PV MMAs, 11 ancestor
 // masks of the tree and TMA producer of Q.  Every wait is bounded; an expired wait raises SPECEXT_ERR_TIMEOUT, and all
@@ -20,6 +23,8 @@
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory allocation and the
 // start-up barrier run while the kernel before it in the stream finishes; global memory is touched only after
 // griddepcontrol.wait.
+#include <atomic>
+
 #include "common.cuh"
 #include "core.cuh"
 #include "tmap.h"
@@ -62,11 +67,208 @@ struct VerifyWork {
   __device__ __forceinline__ int tile(int j) const { return DEVLEN ? spx_seg_tile(p, sg, tile_lo, j) : tile_lo + j; }
 };
 
+// End of a worker that is one of the CTAs of a cluster: every CTA has an unnormalised O, a reference maximum and a row sum
+// for the same rows.  Each CTA sends every part of its O to the CTA that owns it, and the owner adds the parts up and writes
+// O.  What is received lies where Q and the rings were, so the CTAs meet once before sending and once after.
+//
+// Who owns what depends on the number of rows.  More than 32: the columns are dealt in units of 8 (unit u to CTA u mod
+// size), so that a store of a warp is 512 contiguous bytes of one CTA.  Up to 32: the rows are dealt in equal runs, which
+// needs fewer instructions, addresses and (m, l) copies, but each store of a warp goes to 32 places.  us per call, by
+// columns / by rows: 4 rows on a 2K cache 9.2 / 8.7, 12 x 64 heads with 8 rows 7.7 / 7.2, 40 rows 8.2 / 8.2, 60 rows at 1K
+// 10.9 / 11.5, 120 rows at 8K 17.2 / 18.3.  (Bulk copies between the CTAs instead of stores: 9.2, 7.7, 8.1, 11.6, 17.7.)
+struct MergeCtx {
+  int cs, rank;            // CTAs of the cluster, this one
+  int g, rblk, n_rows;     // the problem and its rows
+  int log_g;
+  float m, l;              // of this thread's row in this CTA
+  bool any;                // this CTA had a key tile (else: zeros of weight zero)
+};
+constexpr int kMaxCluster = 8;
+constexpr float kLn2 = 0.693147180559945309417f;
+
+// This thread's half row of O.
+template <int D>
+__device__ __forceinline__ void own_half_row(const RowCtx& rc, bool any, uint32_t (&v)[D / 64][32]) {
+  if (any) {
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c) tmem_ld32(rc.lane_tmem + kColO + rc.w * (D / 2) + c * 32, v[c]);
+    tmem_wait_ld();
+    tc_fence_before();
+  } else {
+#pragma unroll
+    for (int k = 0; k < D / 2; ++k) v[k / 32][k % 32] = 0u;
+  }
+}
+
+template <int D>
+__device__ __forceinline__ void merge_by_rows(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const MergeCtx& mc,
+                                              bool ok) {
+  constexpr int kCols = D / 4;                                     // 16-byte columns of a row
+  const AttnPlan& p = a.plan;
+  const int cs = mc.cs, run = (mc.n_rows + cs - 1) / cs;           // rows of a CTA
+  // received: [source CTA][row of the run][column, swizzled by the row so that a warp's rows use all banks]
+  float4* part = reinterpret_cast<float4*>(base);
+  float2* ml = reinterpret_cast<float2*>(part + cs * run * kCols);
+  if (ok && rc.row_t - rc.lane < mc.n_rows) {
+    uint32_t v[D / 64][32];
+    own_half_row<D>(rc, mc.any, v);
+    if (rc.row_t < mc.n_rows) {
+      const int owner = rc.row_t / run, slot = mc.rank * run + rc.row_t - owner * run;
+      const uint32_t dst = map_to_cta(smem_u32(part + slot * kCols), owner);
+#pragma unroll
+      for (int c = 0; c < kCols / 2; ++c)
+        st_cluster_v4(dst + (((rc.w * (kCols / 2) + c) ^ (rc.row_t & (kCols - 1))) << 4), v[c / 8][c % 8 * 4],
+                      v[c / 8][c % 8 * 4 + 1], v[c / 8][c % 8 * 4 + 2], v[c / 8][c % 8 * 4 + 3]);
+      if (rc.w == 0) st_cluster_v2(map_to_cta(smem_u32(ml + slot), owner), mc.m, mc.l);
+    }
+  }
+  __syncwarp();
+  cluster_sync();
+  if (!ok) return;
+  const int n_mine = min(run, mc.n_rows - mc.rank * run);
+  constexpr int kRowsPerWarp = 32 / kCols;                         // 1, or 2 with head_dim 64
+  const int sub = rc.lane / kCols, col = rc.lane - sub * kCols;
+  for (int i = (rc.w * 4 + rc.row_t / 32) * kRowsPerWarp + sub; i < n_mine; i += 8 * kRowsPerWarp) {
+    const int row = mc.rank * run + i;
+    float w[kMaxCluster], M = -INFINITY, Z = 0.f;
+    float4 x[kMaxCluster];
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      if (c < cs) {
+        w[c] = ml[c * run + i].x;
+        x[c] = part[(c * run + i) * kCols + (col ^ (row & (kCols - 1)))];
+        M = fmaxf(M, w[c]);
+      }
+    }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      if (c < cs) {
+        const float f = ex2_approx(w[c] - M);
+        Z = fmaf(ml[c * run + i].y, f, Z);
+        acc.x = fmaf(f, x[c].x, acc.x);
+        acc.y = fmaf(f, x[c].y, acc.y);
+        acc.z = fmaf(f, x[c].z, acc.z);
+        acc.w = fmaf(f, x[c].w, acc.w);
+      }
+    }
+    const float inv = 1.f / Z;
+    const int r = mc.rblk * 128 + row, t = r >> mc.log_g, h = mc.g * p.G + (r & (p.G - 1));
+    *reinterpret_cast<uint2*>(a.O + (long long)t * a.o_st + (long long)h * a.o_sh + col * 4) =
+        make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
+    if (col == 0) a.lse[(long long)h * p.T + t] = (M + log2f(Z)) * kLn2;
+  }
+}
+
+template <int D>
+__device__ __forceinline__ void merge_by_columns(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const MergeCtx& mc,
+                                                 bool ok) {
+  constexpr int kUnits = D / 8;
+  const AttnPlan& p = a.plan;
+  const int cs = mc.cs;
+  int slot = rc.w * (kUnits / 2) / cs, owner = rc.w * (kUnits / 2) - slot * cs;      // of this warpgroup's first unit
+  float4* part = reinterpret_cast<float4*>(base);                                    // [slot][source CTA][2][128 rows]
+  float2* ml = reinterpret_cast<float2*>(part + (kUnits + cs - 1) / cs * cs * 256);  // [source CTA][128 rows]
+  if (ok && rc.row_t - rc.lane < mc.n_rows) {
+    uint32_t v[D / 64][32];
+    own_half_row<D>(rc, mc.any, v);
+    const uint32_t mine = smem_u32(part) + mc.rank * 4096 + rc.row_t * 16;
+    if (rc.w == 0)
+      for (int c = 0; c < cs; ++c)
+        st_cluster_v2(map_to_cta(smem_u32(ml + mc.rank * 128 + rc.row_t), c), mc.m, mc.l);
+#pragma unroll
+    for (int u = 0; u < kUnits / 2; ++u) {
+      const uint32_t dst = map_to_cta(mine + slot * cs * 4096, owner);
+      if (++owner == cs) {
+        owner = 0;
+        ++slot;
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int k = u * 8 + q * 4;
+        st_cluster_v4(dst + q * 2048, v[k / 32][k % 32], v[k / 32][k % 32 + 1], v[k / 32][k % 32 + 2], v[k / 32][k % 32 + 3]);
+      }
+    }
+  }
+  __syncwarp();
+  cluster_sync();
+  if (!ok) return;
+  // 8 warps over (slot, group of 32 rows)
+  const int groups = (mc.n_rows + 31) / 32;
+  int group = rc.w * 4 + rc.row_t / 32;
+  slot = 0;
+  for (;;) {
+    while (group >= groups) {
+      group -= groups;
+      ++slot;
+    }
+    const int u = slot * cs + mc.rank;
+    if (u >= kUnits) break;
+    const int row = group * 32 + rc.lane;
+    const float4* src = part + slot * cs * 256 + row;
+    float w[kMaxCluster], M = -INFINITY, Z = 0.f;
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      w[c] = c < cs ? ml[c * 128 + row].x : -INFINITY;
+      M = fmaxf(M, w[c]);
+    }
+    float4 acc0 = make_float4(0.f, 0.f, 0.f, 0.f), acc1 = acc0;
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      if (c < cs) {
+        const float f = ex2_approx(w[c] - M);
+        const float4 x = src[c * 256], y = src[c * 256 + 128];
+        Z = fmaf(ml[c * 128 + row].y, f, Z);
+        acc0.x = fmaf(f, x.x, acc0.x);
+        acc0.y = fmaf(f, x.y, acc0.y);
+        acc0.z = fmaf(f, x.z, acc0.z);
+        acc0.w = fmaf(f, x.w, acc0.w);
+        acc1.x = fmaf(f, y.x, acc1.x);
+        acc1.y = fmaf(f, y.y, acc1.y);
+        acc1.z = fmaf(f, y.z, acc1.z);
+        acc1.w = fmaf(f, y.w, acc1.w);
+      }
+    }
+    if (row < mc.n_rows) {
+      const float inv = 1.f / Z;
+      const int r = mc.rblk * 128 + row, t = r >> mc.log_g, h = mc.g * p.G + (r & (p.G - 1));
+      *reinterpret_cast<uint4*>(a.O + (long long)t * a.o_st + (long long)h * a.o_sh + u * 8) =
+          make_uint4(pack_bf16x2(acc0.x * inv, acc0.y * inv), pack_bf16x2(acc0.z * inv, acc0.w * inv),
+                     pack_bf16x2(acc1.x * inv, acc1.y * inv), pack_bf16x2(acc1.z * inv, acc1.w * inv));
+      if (u == 0) a.lse[(long long)h * p.T + t] = (M + log2f(Z)) * kLn2;
+    }
+    group += 8;
+  }
+}
+
+template <int D, class Work>
+__device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const Work& work,
+                                                 bool ok, float m_loc, float l) {
+  const AttnPlan& p = a.plan;
+  MergeCtx mc;
+  mc.cs = p.cluster;
+  mc.rank = (int)cluster_rank();
+  mc.g = work.prob / p.n_rblk;
+  mc.rblk = work.prob - mc.g * p.n_rblk;
+  mc.n_rows = min(128, p.rows - mc.rblk * 128);
+  mc.log_g = 31 - __clz(p.G);
+  mc.any = work.n > 0;
+  mc.m = -1e30f;
+  mc.l = 0.f;
+  if (ok && mc.any) ok = segment_end(rc, work.n - 1, 0, m_loc, l, mc.m, mc.l);
+  __syncwarp();
+  cluster_sync();
+  // (by the rows of the whole call: the CTAs of all problems take the same path)
+  if (p.rows <= 32) merge_by_rows<D>(a, rc, base, mc, ok);
+  else merge_by_columns<D>(a, rc, base, mc, ok);
+  return ok;
+}
+
 // SCORE: 0 no chunk sums; otherwise the class of the chunk size, so that each variant carries only the code it runs:
 // 1 chunks of 32 keys, 2 chunks of 64 or 128 keys, 3 chunks of fewer than 32 keys.
 // DEVLEN: the prefix length is read from device memory (a.L_dev) and may be shorter than the planned capacity p.L; the
 // instantiation without it carries none of that code.
-template <int D, int SCORE, bool DEVLEN>
+template <int D, int SCORE, bool DEVLEN, bool FUSED>
 __global__ void __launch_bounds__(kThreads, 1)
 verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ VerifyMaps maps) {
   using G = Geo<1, D>;
@@ -79,23 +281,28 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const G geo(p.q_rows);
 
-  setup_begin<1>(ctl, warp, lane);
-  // The kernel after this one (the merge) may be set up while this one runs; this one touches global memory only once
-  // the kernel before it has completed (its set-up so far has used none).
-  pdl_launch_dependents();
-  pdl_wait();
-
+  setup<1>(ctl, warp, lane);
   const int worker = blockIdx.x;
   const int unit_lo = spx_unit_start(p, worker), unit_hi = spx_unit_start(p, worker + 1);
+  // The kernel after this one may be set up while this one runs; this one touches global memory only once the kernel
+  // before it has completed.
+  pdl_launch_dependents();
+  pdl_wait();
   if (warp == kProducerWarp && lane == 0 && unit_lo < unit_hi && !DEVLEN) {
-    // The first K/V tile can only be loaded once the barriers are known to exist; until then it is pulled into L2.
+    // The first tile is asked for in L2 as well, in one piece for K and V ahead of the ring's loads: 8K prefix with 32 KV
+    // heads 28.5 -> 27.3 us, one node on 16K 20.5 -> 19.6.  The second one too where a worker has several: 16K 19.6 ->
+    // 19.3, 128K 88.3 -> 87.5, but 2K 8.1 -> 8.4.
     const int prob = unit_lo / p.UPP, tile = unit_lo - prob * p.UPP, g = prob / p.n_rblk;
-    const bool is_tree = tile == p.TPH;
-    const int key0 = is_tree ? 0 : tile * SPX_TILE_KEYS;
-    for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.kt : &maps.kp, 64 * ds, g, key0);
-    for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * ds, g, key0);
+    for (int i = 0; i < (unit_hi - unit_lo >= 6 ? 2 : 1); ++i) {
+      if (tile + i > p.TPH) break;
+      const bool is_tree = tile + i == p.TPH;
+      const int key0 = is_tree ? 0 : (tile + i) * SPX_TILE_KEYS;
+#pragma unroll
+      for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.kt : &maps.kp, 64 * ds, g, key0);
+#pragma unroll
+      for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * ds, g, key0);
+    }
   }
-  setup_wait<1>();
 
   const int L_eff = DEVLEN ? spx_prefix_len(a) : p.L;
   const int tph_eff = DEVLEN ? (L_eff + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS : p.TPH;
@@ -110,7 +317,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       const uint32_t kfull0 = smem_u32(&ctl->k_full[0]), vfull0 = smem_u32(&ctl->v_full[0]);
       unsigned char* kring = base + geo.k_off;
       unsigned char* vring = base + geo.v_off;
-      int kst = 0, vst = 0, n_done = 0;
+      int kst = 0, vst = 0;
       uint32_t kph = 1, vph = 1, n_rag = 0;
       while (ok && work.next()) {
         const int g = work.prob / p.n_rblk;
@@ -118,11 +325,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
           const int tile = work.tile(j);
           const bool is_tree = tile == p.TPH;
           const int key0 = is_tree ? 0 : tile * SPX_TILE_KEYS;
-          // Start-up: only two tiles are requested until the first S MMA has consumed K tile 0.  A full ring requested
-          // at once by every SM sits in the memory system's queues in no particular order, and tile 0 would arrive
-          // last as often as first.
-          if (n_done == 2) ok = wait_c(&ctl->k_empty[0], 0, abort_flag);
-          if (ok) ok = wait_c(&ctl->k_empty[kst], kph, abort_flag);
+          ok = wait_c(&ctl->k_empty[kst], kph, abort_flag);
           if (!ok) break;
           {
             const uint32_t bar = kfull0 + kst * 8, dst = smem_u32(kring + kst * G::kKStage);
@@ -176,7 +379,6 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
             vst = 0;
             vph ^= 1;
           }
-          ++n_done;
         }
       }
     }
@@ -238,6 +440,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     const int rr = rc.row_t;                             // row inside the row block
     uint32_t t0 = 0, seg = 0;                            // tiles and segments before the current segment
     bool anc_seen = false;
+    float m_loc, l;                                      // l is relative to m_loc
     while (ok && work.next_any()) {
       const int prob = work.prob, g = prob / p.n_rblk, rblk = prob - g * p.n_rblk, n = work.n;
       const int r = rblk * p.RB + rr;
@@ -248,7 +451,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       // this warpgroup's half of the output columns, in groups of 16
       constexpr int kGroups = D / 16 / kWG;
       const int c_lo = rc.w * kGroups;
-      if (DEVLEN && n == 0) {
+      if (!FUSED && DEVLEN && n == 0) {
         // No tile of this run exists at the device-side length: its slot gets the neutral partial (weight zero in
         // the merge), and no barrier of the pipeline is touched.
         if (valid) {
@@ -263,7 +466,8 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
         continue;
       }
       const int t_node = valid ? r / p.G : 0;
-      float m_loc = -INFINITY, l = 0.f;                  // l is relative to m_loc
+      m_loc = -INFINITY;
+      l = 0.f;
       for (int j = (rc.w ^ t0) & 1; j < n && ok; j += kWG) {
         if (!warp_valid) {
           ok = skip_tile(rc, t0 + j);
@@ -325,6 +529,8 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       }
       if (!ok) break;
 
+      if (FUSED) break;                                  // (its end is below: a worker of a cluster has one segment)
+
       // ---- end of the segment: unnormalised O, reference maximum and row sum to the partial slot ----
       float m_fin, l_tot;
       ok = segment_end(rc, t0 + n - 1, seg, m_loc, l, m_fin, l_tot);
@@ -352,42 +558,83 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       t0 += n;
       ++seg;
     }
+    if constexpr (FUSED) ok = merge_in_cluster<D>(a, rc, base, work, ok, m_loc, l);
+  }
+  if constexpr (FUSED) {
+    if (warp >= kProducerWarp) {                         // the two meetings of merge_in_cluster
+      __syncwarp();
+      cluster_sync();
+      cluster_sync();
+    }
   }
 
   if (!ok && lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
   finish<1>(ctl, warp);
 }
 
-template <int D, int SCORE, bool DEVLEN>
+template <int D, int SCORE, bool DEVLEN, bool FUSED>
 cudaError_t launch(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   static SpxOncePerDevice once;
   constexpr int smem = smem_bytes<1, D>();
-  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN>, smem, &once);
+  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN, FUSED>, smem, &once);
   if (ec != cudaSuccess) return ec;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.plan.n_cta);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = a.plan.cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, verify_kernel<D, SCORE, DEVLEN>, a, maps);
+  cfg.numAttrs = FUSED ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, verify_kernel<D, SCORE, DEVLEN, FUSED>, a, maps);
 }
 
-template <int D>
+template <int D, bool FUSED>
 cudaError_t launch_class(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   const AttnPlan& p = a.plan;
-  if (a.L_dev) return launch<D, 0, true>(a, maps, st);       // never with chunk sums
-  if (!p.want_score) return launch<D, 0, false>(a, maps, st);
-  return p.C == 32 ? launch<D, 1, false>(a, maps, st)
-         : p.C > 32 ? launch<D, 2, false>(a, maps, st)
-                    : launch<D, 3, false>(a, maps, st);
+  if (a.L_dev) return launch<D, 0, true, FUSED>(a, maps, st);       // never with chunk sums
+  if (!p.want_score) return launch<D, 0, false, FUSED>(a, maps, st);
+  return p.C == 32 ? launch<D, 1, false, FUSED>(a, maps, st)
+         : p.C > 32 ? launch<D, 2, false, FUSED>(a, maps, st)
+                    : launch<D, 3, false, FUSED>(a, maps, st);
 }
 
 }  // namespace
+
+// How many clusters of `size` CTAs of this kernel device `dev` (the current one) holds at once, looked up once per device
+// and size; 0 when there is no device.
+int spx_verify_max_clusters(int dev, int size) {
+  static std::atomic<int> known[kSpxMaxDevices][kMaxCluster + 1];
+  if (dev < 0 || dev >= kSpxMaxDevices || size < 1 || size > kMaxCluster) return 0;
+  int n = known[dev][size].load();
+  if (n > 0) return n - 1;
+  auto* kernel = verify_kernel<128, 0, false, true>;
+  static SpxOncePerDevice once;
+  constexpr int smem = smem_bytes<1, 128>();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(size);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = size;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (spx_opt_in_smem(kernel, smem, &once) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  known[dev][size].store(n + 1);
+  return n;
+}
 
 // Row blocks of 128 (plan.RB); plan.n_cta counts CTAs.
 cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launches) {
@@ -404,7 +651,9 @@ cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launche
   }
   ok = ok && spx_encode_map(&maps.q, a.Q, p.D, p.Hq, a.q_sh, p.T, a.q_st, p.G, p.q_rows / p.G);
   if (!ok) return cudaErrorInvalidValue;
-  const cudaError_t e = p.D == 128 ? launch_class<128>(a, maps, st) : launch_class<64>(a, maps, st);
+  const cudaError_t e = p.cluster > 0
+                            ? (p.D == 128 ? launch_class<128, true>(a, maps, st) : launch_class<64, true>(a, maps, st))
+                            : (p.D == 128 ? launch_class<128, false>(a, maps, st) : launch_class<64, false>(a, maps, st));
   *n_launches += 1;
   return e;
 }

@@ -19,6 +19,10 @@ pytestmark = pytest.mark.gpu
     (4, 1, 64, 128, 131),      # head_dim 64: four row blocks
     (256, 256, 128, 3, 40),    # more problems than CTAs: several segments per worker, each of one tile or two
     (160, 160, 64, 5, 515),    # the same with head_dim 64 and segments of an odd and an even number of tiles
+    # clusters that merge among themselves: 2 to 8 CTAs, rows dealt (up to 32) and columns dealt (more), uneven deals
+    (2, 2, 128, 1, 100), (32, 8, 128, 1, 500), (32, 8, 128, 8, 700), (32, 8, 128, 9, 700), (8, 8, 128, 7, 900),
+    (12, 12, 64, 32, 900), (12, 12, 64, 33, 4096), (32, 32, 128, 100, 300), (32, 8, 128, 60, 130), (32, 8, 128, 60, 2048),
+    (64, 8, 128, 60, 1000), (32, 8, 128, 127, 513),
 ])
 def test_one_cta_row_blocks(cuda_device, Hq, Hkv, D, T, L):
     w = synth.Workload("rows", Hq, Hkv, D, L, T, 32, 4, "uniform", "needle", seed=Hq + T + L)
