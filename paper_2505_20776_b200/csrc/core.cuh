@@ -76,8 +76,8 @@ struct Ctrl {
   uint64_t pv_done[kWG];           // each CTA: the PV is complete
   uint64_t m_pub[kWG];             // this CTA: 4 arrivals, reference maxima of the tile are published
   uint64_t o_done;                 // each CTA: the last PV of a segment is complete
-  uint64_t o_free;                 // leader: every softmax warp has read O of a segment
-  uint64_t epi;                    // this CTA: 8 arrivals, the row sums of a segment are published
+  uint64_t o_free;                 // leader: the softmax warps have read O of a segment
+  uint64_t epi[2];                 // this CTA: the row sums of a segment are published (alternating by segment)
   uint64_t drain;
   uint64_t anc_ready;              // this CTA: the ancestor masks are in shared memory
   uint64_t v_rag;                  // this CTA: a V part whose tail rows must be cleared has landed (device-side length)
@@ -134,8 +134,10 @@ __device__ __forceinline__ void tma_load_hint(uint32_t dst, const CUtensorMap* m
 // ---- set-up and end of a CTA ---------------------------------------------------------------------------
 // Barriers by the producer warp, tensor memory by the MMA warp, and the cluster barrier (block barrier) that publishes
 // them.  None of it touches global memory: it runs ahead of the dependency wait, under the kernel before.
-template <int PAIR>
+// HANDOVER: segments end with segment_handover (else segment_end).
+template <int PAIR, bool HANDOVER = false>
 __device__ __forceinline__ void setup(Ctrl* ctl, int warp, int lane) {
+  constexpr int kEnd = HANDOVER ? 4 : 4 * kWG;    // warps of a CTA that take part in the end of a segment
   if (warp == kProducerWarp) {
     if (lane < kMaxStages) {
       mbar_init(&ctl->k_full[lane], PAIR);
@@ -153,8 +155,9 @@ __device__ __forceinline__ void setup(Ctrl* ctl, int warp, int lane) {
       mbar_init(&ctl->q_full, PAIR);
       mbar_init(&ctl->q_empty, 1);
       mbar_init(&ctl->o_done, 1);
-      mbar_init(&ctl->o_free, 4 * kWG * PAIR);
-      mbar_init(&ctl->epi, 4 * kWG);
+      mbar_init(&ctl->o_free, kEnd * PAIR);
+      mbar_init(&ctl->epi[0], kEnd);
+      mbar_init(&ctl->epi[1], kEnd);
       mbar_init(&ctl->drain, 2);
       mbar_init(&ctl->anc_ready, 1);
       mbar_init(&ctl->v_rag, 1);
@@ -455,11 +458,36 @@ __device__ __forceinline__ bool segment_end(const RowCtx& rc, uint32_t last, uin
   if (m_loc != m_fin) l *= (m_loc == -INFINITY) ? 0.f : ex2_approx(m_loc - m_fin);
   float (*lx)[128] = ctl->l_x[n_seg & 1];
   lx[rc.w][rc.row_t] = l;
-  warp_arrive(&ctl->epi, rc.lane);
+  warp_arrive(&ctl->epi[n_seg & 1], rc.lane);
   if (!wait_c(&ctl->o_done, n_seg & 1, rc.abort_flag)) return false;
   tc_fence_after();
-  if (!mbar_wait(&ctl->epi, n_seg & 1, rc.abort_flag)) return false;
+  if (!mbar_wait(&ctl->epi[n_seg & 1], (n_seg >> 1) & 1, rc.abort_flag)) return false;
   l_tot = lx[0][rc.row_t] + lx[1][rc.row_t];
+  return true;
+}
+
+// End of a segment where the next one follows at once: the warpgroup of the last tile ends the segment alone (`last_wg`;
+// its m_loc is the final reference maximum), the other one leaves its row sums behind and goes on to the next segment,
+// whose first tile is its own.  When both waited for the PV and read half of O each, every segment cost ~5 K cycles on top
+// of its tiles.  l_x and epi alternate by segment: the other warpgroup reaches the segment after next only once the PVs of
+// the next one run, for which this one has handed O over.
+__device__ __forceinline__ bool segment_handover(const RowCtx& rc, uint32_t last, uint32_t n_seg, bool last_wg, float m_loc,
+                                                 float l, float& l_tot) {
+  Ctrl* ctl = rc.ctl;
+  float (*lx)[128] = ctl->l_x[n_seg & 1];
+  uint64_t* epi = &ctl->epi[n_seg & 1];
+  if (!last_wg) {
+    if (!mbar_wait(&ctl->m_pub[last % kWG], (last / kWG) & 1, rc.abort_flag)) return false;
+    lx[0][rc.row_t] = l;
+    lx[1][rc.row_t] = m_loc;
+    warp_arrive(epi, rc.lane);
+    return true;
+  }
+  if (!mbar_wait(epi, (n_seg >> 1) & 1, rc.abort_flag)) return false;
+  const float m_o = lx[1][rc.row_t];
+  l_tot = l + (m_o == -INFINITY ? 0.f : lx[0][rc.row_t] * ex2_approx(m_o - m_loc));
+  if (!wait_c(&ctl->o_done, n_seg & 1, rc.abort_flag)) return false;
+  tc_fence_after();
   return true;
 }
 

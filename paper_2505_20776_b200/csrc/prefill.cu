@@ -10,9 +10,11 @@
 // next problem are fetched and computed under the last tiles of the one before.
 //
 // What bounds it: the tensor pipe's 1.0 K cycles a tile, the special-function unit's 1.0 K and the power cap together.
-// us per call, replayed, against the same loop with one P buffer, Q in tensor memory by plain loads and a stop between
-// problems (32 query / 8 KV heads): 256 tokens 12.3 -> 10.3, 2K 52.8 -> 43.0, 4K 135 -> 117, 16K 1640 -> 1589 (1383
-// TFLOP/s), under the power cap 1825 -> 1720; 32 heads of their own, 8K: 489 -> 464.
+// Between problems the warpgroup of the last tile writes O and the other one is already in the next problem (core.cuh,
+// segment_handover).  us per call, replayed, against the same loop with one P buffer, Q in tensor memory by plain loads and a
+// stop between problems / with both warpgroups ending a problem (32 query / 8 KV heads): 1K tokens 22.6 / 20.5 -> 18.4,
+// 2K 52.5 / 45.0 -> 40.6, 4K 135 / 121 -> 115, 16K 1655 / 1628 -> 1600 (1374 TFLOP/s; under the power cap 1825 -> 1720
+// before the last step).  Prefetching the tensor maps at the start costs 0.4 us at 2K.
 #include "common.cuh"
 #include "core.cuh"
 #include "tmap.h"
@@ -73,12 +75,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const G geo(128);
 
-  if (warp == kProducerWarp && lane == 0) {
-    prefetch_tensormap(&maps.q);
-    prefetch_tensormap(&maps.k);
-    prefetch_tensormap(&maps.v);
-  }
-  setup<2>(ctl, warp, lane);
+  setup<2, true>(ctl, warp, lane);
   const uint32_t rank = cluster_rank();
   PrefillWork work(a, blockIdx.x >> 1);
   pdl_launch_dependents();
@@ -179,31 +176,36 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
       if (!ok) break;
 
       // ---- end of the problem: the result is final ----
-      float m_fin, l_tot;
-      ok = segment_end(rc, t0 + n - 1, seg, m_loc, l, m_fin, l_tot);
+      const bool last_wg = ((t0 + n - 1) & 1) == (uint32_t)rc.w;
+      float l_tot = 1.f;
+      ok = segment_handover(rc, t0 + n - 1, seg, last_wg, m_loc, l, l_tot);
       if (!ok) break;
-      const float inv = 1.f / l_tot;
-      __nv_bfloat16* out = a.O + (long long)tok * a.o_st + (long long)head * a.o_sh + rc.w * (D / kWG);
+      if (last_wg) {
+        const float inv = 1.f / l_tot;
+        __nv_bfloat16* out = a.O + (long long)tok * a.o_st + (long long)head * a.o_sh;
 #pragma unroll
-      for (int c = 0; c < D / kWG / 32; ++c) {           // this warpgroup's half of the columns
-        uint32_t v[32];
-        tmem_ld32(rc.lane_tmem + kColO + rc.w * (D / kWG) + c * 32, v);
-        tmem_wait_ld();
-        if (valid) {
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t v[32];
+          tmem_ld32(rc.lane_tmem + kColO + c * 32, v);
+          tmem_wait_ld();
+          if (c == D / 32 - 1) {
+            tc_fence_before();
+            warp_arrive_cluster(o_free_l, lane);         // O may be overwritten
+          }
+          if (valid) {
 #pragma unroll
-          for (int q8 = 0; q8 < 4; ++q8) {
-            uint4 x;
-            x.x = pack_bf16x2(__uint_as_float(v[q8 * 8]) * inv, __uint_as_float(v[q8 * 8 + 1]) * inv);
-            x.y = pack_bf16x2(__uint_as_float(v[q8 * 8 + 2]) * inv, __uint_as_float(v[q8 * 8 + 3]) * inv);
-            x.z = pack_bf16x2(__uint_as_float(v[q8 * 8 + 4]) * inv, __uint_as_float(v[q8 * 8 + 5]) * inv);
-            x.w = pack_bf16x2(__uint_as_float(v[q8 * 8 + 6]) * inv, __uint_as_float(v[q8 * 8 + 7]) * inv);
-            *reinterpret_cast<uint4*>(out + c * 32 + q8 * 8) = x;
+            for (int q8 = 0; q8 < 4; ++q8) {
+              uint4 x;
+              x.x = pack_bf16x2(__uint_as_float(v[q8 * 8]) * inv, __uint_as_float(v[q8 * 8 + 1]) * inv);
+              x.y = pack_bf16x2(__uint_as_float(v[q8 * 8 + 2]) * inv, __uint_as_float(v[q8 * 8 + 3]) * inv);
+              x.z = pack_bf16x2(__uint_as_float(v[q8 * 8 + 4]) * inv, __uint_as_float(v[q8 * 8 + 5]) * inv);
+              x.w = pack_bf16x2(__uint_as_float(v[q8 * 8 + 6]) * inv, __uint_as_float(v[q8 * 8 + 7]) * inv);
+              *reinterpret_cast<uint4*>(out + c * 32 + q8 * 8) = x;
+            }
           }
         }
+        if (valid) a.lse[(long long)head * a.L + tok] = (m_loc + log2f(l_tot)) * kLn2;
       }
-      if (rc.w == 0 && valid) a.lse[(long long)head * a.L + tok] = (m_fin + log2f(l_tot)) * kLn2;
-      tc_fence_before();
-      warp_arrive_cluster(o_free_l, lane);
       t0 += n;
       ++seg;
     }
