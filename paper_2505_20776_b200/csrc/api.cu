@@ -114,7 +114,7 @@ int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
     p.max_segs = (p.UPP + p.q - 1) / p.q + 1;
   }
   if (p.max_segs > p.n_cta) p.max_segs = p.n_cta;
-  p.n_slots = p.cluster > 0 ? 1 : p.n_cta + p.NP - 1;           // (a cluster merges in shared memory)
+  p.n_slots = p.cluster > 0 ? p.n_cta : p.n_cta + p.NP - 1;
   long long off = 0;
   p.off_part_o = off; off += (long long)p.n_slots * p.D * p.RB;
   p.off_part_m = off; off += (long long)p.n_slots * p.RB;
@@ -149,13 +149,14 @@ int cluster_size(const AttnPlan& p, bool pair) {
   } else {
     split = (int)((np * p.UPP + sm_count() - 1) / sm_count());
   }
-  // What merging in the cluster saves (4 us with the second launch) against the tiles it adds; the pairs, whose CTAs fetch
-  // half of every K/V tile, win again when the tiles are many.  us per call, split / cluster (32 query / 8 KV heads unless said):
-  //   60 nodes: 1K 10.9 / 10.6, 2K 11.6 / 11.5 (3 tiles against 2), 4K 13.4 / 14.4 (5 against 4)
-  //   60 nodes, 64 query heads: 1K 13.4 / 11.4, 4K 18.3 / 16.8 (9 against 9), 16K 36.6 / 38.4 (33 against 33)
-  //   60 nodes, 32 KV heads: 1K 13.5 / 10.9, 8K 31.6 / 29.3 (17 against 15), 32K 91.3 / 88.9 (65 against 56)
-  //   1 node: 2K 10.8 / 8.5, 8K 15.8 / 14.8 (9 against 4), 16K 20.4 / 22.5 (17 against 7)
-  //   12 x 64 heads: 4K 11.7 / 9.7 (5 against 3);  60 nodes, 32 x 64 query / 8 KV heads, 16K: 24.0 / 24.5 (19 against 14)
+  // What merging in the cluster saves (3 to 4 us with the second launch) against the tiles it adds; the pairs, whose CTAs
+  // fetch half of every K/V tile, win again when the tiles are many.  us per call, split / cluster, replayed (32 query / 8 KV
+  // heads unless said; launched one by one the cluster form gains another 0.5):
+  //   60 nodes: 1K 10.9 / 9.9, 2K 11.6 / 10.7 (3 tiles against 2), 3K 12.5 / 13.1 (4 against 3), 4K 13.4 / 13.6 (5 against 4)
+  //   60 nodes, 64 query heads: 1K 13.4 / 11.5, 4K 16.2 / 16.8 (9 against 9; one by one 17.5 / 17.2), 16K 34.3 / 38.0 (33)
+  //   60 nodes, 32 KV heads: 1K 13.5 / 10.7, 8K 29.5 / 26.6 (17 against 15), 32K 91.3 / 88.9 (65 against 56)
+  //   1 node: 2K 10.8 / 8.0, 8K 15.8 / 14.8 (9 against 4), 16K 19.3 / 22.5 (17 against 7)
+  //   12 x 64 heads: 4K 11.7 / 9.3 (5 against 3);  60 nodes, 32 x 64 query / 8 KV heads, 16K: 22.7 / 24.5 (19 against 14)
   const int most = pair ? (tiles <= 16 ? (split > 3 ? split : 3) : 0)
                         : split + (p.D == 64 ? 3 : split > 30 ? split / 6 : 5);
   if (tiles > most) return 0;

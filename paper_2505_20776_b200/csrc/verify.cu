@@ -13,8 +13,8 @@
 //   32 query / 8 KV heads, one node, 16K prefix   27.9 -> 19.3   128K 113.8 -> 87.5 = 6.1 TB/s
 //   12 heads x 64, 8 nodes, 4K prefix             15.6 -> 9.6
 //
-// FUSED: the workers of a problem form one cluster and merge their results through each other's shared memory, so that the
-// call is one kernel: no partials in memory, no second launch waiting for the slowest block of the first.
+// MERGE != 0: the workers of a problem form one cluster and merge their results among themselves (1 through shared memory,
+// 2 through L2), so that the call is one kernel: no second launch waiting for the slowest block of the first.
 //
 // Warps: 0-7 softmax (two warpgroups), 8 TMA producer of K and V, 9 issuer of the S MMAs, 10 of the PV MMAs, 11 ancestor
 // masks of the tree and TMA producer of Q.  Every wait is bounded; an expired wait raises SPECEXT_ERR_TIMEOUT, and all
@@ -68,22 +68,25 @@ struct VerifyWork {
 };
 
 // End of a worker that is one of the CTAs of a cluster: every CTA has an unnormalised O, a reference maximum and a row sum
-// for the same rows.  Each CTA sends every part of its O to the CTA that owns it, and the owner adds the parts up and writes
-// O.  What is received lies where Q and the rings were, so the CTAs meet once before sending and once after.
+// for the same rows.  Each CTA passes its part on, the cluster meets, and each CTA adds up and writes its share of O.  How
+// depends on the number of rows of the call.
 //
-// Who owns what depends on the number of rows.  More than 32: the columns are dealt in units of 8 (unit u to CTA u mod
-// size), so that a store of a warp is 512 contiguous bytes of one CTA.  Up to 32: the rows are dealt in equal runs, which
-// needs fewer instructions, addresses and (m, l) copies, but each store of a warp goes to 32 places.  us per call, by
-// columns / by rows: 4 rows on a 2K cache 9.2 / 8.7, 12 x 64 heads with 8 rows 7.7 / 7.2, 40 rows 8.2 / 8.2, 60 rows at 1K
-// 10.9 / 11.5, 120 rows at 8K 17.2 / 18.3.  (Bulk copies between the CTAs instead of stores: 9.2, 7.7, 8.1, 11.6, 17.7.)
+// Up to 32: through the other CTAs' shared memory (where Q and the rings were, so the CTAs meet before as well), the rows
+// dealt in equal runs.  More: through the workspace, that is through L2, the columns dealt in units of 8.  Shared memory of
+// another CTA takes stores at ~20 GB/s, 64 KB of 128 rows in 3 us, and shared-memory room needs the second meeting; L2
+// costs two of its latencies.  us per call, by shared memory / by L2: 4 rows on 2K 8.0 / 8.5, 12 x 64 heads with 8 rows
+// 7.4 / 7.6, 10 rows of 32 KV heads 10.2 / 10.1, 40 rows 8.3 / 7.6, 120 rows at 8K 17.2 / 15.9, 240 rows at 1K 10.6 / 9.7.
+// (Bulk copies between the CTAs instead of stores were slower than either: 8.8, 7.7, 10.5, 8.1, 17.7, 11.2.)  Each is an
+// instantiation of its own: with both in one kernel a call was 0.1 to 0.3 us longer.
 struct MergeCtx {
   int cs, rank;            // CTAs of the cluster, this one
-  int g, rblk, n_rows;     // the problem and its rows
-  int log_g;
+  int prob, g, rblk;       // the problem
+  int n_rows, log_g;
   float m, l;              // of this thread's row in this CTA
   bool any;                // this CTA had a key tile (else: zeros of weight zero)
 };
 constexpr int kMaxCluster = 8;
+constexpr int kRowsBySmem = 32;
 constexpr float kLn2 = 0.693147180559945309417f;
 
 // This thread's half row of O.
@@ -101,8 +104,9 @@ __device__ __forceinline__ void own_half_row(const RowCtx& rc, bool any, uint32_
 }
 
 template <int D>
-__device__ __forceinline__ void merge_by_rows(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const MergeCtx& mc,
+__device__ __forceinline__ void merge_by_smem(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const MergeCtx& mc,
                                               bool ok) {
+  cluster_sync();                                                  // the rings are free everywhere
   constexpr int kCols = D / 4;                                     // 16-byte columns of a row
   const AttnPlan& p = a.plan;
   const int cs = mc.cs, run = (mc.n_rows + cs - 1) / cs;           // rows of a CTA
@@ -161,93 +165,101 @@ __device__ __forceinline__ void merge_by_rows(const AttnArgs& a, const RowCtx& r
 }
 
 template <int D>
-__device__ __forceinline__ void merge_by_columns(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const MergeCtx& mc,
-                                                 bool ok) {
+__device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc, const MergeCtx& mc, bool ok) {
   constexpr int kUnits = D / 8;
   const AttnPlan& p = a.plan;
   const int cs = mc.cs;
-  int slot = rc.w * (kUnits / 2) / cs, owner = rc.w * (kUnits / 2) - slot * cs;      // of this warpgroup's first unit
-  float4* part = reinterpret_cast<float4*>(base);                                    // [slot][source CTA][2][128 rows]
-  float2* ml = reinterpret_cast<float2*>(part + (kUnits + cs - 1) / cs * cs * 256);  // [source CTA][128 rows]
+  // [CTA][D / 4][128 rows] of float4 and [CTA][128 rows] of (m, l)
+  float4* part = reinterpret_cast<float4*>(a.ws + p.off_part_o) + (long long)mc.prob * cs * (D / 4) * 128;
+  float2* ml = reinterpret_cast<float2*>(a.ws + p.off_part_m) + mc.prob * cs * 128;
   if (ok && rc.row_t - rc.lane < mc.n_rows) {
     uint32_t v[D / 64][32];
     own_half_row<D>(rc, mc.any, v);
-    const uint32_t mine = smem_u32(part) + mc.rank * 4096 + rc.row_t * 16;
-    if (rc.w == 0)
-      for (int c = 0; c < cs; ++c)
-        st_cluster_v2(map_to_cta(smem_u32(ml + mc.rank * 128 + rc.row_t), c), mc.m, mc.l);
+    if (rc.row_t < mc.n_rows) {
+      uint4* dst = reinterpret_cast<uint4*>(part) + (mc.rank * (D / 4) + rc.w * (D / 8)) * 128 + rc.row_t;
 #pragma unroll
-    for (int u = 0; u < kUnits / 2; ++u) {
-      const uint32_t dst = map_to_cta(mine + slot * cs * 4096, owner);
-      if (++owner == cs) {
-        owner = 0;
-        ++slot;
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int k = u * 8 + q * 4;
-        st_cluster_v4(dst + q * 2048, v[k / 32][k % 32], v[k / 32][k % 32 + 1], v[k / 32][k % 32 + 2], v[k / 32][k % 32 + 3]);
-      }
+      for (int q = 0; q < D / 8; ++q)
+        __stcg(dst + q * 128,
+               make_uint4(v[q / 8][q % 8 * 4], v[q / 8][q % 8 * 4 + 1], v[q / 8][q % 8 * 4 + 2], v[q / 8][q % 8 * 4 + 3]));
+      if (rc.w == 0) __stcg(ml + mc.rank * 128 + rc.row_t, make_float2(mc.m, mc.l));
     }
   }
   __syncwarp();
   cluster_sync();
   if (!ok) return;
-  // 8 warps over (slot, group of 32 rows)
   const int groups = (mc.n_rows + 31) / 32;
-  int group = rc.w * 4 + rc.row_t / 32;
-  slot = 0;
-  for (;;) {
+  // 8 warps over (unit, group of 32 rows), two at a time so that their loads are in flight together
+  struct Task {
+    int u, row;
+    float2 s[kMaxCluster];
+    float4 x[kMaxCluster], y[kMaxCluster];
+  };
+  int group = rc.w * 4 + rc.row_t / 32, u = mc.rank;
+  auto load = [&](Task& t) {
     while (group >= groups) {
       group -= groups;
-      ++slot;
+      u += cs;
     }
-    const int u = slot * cs + mc.rank;
-    if (u >= kUnits) break;
-    const int row = group * 32 + rc.lane;
-    const float4* src = part + slot * cs * 256 + row;
-    float w[kMaxCluster], M = -INFINITY, Z = 0.f;
+    t.u = u;
+    t.row = group * 32 + rc.lane;
+    group += 8;
+    if (t.u >= kUnits) return;
+    const float4* src = part + t.u * 256 + t.row;
 #pragma unroll
     for (int c = 0; c < kMaxCluster; ++c) {
-      w[c] = c < cs ? ml[c * 128 + row].x : -INFINITY;
-      M = fmaxf(M, w[c]);
+      if (c < cs) {
+        t.s[c] = __ldcg(ml + c * 128 + t.row);
+        t.x[c] = __ldcg(src + c * (D / 4) * 128);
+        t.y[c] = __ldcg(src + c * (D / 4) * 128 + 128);
+      }
     }
+  };
+  auto finish = [&](const Task& t) {
+    if (t.u >= kUnits || t.row >= mc.n_rows) return;
+    float M = -INFINITY, Z = 0.f;
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c)
+      if (c < cs) M = fmaxf(M, t.s[c].x);
     float4 acc0 = make_float4(0.f, 0.f, 0.f, 0.f), acc1 = acc0;
 #pragma unroll
     for (int c = 0; c < kMaxCluster; ++c) {
       if (c < cs) {
-        const float f = ex2_approx(w[c] - M);
-        const float4 x = src[c * 256], y = src[c * 256 + 128];
-        Z = fmaf(ml[c * 128 + row].y, f, Z);
-        acc0.x = fmaf(f, x.x, acc0.x);
-        acc0.y = fmaf(f, x.y, acc0.y);
-        acc0.z = fmaf(f, x.z, acc0.z);
-        acc0.w = fmaf(f, x.w, acc0.w);
-        acc1.x = fmaf(f, y.x, acc1.x);
-        acc1.y = fmaf(f, y.y, acc1.y);
-        acc1.z = fmaf(f, y.z, acc1.z);
-        acc1.w = fmaf(f, y.w, acc1.w);
+        const float f = ex2_approx(t.s[c].x - M);
+        Z = fmaf(t.s[c].y, f, Z);
+        acc0.x = fmaf(f, t.x[c].x, acc0.x);
+        acc0.y = fmaf(f, t.x[c].y, acc0.y);
+        acc0.z = fmaf(f, t.x[c].z, acc0.z);
+        acc0.w = fmaf(f, t.x[c].w, acc0.w);
+        acc1.x = fmaf(f, t.y[c].x, acc1.x);
+        acc1.y = fmaf(f, t.y[c].y, acc1.y);
+        acc1.z = fmaf(f, t.y[c].z, acc1.z);
+        acc1.w = fmaf(f, t.y[c].w, acc1.w);
       }
     }
-    if (row < mc.n_rows) {
-      const float inv = 1.f / Z;
-      const int r = mc.rblk * 128 + row, t = r >> mc.log_g, h = mc.g * p.G + (r & (p.G - 1));
-      *reinterpret_cast<uint4*>(a.O + (long long)t * a.o_st + (long long)h * a.o_sh + u * 8) =
-          make_uint4(pack_bf16x2(acc0.x * inv, acc0.y * inv), pack_bf16x2(acc0.z * inv, acc0.w * inv),
-                     pack_bf16x2(acc1.x * inv, acc1.y * inv), pack_bf16x2(acc1.z * inv, acc1.w * inv));
-      if (u == 0) a.lse[(long long)h * p.T + t] = (M + log2f(Z)) * kLn2;
-    }
-    group += 8;
-  }
+    const float inv = 1.f / Z;
+    const int r = mc.rblk * 128 + t.row, node = r >> mc.log_g, h = mc.g * p.G + (r & (p.G - 1));
+    *reinterpret_cast<uint4*>(a.O + (long long)node * a.o_st + (long long)h * a.o_sh + t.u * 8) =
+        make_uint4(pack_bf16x2(acc0.x * inv, acc0.y * inv), pack_bf16x2(acc0.z * inv, acc0.w * inv),
+                   pack_bf16x2(acc1.x * inv, acc1.y * inv), pack_bf16x2(acc1.z * inv, acc1.w * inv));
+    if (t.u == 0) a.lse[(long long)h * p.T + node] = (M + log2f(Z)) * kLn2;
+  };
+  Task t0, t1;
+  do {
+    load(t0);
+    load(t1);
+    finish(t0);
+    finish(t1);
+  } while (t1.u < kUnits);
 }
 
-template <int D, class Work>
+template <int D, int MERGE, class Work>
 __device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const Work& work,
                                                  bool ok, float m_loc, float l) {
   const AttnPlan& p = a.plan;
   MergeCtx mc;
   mc.cs = p.cluster;
   mc.rank = (int)cluster_rank();
+  mc.prob = work.prob;
   mc.g = work.prob / p.n_rblk;
   mc.rblk = work.prob - mc.g * p.n_rblk;
   mc.n_rows = min(128, p.rows - mc.rblk * 128);
@@ -257,10 +269,8 @@ __device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx
   mc.l = 0.f;
   if (ok && mc.any) ok = segment_end(rc, work.n - 1, 0, m_loc, l, mc.m, mc.l);
   __syncwarp();
-  cluster_sync();
-  // (by the rows of the whole call: the CTAs of all problems take the same path)
-  if (p.rows <= 32) merge_by_rows<D>(a, rc, base, mc, ok);
-  else merge_by_columns<D>(a, rc, base, mc, ok);
+  if constexpr (MERGE == 1) merge_by_smem<D>(a, rc, base, mc, ok);
+  else merge_by_l2<D>(a, rc, mc, ok);
   return ok;
 }
 
@@ -268,7 +278,7 @@ __device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx
 // 1 chunks of 32 keys, 2 chunks of 64 or 128 keys, 3 chunks of fewer than 32 keys.
 // DEVLEN: the prefix length is read from device memory (a.L_dev) and may be shorter than the planned capacity p.L; the
 // instantiation without it carries none of that code.
-template <int D, int SCORE, bool DEVLEN, bool FUSED>
+template <int D, int SCORE, bool DEVLEN, int MERGE>
 __global__ void __launch_bounds__(kThreads, 1)
 verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ VerifyMaps maps) {
   using G = Geo<1, D>;
@@ -451,7 +461,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       // this warpgroup's half of the output columns, in groups of 16
       constexpr int kGroups = D / 16 / kWG;
       const int c_lo = rc.w * kGroups;
-      if (!FUSED && DEVLEN && n == 0) {
+      if (MERGE == 0 && DEVLEN && n == 0) {
         // No tile of this run exists at the device-side length: its slot gets the neutral partial (weight zero in
         // the merge), and no barrier of the pipeline is touched.
         if (valid) {
@@ -529,7 +539,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       }
       if (!ok) break;
 
-      if (FUSED) break;                                  // (its end is below: a worker of a cluster has one segment)
+      if (MERGE != 0) break;                                  // (its end is below: a worker of a cluster has one segment)
 
       // ---- end of the segment: unnormalised O, reference maximum and row sum to the partial slot ----
       float m_fin, l_tot;
@@ -558,12 +568,12 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       t0 += n;
       ++seg;
     }
-    if constexpr (FUSED) ok = merge_in_cluster<D>(a, rc, base, work, ok, m_loc, l);
+    if constexpr (MERGE != 0) ok = merge_in_cluster<D, MERGE>(a, rc, base, work, ok, m_loc, l);
   }
-  if constexpr (FUSED) {
-    if (warp >= kProducerWarp) {                         // the two meetings of merge_in_cluster
+  if constexpr (MERGE != 0) {
+    if (warp >= kProducerWarp) {                         // the meetings of merge_in_cluster
       __syncwarp();
-      cluster_sync();
+      if (MERGE == 1) cluster_sync();
       cluster_sync();
     }
   }
@@ -572,11 +582,11 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
   finish<1>(ctl, warp);
 }
 
-template <int D, int SCORE, bool DEVLEN, bool FUSED>
+template <int D, int SCORE, bool DEVLEN, int MERGE>
 cudaError_t launch(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   static SpxOncePerDevice once;
   constexpr int smem = smem_bytes<1, D>();
-  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN, FUSED>, smem, &once);
+  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN, MERGE>, smem, &once);
   if (ec != cudaSuccess) return ec;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.plan.n_cta);
@@ -591,18 +601,18 @@ cudaError_t launch(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = FUSED ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, verify_kernel<D, SCORE, DEVLEN, FUSED>, a, maps);
+  cfg.numAttrs = MERGE != 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, verify_kernel<D, SCORE, DEVLEN, MERGE>, a, maps);
 }
 
-template <int D, bool FUSED>
+template <int D, int MERGE>
 cudaError_t launch_class(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   const AttnPlan& p = a.plan;
-  if (a.L_dev) return launch<D, 0, true, FUSED>(a, maps, st);       // never with chunk sums
-  if (!p.want_score) return launch<D, 0, false, FUSED>(a, maps, st);
-  return p.C == 32 ? launch<D, 1, false, FUSED>(a, maps, st)
-         : p.C > 32 ? launch<D, 2, false, FUSED>(a, maps, st)
-                    : launch<D, 3, false, FUSED>(a, maps, st);
+  if (a.L_dev) return launch<D, 0, true, MERGE>(a, maps, st);       // never with chunk sums
+  if (!p.want_score) return launch<D, 0, false, MERGE>(a, maps, st);
+  return p.C == 32 ? launch<D, 1, false, MERGE>(a, maps, st)
+         : p.C > 32 ? launch<D, 2, false, MERGE>(a, maps, st)
+                    : launch<D, 3, false, MERGE>(a, maps, st);
 }
 
 }  // namespace
@@ -614,7 +624,7 @@ int spx_verify_max_clusters(int dev, int size) {
   if (dev < 0 || dev >= kSpxMaxDevices || size < 1 || size > kMaxCluster) return 0;
   int n = known[dev][size].load();
   if (n > 0) return n - 1;
-  auto* kernel = verify_kernel<128, 0, false, true>;
+  auto* kernel = verify_kernel<128, 0, false, 2>;
   static SpxOncePerDevice once;
   constexpr int smem = smem_bytes<1, 128>();
   cudaLaunchConfig_t cfg = {};
@@ -651,9 +661,13 @@ cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launche
   }
   ok = ok && spx_encode_map(&maps.q, a.Q, p.D, p.Hq, a.q_sh, p.T, a.q_st, p.G, p.q_rows / p.G);
   if (!ok) return cudaErrorInvalidValue;
-  const cudaError_t e = p.cluster > 0
-                            ? (p.D == 128 ? launch_class<128, true>(a, maps, st) : launch_class<64, true>(a, maps, st))
-                            : (p.D == 128 ? launch_class<128, false>(a, maps, st) : launch_class<64, false>(a, maps, st));
+  cudaError_t e;
+  if (p.cluster == 0)
+    e = p.D == 128 ? launch_class<128, 0>(a, maps, st) : launch_class<64, 0>(a, maps, st);
+  else if (p.rows <= kRowsBySmem)
+    e = p.D == 128 ? launch_class<128, 1>(a, maps, st) : launch_class<64, 1>(a, maps, st);
+  else
+    e = p.D == 128 ? launch_class<128, 2>(a, maps, st) : launch_class<64, 2>(a, maps, st);
   *n_launches += 1;
   return e;
 }
