@@ -81,13 +81,14 @@ struct SpxOncePerDevice {
   unsigned char done[kSpxMaxDevices] = {};
 };
 template <typename Kernel>
-cudaError_t spx_opt_in_smem(Kernel* kernel, int bytes, SpxOncePerDevice* once) {
+cudaError_t spx_opt_in_smem(Kernel* kernel, int bytes, SpxOncePerDevice* once, bool any_cluster_size = false) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const bool cached = dev >= 0 && dev < kSpxMaxDevices;
   if (cached && __atomic_load_n(&once->done[dev], __ATOMIC_ACQUIRE)) return cudaSuccess;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && any_cluster_size) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && cached) __atomic_store_n(&once->done[dev], (unsigned char)1, __ATOMIC_RELEASE);
   return e;
 }
@@ -98,6 +99,9 @@ cudaError_t spx_launch_attn_simt(const AttnArgs& a, cudaStream_t st, int* n_laun
 #endif
 cudaError_t spx_launch_attn_tc2(const AttnArgs& a, cudaStream_t st, int* n_launches);
 cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launches);
+// Clusters that merge among themselves: up to this many stacked rows through shared memory (sizes up to 8), above through L2
+// (sizes up to 16).
+constexpr int kSpxClusterRowsBySmem = 32;
 int spx_verify_max_clusters(int dev, int size);
 cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches);
 

@@ -14,7 +14,8 @@
 //   12 heads x 64, 8 nodes, 4K prefix             15.6 -> 9.6
 //
 // MERGE != 0: the workers of a problem form one cluster and merge their results among themselves (1 through shared memory,
-// 2 through L2), so that the call is one kernel: no second launch waiting for the slowest block of the first.
+// 2 through L2, 3 through L2 with more than 8 CTAs), so that the call is one kernel: no second launch waiting for the
+// slowest block of the first.
 //
 // Warps: 0-7 softmax (two warpgroups), 8 TMA producer of K and V, 9 issuer of the S MMAs, 10 of the PV MMAs, 11 ancestor
 // masks of the tree and TMA producer of Q.  Every wait is bounded; an expired wait raises SPECEXT_ERR_TIMEOUT, and all
@@ -85,8 +86,8 @@ struct MergeCtx {
   float m, l;              // of this thread's row in this CTA
   bool any;                // this CTA had a key tile (else: zeros of weight zero)
 };
-constexpr int kMaxCluster = 8;
-constexpr int kRowsBySmem = 32;
+constexpr int kMaxCluster = 16;
+constexpr int kRowsBySmem = kSpxClusterRowsBySmem;
 constexpr float kLn2 = 0.693147180559945309417f;
 
 // This thread's half row of O.
@@ -134,10 +135,10 @@ __device__ __forceinline__ void merge_by_smem(const AttnArgs& a, const RowCtx& r
   const int sub = rc.lane / kCols, col = rc.lane - sub * kCols;
   for (int i = (rc.w * 4 + rc.row_t / 32) * kRowsPerWarp + sub; i < n_mine; i += 8 * kRowsPerWarp) {
     const int row = mc.rank * run + i;
-    float w[kMaxCluster], M = -INFINITY, Z = 0.f;
-    float4 x[kMaxCluster];
+    float w[8], M = -INFINITY, Z = 0.f;
+    float4 x[8];
 #pragma unroll
-    for (int c = 0; c < kMaxCluster; ++c) {
+    for (int c = 0; c < 8; ++c) {
       if (c < cs) {
         w[c] = ml[c * run + i].x;
         x[c] = part[(c * run + i) * kCols + (col ^ (row & (kCols - 1)))];
@@ -146,7 +147,7 @@ __device__ __forceinline__ void merge_by_smem(const AttnArgs& a, const RowCtx& r
     }
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < kMaxCluster; ++c) {
+    for (int c = 0; c < 8; ++c) {
       if (c < cs) {
         const float f = ex2_approx(w[c] - M);
         Z = fmaf(ml[c * run + i].y, f, Z);
@@ -164,7 +165,8 @@ __device__ __forceinline__ void merge_by_smem(const AttnArgs& a, const RowCtx& r
   }
 }
 
-template <int D>
+// MAX: bound on the cluster's size (8 or 16).
+template <int D, int MAX>
 __device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc, const MergeCtx& mc, bool ok) {
   constexpr int kUnits = D / 8;
   const AttnPlan& p = a.plan;
@@ -191,8 +193,8 @@ __device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc,
   // 8 warps over (unit, group of 32 rows), two at a time so that their loads are in flight together
   struct Task {
     int u, row;
-    float2 s[kMaxCluster];
-    float4 x[kMaxCluster], y[kMaxCluster];
+    float2 s[MAX];
+    float4 x[MAX], y[MAX];
   };
   int group = rc.w * 4 + rc.row_t / 32, u = mc.rank;
   auto load = [&](Task& t) {
@@ -206,7 +208,7 @@ __device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc,
     if (t.u >= kUnits) return;
     const float4* src = part + t.u * 256 + t.row;
 #pragma unroll
-    for (int c = 0; c < kMaxCluster; ++c) {
+    for (int c = 0; c < MAX; ++c) {
       if (c < cs) {
         t.s[c] = __ldcg(ml + c * 128 + t.row);
         t.x[c] = __ldcg(src + c * (D / 4) * 128);
@@ -218,11 +220,11 @@ __device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc,
     if (t.u >= kUnits || t.row >= mc.n_rows) return;
     float M = -INFINITY, Z = 0.f;
 #pragma unroll
-    for (int c = 0; c < kMaxCluster; ++c)
+    for (int c = 0; c < MAX; ++c)
       if (c < cs) M = fmaxf(M, t.s[c].x);
     float4 acc0 = make_float4(0.f, 0.f, 0.f, 0.f), acc1 = acc0;
 #pragma unroll
-    for (int c = 0; c < kMaxCluster; ++c) {
+    for (int c = 0; c < MAX; ++c) {
       if (c < cs) {
         const float f = ex2_approx(t.s[c].x - M);
         Z = fmaf(t.s[c].y, f, Z);
@@ -243,13 +245,20 @@ __device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc,
                    pack_bf16x2(acc1.x * inv, acc1.y * inv), pack_bf16x2(acc1.z * inv, acc1.w * inv));
     if (t.u == 0) a.lse[(long long)h * p.T + node] = (M + log2f(Z)) * kLn2;
   };
-  Task t0, t1;
-  do {
+  if constexpr (MAX > 8) {
+    // at least 9 CTAs: at most two units each, a task per warp
+    Task t0;
     load(t0);
-    load(t1);
     finish(t0);
-    finish(t1);
-  } while (t1.u < kUnits);
+  } else {
+    Task t0, t1;
+    do {
+      load(t0);
+      load(t1);
+      finish(t0);
+      finish(t1);
+    } while (t1.u < kUnits);
+  }
 }
 
 template <int D, int MERGE, class Work>
@@ -270,7 +279,7 @@ __device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx
   if (ok && mc.any) ok = segment_end(rc, work.n - 1, 0, m_loc, l, mc.m, mc.l);
   __syncwarp();
   if constexpr (MERGE == 1) merge_by_smem<D>(a, rc, base, mc, ok);
-  else merge_by_l2<D>(a, rc, mc, ok);
+  else merge_by_l2<D, MERGE == 2 ? 8 : 16>(a, rc, mc, ok);
   return ok;
 }
 
@@ -586,7 +595,7 @@ template <int D, int SCORE, bool DEVLEN, int MERGE>
 cudaError_t launch(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   static SpxOncePerDevice once;
   constexpr int smem = smem_bytes<1, D>();
-  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN, MERGE>, smem, &once);
+  const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN, MERGE>, smem, &once, MERGE != 0);
   if (ec != cudaSuccess) return ec;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.plan.n_cta);
@@ -615,6 +624,11 @@ cudaError_t launch_class(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t
                     : launch<D, 3, false, MERGE>(a, maps, st);
 }
 
+template <int MERGE>
+cudaError_t launch_dim(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
+  return a.plan.D == 128 ? launch_class<128, MERGE>(a, maps, st) : launch_class<64, MERGE>(a, maps, st);
+}
+
 }  // namespace
 
 // How many clusters of `size` CTAs of this kernel device `dev` (the current one) holds at once, looked up once per device
@@ -624,7 +638,7 @@ int spx_verify_max_clusters(int dev, int size) {
   if (dev < 0 || dev >= kSpxMaxDevices || size < 1 || size > kMaxCluster) return 0;
   int n = known[dev][size].load();
   if (n > 0) return n - 1;
-  auto* kernel = verify_kernel<128, 0, false, 2>;
+  auto* kernel = verify_kernel<128, 0, false, 3>;
   static SpxOncePerDevice once;
   constexpr int smem = smem_bytes<1, 128>();
   cudaLaunchConfig_t cfg = {};
@@ -638,7 +652,7 @@ int spx_verify_max_clusters(int dev, int size) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (spx_opt_in_smem(kernel, smem, &once) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+  if (spx_opt_in_smem(kernel, smem, &once, true) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
@@ -661,13 +675,14 @@ cudaError_t spx_launch_verify(const AttnArgs& a, cudaStream_t st, int* n_launche
   }
   ok = ok && spx_encode_map(&maps.q, a.Q, p.D, p.Hq, a.q_sh, p.T, a.q_st, p.G, p.q_rows / p.G);
   if (!ok) return cudaErrorInvalidValue;
+  const int merge = p.cluster == 0 ? 0 : p.rows <= kRowsBySmem ? 1 : p.cluster <= 8 ? 2 : 3;
   cudaError_t e;
-  if (p.cluster == 0)
-    e = p.D == 128 ? launch_class<128, 0>(a, maps, st) : launch_class<64, 0>(a, maps, st);
-  else if (p.rows <= kRowsBySmem)
-    e = p.D == 128 ? launch_class<128, 1>(a, maps, st) : launch_class<64, 1>(a, maps, st);
-  else
-    e = p.D == 128 ? launch_class<128, 2>(a, maps, st) : launch_class<64, 2>(a, maps, st);
+  switch (merge) {
+    case 0: e = launch_dim<0>(a, maps, st); break;
+    case 1: e = launch_dim<1>(a, maps, st); break;
+    case 2: e = launch_dim<2>(a, maps, st); break;
+    default: e = launch_dim<3>(a, maps, st); break;
+  }
   *n_launches += 1;
   return e;
 }

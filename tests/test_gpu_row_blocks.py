@@ -23,6 +23,7 @@ pytestmark = pytest.mark.gpu
     (2, 2, 128, 1, 100), (32, 8, 128, 1, 500), (32, 8, 128, 8, 700), (32, 8, 128, 9, 700), (8, 8, 128, 7, 900),
     (12, 12, 64, 32, 900), (12, 12, 64, 33, 4096), (32, 32, 128, 100, 300), (32, 8, 128, 60, 130), (32, 8, 128, 60, 2048),
     (64, 8, 128, 60, 1000), (32, 8, 128, 127, 513),
+    (32, 8, 128, 10, 1012), (32, 8, 128, 30, 1300), (16, 4, 128, 32, 2000), (8, 2, 64, 40, 2048),    # more than 8 CTAs
 ])
 def test_one_cta_row_blocks(cuda_device, Hq, Hkv, D, T, L):
     w = synth.Workload("rows", Hq, Hkv, D, L, T, 32, 4, "uniform", "needle", seed=Hq + T + L)
