@@ -117,6 +117,8 @@ PyObject* guarded(Py_ssize_t nargs, Py_ssize_t want, Body&& body) {
     return nullptr;
   }
 }
+// Runs the entry point without the interpreter lock.  `call` holds plain values only: what a tensor's accessors throw (a
+// wrapped tensor has no data pointer) has to be thrown before, while the lock is held.
 template <typename Call>
 PyObject* released(Call&& call) {
   int rc;
@@ -171,11 +173,12 @@ PyObject* verify_attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
     float* lse = f32(a[9], kAttnTypes);
     float* score = a[10] == Py_None ? nullptr : f32(a[10], "chunk_score must be fp32");
     int32_t* status = i32(a[12], kAttnTypes);
-    const at::Tensor& ws = cuda_tensor(a[11]);
+    void* ws = ptr(a[11]);
+    const size_t ws_bytes = tensor(a[11]).nbytes();
     const auto fn = entry<decltype(&specext_verify_attn)>(a[0]);
     void *Q = ptr(a[2]), *Kp = ptr(a[3]), *Vp = ptr(a[4]), *Kt = ptr(a[5]), *Vt = ptr(a[6]), *O = ptr(a[8]);
     void* st = stream();
-    return released([&] { return fn(d.get(), Q, Kp, Vp, Kt, Vt, parent, O, lse, score, ws.data_ptr(), ws.nbytes(), status, st); });
+    return released([&] { return fn(d.get(), Q, Kp, Vp, Kt, Vt, parent, O, lse, score, ws, ws_bytes, status, st); });
   });
 }
 
@@ -190,11 +193,12 @@ PyObject* draft_attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int32_t* parent = i32(a[8], types);
     float* lse = f32(a[10], types);
     int32_t* status = i32(a[12], types);
-    const at::Tensor& ws = cuda_tensor(a[11]);
+    void* ws = ptr(a[11]);
+    const size_t ws_bytes = tensor(a[11]).nbytes();
     const auto fn = entry<decltype(&specext_draft_attn)>(a[0]);
     void *Q = ptr(a[2]), *K = ptr(a[3]), *V = ptr(a[4]), *Kt = ptr(a[6]), *Vt = ptr(a[7]), *O = ptr(a[9]);
     void* st = stream();
-    return released([&] { return fn(d.get(), Q, K, V, n_tokens, Kt, Vt, parent, O, lse, ws.data_ptr(), ws.nbytes(), status, st); });
+    return released([&] { return fn(d.get(), Q, K, V, n_tokens, Kt, Vt, parent, O, lse, ws, ws_bytes, status, st); });
   });
 }
 
@@ -257,11 +261,12 @@ PyObject* select_gather(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* n_tokens = static_cast<int32_t*>(ptr(a[16]));
     int32_t* status = static_cast<int32_t*>(ptr_or_null(a[17]));
     const auto fn = entry<decltype(&specext_select_gather)>(a[0]);
+    void *k_in = dK.data_ptr(), *v_in = dV.data_ptr(), *k_out = Ko.data_ptr(), *v_out = Vo.data_ptr();
+    const int64_t s_layer = dK.stride(0), s_l = dK.stride(1), s_h = dK.stride(2);
     void* st = stream();
     return released([&] {
-      return fn(score, n_tree, n_chunks, row, L, C, k, n_sink, n_recent, dK.data_ptr(), dV.data_ptr(), (int32_t)nl,
-                (int32_t)H, (int32_t)D, dK.stride(0), dK.stride(1), dK.stride(2), idx, n_selected, Ko.data_ptr(),
-                Vo.data_ptr(), n_tokens, status, st);
+      return fn(score, n_tree, n_chunks, row, L, C, k, n_sink, n_recent, k_in, v_in, (int32_t)nl, (int32_t)H, (int32_t)D,
+                s_layer, s_l, s_h, idx, n_selected, k_out, v_out, n_tokens, status, st);
     });
   });
 }
