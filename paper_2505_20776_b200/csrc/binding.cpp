@@ -9,6 +9,8 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#include <initializer_list>
+
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -80,6 +82,15 @@ float real(PyObject* o) {
   const double v = PyFloat_AsDouble(o);
   if (v == -1.0 && PyErr_Occurred()) throw PyFailure();
   return static_cast<float>(v);
+}
+// Whether `t` holds the product of the factors (none of them negative), which may not fit 64 bits.
+bool holds(const at::Tensor& t, std::initializer_list<int64_t> factors) {
+  int64_t need = 1;
+  for (const int64_t f : factors)
+    if (f == 0) return true;
+  for (const int64_t f : factors)
+    if (__builtin_mul_overflow(need, f, &need)) return false;
+  return t.numel() >= need;
 }
 template <typename F>
 F entry(PyObject* address) {
@@ -255,8 +266,9 @@ PyObject* select_gather(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* n_selected = i32(a[13], "idx and n_selected must be int32");
     if (tensor(a[12]).numel() < (k < n_chunks ? k : n_chunks)) fail("idx is too small");
     const at::Tensor &Ko = cuda_tensor(a[14]), &Vo = cuda_tensor(a[15]);
-    const int64_t nl = dK.size(0), H = dK.size(2), D = dK.size(3), need = nl * k * C * H * D;
-    if (!Ko.is_contiguous() || !Vo.is_contiguous() || Ko.numel() < need || Vo.numel() < need)
+    const int64_t nl = dK.size(0), H = dK.size(2), D = dK.size(3);
+    const std::initializer_list<int64_t> out = {nl, k < 0 ? 0 : k, C < 0 ? 0 : C, H, D};   // (negative: refused by the library)
+    if (!Ko.is_contiguous() || !Vo.is_contiguous() || !holds(Ko, out) || !holds(Vo, out))
       fail("K_out/V_out must be contiguous and hold [layers][k*C][H][D]");
     int32_t* n_tokens = static_cast<int32_t*>(ptr(a[16]));
     int32_t* status = static_cast<int32_t*>(ptr_or_null(a[17]));

@@ -36,3 +36,15 @@ def test_a_tensor_without_memory_raises_before_the_lock_is_released(call):
     batched = _fake(1, 4096, dtype=torch.bfloat16)
     with pytest.raises(RuntimeError, match=NO_POINTER):
         torch.func.vmap(lambda t: call(t))(batched)
+
+
+@pytest.mark.parametrize("k,C,layers,heads,dim", [
+    (2 ** 31 - 1, 2 ** 31 - 1, 1, 4, 8),           # the product wraps to a negative number
+    (2 ** 14, 2 ** 14, 2 ** 15, 2 ** 11, 2 ** 10), # to zero, with every factor in the library's range
+    (9, 1, 1, 4, 8),                               # one token too many
+])
+def test_select_gather_output_size_does_not_wrap(k, C, layers, heads, dim):
+    """A compact cache that is too small for [layers][k * C][heads][dim] is refused whatever the product."""
+    draft = _fake(1, 1, heads, dim, dtype=torch.bfloat16).expand(layers, 100, heads, dim)
+    with pytest.raises(ValueError, match="must be contiguous and hold"):
+        _select_gather(_fake(8 * 32, dtype=torch.bfloat16), k, C, draft)
