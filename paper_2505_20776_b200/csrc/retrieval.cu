@@ -230,8 +230,10 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
 // loads a lane) in flight.  Where a segment lies is worked out once for the warp: per vector, the integer divisions took
 // longer than the copy.
 __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32_t* s_idx, int keff) {
-  const int vpr = g.D / 8, vpt = g.H * vpr, vpc = g.C * vpt;       // vectors per head row, token, chunk
-  const uint32_t spc = (uint32_t)(vpc + 63) / 64;                  // segments per chunk
+  const int vpr = g.D / 8, vpt = g.H * vpr;                        // vectors per head row, token
+  const long long vpc = (long long)g.C * vpt;                      // per chunk of the compact cache
+  // segments per chunk (which may be longer than the prefix)
+  const uint32_t spc = (uint32_t)(((long long)min(g.C, g.L) * vpt + 63) / 64);
   const uint32_t n_seg = 2u * g.n_layers * keff * spc;
   const bool contiguous = g.s_h == g.D && g.s_l == (long long)g.H * g.D;
   const int lane = threadIdx.x & 31;
@@ -251,7 +253,8 @@ __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32
         const uint32_t part = chunk / (uint32_t)keff, i = chunk - part * keff;
         const uint32_t which = part / (uint32_t)g.n_layers, layer = part - which * g.n_layers;
         const int c = s_idx[i];
-        if (c >= 0 && c < g.NC) lim[q] = min(g.C, g.L - c * g.C) * vpt - (int)w0;     // vectors of the chunk from here on
+        // vectors of the chunk from here on, as far as this segment goes
+        if (c >= 0 && c < g.NC) lim[q] = (int)max(0ll, min((long long)min(g.C, g.L - c * g.C) * vpt - w0, 64ll));
         const __nv_bfloat16* base = g.src[which] + (long long)layer * g.s_layer + (long long)c * g.C * g.s_l;
         dst[q] = reinterpret_cast<uint4*>(g.dst[which]) + ((long long)layer * g.max_selected + i) * vpc + w0 + lane;
         if (contiguous) {
@@ -262,7 +265,8 @@ __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32
         } else {
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            const int w = (int)w0 + lane + 32 * e, o = w / vpt, r = w - o * vpt, h = r / vpr;
+            const uint32_t w = w0 + lane + 32 * e, o = w / (uint32_t)vpt;
+            const int r = (int)(w - o * vpt), h = r / vpr;
             if (lane + 32 * e < lim[q])
               x[q][e] = __ldg(reinterpret_cast<const uint4*>(base + (long long)o * g.s_l + (long long)h * g.s_h + (r - h * vpr) * 8));
           }
@@ -386,7 +390,7 @@ cudaError_t spx_launch_select_gather(const float* score_row, int k, int n_sink, 
   g.n_recent = n_recent;
   void* args[] = {&g};
   const int keff = k < g.NC ? k : g.NC;
-  const long long segments = 2ll * n_layers * keff * (((long long)C * H * (D / 8) + 63) / 64);
+  const long long segments = 2ll * n_layers * keff * (((long long)(C < L ? C : L) * H * (D / 8) + 63) / 64);
   const long long blocks = (segments + kSelThreads / 32 - 1) / (kSelThreads / 32);
   const void* kernel = g.NC <= kSelThreads       ? reinterpret_cast<const void*>(select_gather_kernel<1>)
                        : g.NC <= 4 * kSelThreads ? reinterpret_cast<const void*>(select_gather_kernel<4>)

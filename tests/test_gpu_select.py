@@ -38,3 +38,23 @@ def test_select_gather_chunk_counts(cuda_device, L, C, k, ties):
         ref, _, n = orc.gather_kv(bf16_bits(src), bf16_bits(src), want, L, C)
         assert int(nt.item()) == n
         np.testing.assert_array_equal(bf16_bits(out)[:, :n], ref)
+
+
+def test_chunk_size_far_beyond_the_prefix(cuda_device):
+    """One chunk of 2^24 tokens, 2^32 vectors of 16 bytes in the compact cache's layout, of which 100 tokens exist: they are
+    copied (only valid tokens are written, so the buffers hold just these; the binding would ask for the whole layout)."""
+    dev, L, C, H, D = cuda_device, 100, 1 << 24, 16, 128
+    dK, dV = (torch.randn(1, L, H, D, device=dev).to(torch.bfloat16) for _ in range(2))
+    g = GuardedAlloc(dev)
+    idx, ns, nt = (g.alloc((1,), torch.int32).fill_(-1) for _ in range(3))
+    status = g.alloc((1,), torch.int32).zero_()
+    K, V = (g.alloc((L, H, D), torch.bfloat16).zero_() for _ in range(2))
+    scores = torch.ones(1, 1, device=dev)
+    torch.cuda.synchronize()
+    rc = api.lib().specext_select_gather(scores.data_ptr(), 1, 1, 0, L, C, 1, 0, 0, dK.data_ptr(), dV.data_ptr(), 1, H, D,
+                                         L * H * D, H * D, D, idx.data_ptr(), ns.data_ptr(), K.data_ptr(), V.data_ptr(),
+                                         nt.data_ptr(), status.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and api.specext_read_status(status) == 0
+    g.check()
+    assert [int(x.item()) for x in (idx, ns, nt)] == [0, 1, L]
+    assert torch.equal(K, dK[0]) and torch.equal(V, dV[0])
