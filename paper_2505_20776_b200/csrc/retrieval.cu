@@ -1,7 +1,8 @@
 // SelectChunks and UpdateDraftCache kernels.
 //
 // The ranking key of chunk c is score[c] / len_c, a non-negative fp32 whose bit pattern orders like the value.  A block
-// reads every key once, into registers (thread t holds the keys of consecutive chunks), finds the k-th largest by a
+// reads every key once, into registers (thread t holds the keys of consecutive chunks; above 16384 chunks 64 of them, which
+// is all the registers a thread of 1024 has, so that some are spilled), finds the k-th largest by a
 // most-significant-digit radix select (at most 4 passes of 8 bits over shared-memory histograms) and emits the kept
 // chunks in ascending order after one block-wide scan: a chunk with a larger key is kept, and of the chunks equal to the
 // k-th the lowest-indexed are kept until k are chosen.
@@ -10,7 +11,8 @@
 // emission; the copy that follows has all its loads in flight at once.  select_gather_kernel, us per call replayed alone
 // (draft cache in L2), against the form with two barriers per pass, one emission round per 256 chunks and the selection
 // repeated by 256 to 512 blocks: 128 chunks 5.5 -> 5.6, 512 chunks 6.5 -> 5.1, 4096 chunks 29.7 -> 10.2, two layers of
-// 12 x 64 heads and 257 chunks 7.9 -> 6.2.
+// 12 x 64 heads and 257 chunks 7.9 -> 6.2.  select_kernel above 8192 chunks, against the form that recomputed the keys in
+// every pass: 10000 chunks 30.7 -> 11.8, 16384 46.3 -> 14.3 (with 64 keys a thread 39.5), 20000 56.7 -> 42.5, 65536 193 -> 72.
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -351,10 +353,13 @@ cudaError_t spx_launch_select(const float* score_row, int NC, int L, int C, int 
                               int32_t* idx, int32_t* n_selected, cudaStream_t st) {
   SelShape sh = {NC, L, C, n_sink, n_recent};
   void* args[] = {&score_row, &sh, &k, &idx, &n_selected};
-  const void* kernel = NC <= 512    ? reinterpret_cast<const void*>(select_kernel<512, 1>)
-                       : NC <= 2048 ? reinterpret_cast<const void*>(select_kernel<512, 4>)
-                       : NC <= 8192 ? reinterpret_cast<const void*>(select_kernel<512, 16>)
-                                    : reinterpret_cast<const void*>(select_kernel<1024, 64>);
+  // The fewest keys a thread that hold NC: one block, whose time is its threads' chain of keys.  1024 threads with 16 keys
+  // between the two largest classes: 8193 to 10000 chunks took 40 us with 64 keys, more than the 28 to 31 of the form before.
+  const void* kernel = NC <= 512     ? reinterpret_cast<const void*>(select_kernel<512, 1>)
+                       : NC <= 2048  ? reinterpret_cast<const void*>(select_kernel<512, 4>)
+                       : NC <= 8192  ? reinterpret_cast<const void*>(select_kernel<512, 16>)
+                       : NC <= 16384 ? reinterpret_cast<const void*>(select_kernel<1024, 16>)
+                                     : reinterpret_cast<const void*>(select_kernel<1024, 64>);
   return launch_pdl(kernel, dim3(1), dim3(NC <= 8192 ? 512 : 1024), args, st);
 }
 

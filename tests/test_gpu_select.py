@@ -58,3 +58,10 @@ def test_chunk_size_far_beyond_the_prefix(cuda_device):
     g.check()
     assert [int(x.item()) for x in (idx, ns, nt)] == [0, 1, L]
     assert torch.equal(K, dK[0]) and torch.equal(V, dV[0])
+
+
+@pytest.mark.parametrize("L,k", [(16384, 900), (16385, 900), (16000, 16000)])
+@pytest.mark.parametrize("ties", [False, True])
+def test_select_gather_sixteen_keys_a_thread_of_1024(cuda_device, L, k, ties):
+    """Both sides of the line between 16 and 64 keys per thread, and every chunk kept."""
+    test_select_gather_chunk_counts(cuda_device, L, 1, k, ties)
