@@ -161,6 +161,12 @@ int cluster_size(const AttnPlan& p, bool pair) {
   const int most = pair ? (tiles <= 16 ? (split > 3 ? split : 3) : 0)
                         : split + (p.D == 64 ? 3 : split > 30 ? split / 6 : 5);
   if (tiles > most) return 0;
+  // Chunks of fewer than 32 keys make a tile cost more than twice as much (a running sum and a store per chunk), so that an
+  // extra tile outweighs the launch.  Chunks of 16, before clusters / split / cluster: 60 nodes at 2K 24.0 / 22.0 / 26.1
+  // (clusters of 9 with 2 tiles), 32 x 64 query / 8 KV heads at 8K 52.0 / 47.0 / 58.7 (8 tiles against 8), one node of 16
+  // query / 2 KV heads at 4K 25.8 / 21.1 / 29.9 (5 against 1); with 2 tiles in at most 8 CTAs, 100 nodes at 500 tokens
+  // 23.3 / 19.5 / 19.2, with one tile 60 nodes of 32 KV heads at 200 23.2 / 20.5 / 18.5.
+  if (p.want_score && p.C < 32 && (tiles > 2 || (tiles == 2 && size > 8))) return 0;
   while (size > 2 && (p.UPP + size - 2) / (size - 1) == tiles) --size;     // no more CTAs than the tile count needs
   return size;
 }

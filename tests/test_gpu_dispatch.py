@@ -1,0 +1,41 @@
+"""Which form a call takes, seen by the kernels it launches: one whose clusters merge by themselves is one launch, one that
+leaves partial results two, and the chunk scores are one more.  On the B200 (clusters of up to 16 of its CTAs)."""
+import pytest
+import torch
+
+from paper_2505_20776_b200 import api
+
+pytestmark = pytest.mark.gpu
+
+
+def launches(dev, Hq, Hkv, D, T, L, C=32, scored=False, n_tokens=None):
+    """Kernels launched by one call on zeros; n_tokens: the device-side length of a draft call."""
+    z = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device=dev)
+    Q, K, Kt, O = z(T, Hq, D), z(max(L, 1), Hkv, D), z(T, Hkv, D), z(T, Hq, D)
+    lse = torch.zeros(Hq, T, device=dev)
+    score = torch.zeros(T, -(-L // C), device=dev) if scored else None
+    parent = torch.full((T,), -1, dtype=torch.int32, device=dev)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    d = api.make_attn_desc(Q, K, Kt, O, L, C, 0.0, scored)
+    ws = torch.empty(api.specext_verify_attn_workspace(d), dtype=torch.uint8, device=dev)
+    before = api.specext_launch_count()
+    if n_tokens is None:
+        api.specext_verify_attn(d, Q, K, K, Kt, Kt, parent, O, lse, score, ws, status)
+    else:
+        n = torch.tensor([n_tokens], dtype=torch.int32, device=dev)
+        api.specext_draft_attn(d, Q, K, K, n, Kt, Kt, parent, O, lse, ws, status)
+    after = api.specext_launch_count()
+    assert api.specext_read_status(status) == 0
+    return after - before
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,L,C,want", [
+    (32, 8, 128, 60, 2048, 16, 3),      # clusters of 9 with two tiles: split for small chunks
+    (32, 8, 128, 60, 2048, 32, 2),      # and not for larger ones
+    (32, 8, 64, 60, 8192, 4, 3), (32, 8, 64, 60, 8192, 64, 2),
+    (16, 2, 128, 1, 4096, 16, 3), (16, 2, 128, 1, 4096, 128, 2),
+    (32, 8, 128, 100, 500, 16, 2),      # two tiles in clusters of 3
+    (32, 32, 128, 60, 200, 1, 2),       # one tile
+])
+def test_small_chunks_stay_on_the_split_path(cuda_device, Hq, Hkv, D, T, L, C, want):
+    assert launches(cuda_device, Hq, Hkv, D, T, L, C, scored=True) == want
