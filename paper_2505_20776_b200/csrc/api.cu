@@ -158,15 +158,21 @@ int cluster_size(const AttnPlan& p, bool pair) {
   //   60 nodes, 32 KV heads: 1K 13.5 / 10.7, 8K 29.5 / 26.6 (17 against 15), 32K 91.3 / 88.9 (65 against 56)
   //   1 node: 2K 10.8 / 8.0, 8K 15.8 / 14.8 (9 against 4), 16K 19.3 / 22.5 (17 against 7)
   //   12 x 64 heads: 4K 11.7 / 9.3 (5 against 3);  60 nodes, 32 x 64 query / 8 KV heads, 16K: 22.7 / 24.5 (19 against 14)
-  const int most = pair ? (tiles <= 16 ? (split > 3 ? split : 3) : 0)
-                        : split + (p.D == 64 ? 3 : split > 30 ? split / 6 : 5);
+  int most = pair ? (tiles <= 16 ? (split > 3 ? split : 3) : 0)
+                  : split + (p.D == 64 ? 3 : split > 30 ? split / 6 : 5);
+  // Chunks of fewer than 32 keys make a tile cost more than twice as much (a running sum and a store per chunk), so that extra
+  // tiles outweigh the launch they save.  Chunks of 16, before clusters / split / cluster: 60 nodes at 2K 24.0 / 22.0 / 26.1
+  // (3 tiles against 2), 32 x 64 query / 8 KV heads at 8K 52.0 / 47.0 / 58.7 (11 against 8), one node of 16 query / 2 KV heads
+  // at 4K 25.8 / 21.1 / 29.9 (5 against 1); but 100 nodes at 1K 30.3 / 28.3 / 26.4 (3 against 3), 32 KV heads of 60 nodes at
+  // 6K 124 / 67.4 / 65.3 (12 against 11), 12 x 64 heads of 100 nodes at 4K 37.9 / 30.6 / 25.2 (4 against 3).
+  if (p.want_score && p.C < 32) {
+    int most_small;
+    if (pair) most_small = tiles <= (p.C == 16 ? 12 : 5) ? split : 0;    // 4 keys: 7 against 7 0.3 to 9 % slower, 12 1 to 11 %
+    else most_small = tiles <= 4 && (size > 8 || split >= 3) ? 4 : p.D == 64 ? split : split * 6 / 5;
+    if (most_small < 2) most_small = 2;
+    if (most > most_small) most = most_small;
+  }
   if (tiles > most) return 0;
-  // Chunks of fewer than 32 keys make a tile cost more than twice as much (a running sum and a store per chunk), so that an
-  // extra tile outweighs the launch.  Chunks of 16, before clusters / split / cluster: 60 nodes at 2K 24.0 / 22.0 / 26.1
-  // (clusters of 9 with 2 tiles), 32 x 64 query / 8 KV heads at 8K 52.0 / 47.0 / 58.7 (8 tiles against 8), one node of 16
-  // query / 2 KV heads at 4K 25.8 / 21.1 / 29.9 (5 against 1); with 2 tiles in at most 8 CTAs, 100 nodes at 500 tokens
-  // 23.3 / 19.5 / 19.2, with one tile 60 nodes of 32 KV heads at 200 23.2 / 20.5 / 18.5.
-  if (p.want_score && p.C < 32 && (tiles > 2 || (tiles == 2 && size > 8))) return 0;
   while (size > 2 && (p.UPP + size - 2) / (size - 1) == tiles) --size;     // no more CTAs than the tile count needs
   return size;
 }

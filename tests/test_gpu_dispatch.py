@@ -30,11 +30,14 @@ def launches(dev, Hq, Hkv, D, T, L, C=32, scored=False, n_tokens=None):
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,T,L,C,want", [
-    (32, 8, 128, 60, 2048, 16, 3),      # clusters of 9 with two tiles: split for small chunks
-    (32, 8, 128, 60, 2048, 32, 2),      # and not for larger ones
-    (32, 8, 64, 60, 8192, 4, 3), (32, 8, 64, 60, 8192, 64, 2),
-    (16, 2, 128, 1, 4096, 16, 3), (16, 2, 128, 1, 4096, 128, 2),
-    (32, 8, 128, 100, 500, 16, 2),      # two tiles in clusters of 3
+    (32, 8, 128, 60, 2048, 16, 3),      # clusters of 6: 3 tiles instead of 2
+    (32, 8, 128, 60, 2048, 32, 2),      # which is fine for larger chunks
+    (32, 8, 64, 60, 8192, 4, 3), (32, 8, 64, 60, 8192, 64, 2),          # 11 tiles instead of 8
+    (16, 2, 128, 1, 4096, 16, 3), (16, 2, 128, 1, 4096, 128, 2),        # 5 instead of 1
+    (32, 8, 128, 100, 1000, 16, 2),     # 3 instead of 3
+    (32, 8, 128, 100, 2048, 4, 2), (32, 8, 128, 100, 3000, 4, 3),       # 5, 7
+    (32, 32, 128, 60, 6000, 16, 2),     # 12 instead of 11
+    (12, 12, 64, 100, 4096, 16, 2),     # 4 instead of 3
     (32, 32, 128, 60, 200, 1, 2),       # one tile
 ])
 def test_small_chunks_stay_on_the_split_path(cuda_device, Hq, Hkv, D, T, L, C, want):
