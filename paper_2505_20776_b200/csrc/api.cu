@@ -154,11 +154,25 @@ int cluster_size(const AttnPlan& p, bool pair) {
   // fetch half of every K/V tile, win again when the tiles are many.  us per call, split / cluster, replayed (32 query / 8 KV
   // heads unless said; launched one by one the cluster form gains another 0.5):
   //   60 nodes: 1K 10.9 / 9.9, 2K 11.6 / 10.7 (3 tiles against 2), 3K 12.5 / 13.1 (4 against 3), 4K 13.4 / 13.6 (5 against 4)
-  //   60 nodes, 64 query heads: 1K 13.4 / 11.5, 4K 16.2 / 16.8 (9 against 9; one by one 17.5 / 17.2), 16K 34.3 / 38.0 (33)
+  //   60 nodes, 64 query heads: 1K 13.4 / 11.5, 2K 13.2 / 13.1 (5 against 5), 4K 16.3 / 16.9 (9; one by one 17.5 / 17.2)
   //   60 nodes, 32 KV heads: 1K 13.5 / 10.7, 8K 29.5 / 26.6 (17 against 15), 32K 91.3 / 88.9 (65 against 56)
   //   1 node: 2K 10.8 / 8.0, 8K 15.8 / 14.8 (9 against 4), 16K 19.3 / 22.5 (17 against 7)
   //   12 x 64 heads: 4K 11.7 / 9.3 (5 against 3);  60 nodes, 32 x 64 query / 8 KV heads, 16K: 22.7 / 24.5 (19 against 14)
-  int most = pair ? (tiles <= 16 ? (split > 3 ? split : 3) : 0)
+  // Against the pairs the gain is used up at six tiles (7 against 7, 100 nodes at 3K 14.6 / 15.0, scored 17.9 / 18.4), unless
+  //   the pairs have more tiles (80 nodes at 8K 22.2 / 20.7, 17 against 13: blocks of 256 rows pad 320 to 512) or
+  //   their merge takes a second wave of blocks (256 threads: 32 query / 4 KV heads, 80 nodes at 5K 17.1 / 14.9, scored
+  //   20.5 / 18.2; 512 threads: 64 query / 8 KV heads, 80 nodes at 5K 22.2 / 21.6, scored 26.8 / 25.9), which two segments a
+  //   row make up for sooner (100 nodes at 2K 18.0 / 17.6 with 9 tiles, 3K 21.0 / 21.2 with 13);
+  //   without scores also a cluster of more than 8 CTAs (100 nodes of 16 query / 2 KV heads at 8K 15.8 / 15.1 with 8 tiles,
+  //   scored 19.5 / 20.3).
+  int limit = 0;
+  if (pair) {
+    const int np2 = p.Hkv * ((p.rows + 255) / 256), per = sm_count() / 2 / np2;      // (np2 <= np <= half of the SMs)
+    const bool second_wave = 8 * np2 * (per > 4 ? 2 : 1) > sm_count();
+    limit = tiles < split || (second_wave && per > 2) ? 16 : second_wave || (!p.want_score && size > 8) ? 11 : 6;
+    if (p.want_score && p.C < 32) limit = 16;                                         // (see below)
+  }
+  int most = pair ? (tiles <= limit ? (split > 3 ? split : 3) : 0)
                   : split + (p.D == 64 ? 3 : split > 30 ? split / 6 : 5);
   // Chunks of fewer than 32 keys make a tile cost more than twice as much (a running sum and a store per chunk), so that extra
   // tiles outweigh the launch they save.  Chunks of 16, before clusters / split / cluster: 60 nodes at 2K 24.0 / 22.0 / 26.1

@@ -42,3 +42,16 @@ def launches(dev, Hq, Hkv, D, T, L, C=32, scored=False, n_tokens=None):
 ])
 def test_small_chunks_stay_on_the_split_path(cuda_device, Hq, Hkv, D, T, L, C, want):
     assert launches(cuda_device, Hq, Hkv, D, T, L, C, scored=True) == want
+
+
+@pytest.mark.parametrize("Hq,Hkv,T,L,scored,want", [
+    (64, 8, 60, 2048, False, 1), (64, 8, 60, 3000, False, 2),        # 5 and 7 tiles in clusters of 4
+    (64, 8, 60, 2048, True, 2), (64, 8, 60, 4096, True, 3),
+    (64, 8, 100, 2048, False, 1), (64, 8, 100, 2048, True, 2),       # 9 tiles, 32 blocks of 256 rows
+    (16, 2, 100, 8192, False, 1), (16, 2, 100, 8192, True, 3),       # 8 tiles in clusters of 9
+    (64, 8, 100, 3000, False, 2), (64, 8, 80, 4096, True, 2),        # 13 tiles; 11, 24 blocks
+    (32, 8, 80, 8192, True, 2),                                      # 13 tiles against 17
+    (32, 4, 80, 6000, True, 2),                                      # 8 tiles, 12 blocks of 256 rows and 6 segments to merge
+])
+def test_many_tiles_go_to_the_pairs(cuda_device, Hq, Hkv, T, L, scored, want):
+    assert launches(cuda_device, Hq, Hkv, 128, T, L, 32, scored) == want
