@@ -148,9 +148,12 @@ __global__ void __launch_bounds__(kScoreThreads) score_kernel(const __grid_const
         if (g < p.Hkv) {
           const long long base = ((long long)(g * p.n_rblk + rblk) * p.TPH + tile) * p.RB + rr;
           const float* src = a.ws + p.off_mass + base * p.CPT + c0;
-          if (VW == 4) {
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
-            m[q][0] = v.x; m[q][1 % VW] = v.y; m[q][2 % VW] = v.z; m[q][3 % VW] = v.w;
+          if (VW >= 4) {
+#pragma unroll
+            for (int e = 0; e < VW / 4; ++e) {
+              const float4 v = __ldcg(reinterpret_cast<const float4*>(src) + e);
+              m[q][e * 4] = v.x; m[q][(e * 4 + 1) % VW] = v.y; m[q][(e * 4 + 2) % VW] = v.z; m[q][(e * 4 + 3) % VW] = v.w;
+            }
           } else if (VW == 2) {
             const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
             m[q][0] = v.x; m[q][1 % VW] = v.y;
@@ -248,7 +251,14 @@ cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches
     if (e != cudaSuccess) return e;
   }
   if (p.want_score && p.NC > 0) {
-    e = p.CPT >= 4 ? launch_score<4>(a, st) : p.CPT == 2 ? launch_score<2>(a, st) : launch_score<1>(a, st);
+    // With 16 chunks and more in a tile groups of 8: a 32-byte sector of a row's sums is then read by one block and not by two
+    // (chunks of 4 at 12K, 32 query / 4 KV heads with 100 nodes 147 -> 142 us a call, 64 / 2 heads with 60 nodes 175 -> 160).  Not where they make
+    // fewer than four blocks per SM (60 nodes at 3K 36.8 -> 40.3, 100 nodes of 16 KV heads at 500 tokens 19.4 -> 20.9).
+    const long long wide = (long long)p.TPH * (p.CPT / 8) * p.n_rblk;
+    e = p.CPT >= 16 && wide >= 4 * 148 ? launch_score<8>(a, st)
+        : p.CPT >= 4                   ? launch_score<4>(a, st)
+        : p.CPT == 2                   ? launch_score<2>(a, st)
+                                       : launch_score<1>(a, st);
     *n_launches += 1;
   }
   return e;

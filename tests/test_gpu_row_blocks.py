@@ -37,3 +37,12 @@ def test_prefill_wide_groups(cuda_device, G):
     Q, K, V = _inputs(L, G, 1, seed=G)
     O, lse = _run(cuda_device, Q, K, V)
     _compare(O, lse, Q, K, V, [0, 1, 2, 3, 4, 63, 64, 126, 127, 128, 129, 130], f"prefill-small-G{G}")
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,L,C", [
+    (8, 2, 128, 128, 9500, 4),      # groups of 8 chunks: two row blocks, 32 chunks in a tile, a ragged last one
+    (8, 8, 64, 3, 6400, 1),         # 128 chunks in a tile
+])
+def test_chunk_scores_in_groups_of_eight(cuda_device, Hq, Hkv, D, T, L, C):
+    w = synth.Workload("score8", Hq, Hkv, D, L, T, C, 4, "uniform", "needle", seed=T + C)
+    check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, C)
