@@ -39,6 +39,7 @@ def launches(dev, Hq, Hkv, D, T, L, C=32, scored=False, n_tokens=None):
     (32, 32, 128, 60, 6000, 16, 2),     # 12 instead of 11
     (12, 12, 64, 100, 4096, 16, 2),     # 4 instead of 3
     (32, 32, 128, 60, 200, 1, 2),       # one tile
+    (32, 8, 128, 60, 1000, 1, 3), (32, 8, 128, 60, 1000, 4, 2),         # 2 instead of 1
 ])
 def test_small_chunks_stay_on_the_split_path(cuda_device, Hq, Hkv, D, T, L, C, want):
     assert launches(cuda_device, Hq, Hkv, D, T, L, C, scored=True) == want
