@@ -523,11 +523,12 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
                 cg[c] = sum;
               } else if (SCORE == 3 && mass) {
                 float acc = 0.f;
+                float* dst = mass + c * (32 / p.C);      // (one division here, none per store)
 #pragma unroll
                 for (int k = 0; k < 32; ++k) {
                   acc += __uint_as_float(v[k]);
                   if (((k + 1) & (p.C - 1)) == 0) {
-                    mass[(c * 32 + k) / p.C] = acc;
+                    *dst++ = acc;
                     acc = 0.f;
                   }
                 }
