@@ -142,6 +142,12 @@ int cluster_size(const AttnPlan& p, bool pair) {
   for (int s = p.rows > kSpxClusterRowsBySmem ? 16 : 8; s >= 2 && size == 0; --s)
     if (s <= p.UPP && np * s <= sm_count() && np <= spx_verify_max_clusters(dev, s)) size = s;
   if (size == 0) return 0;
+  // A prefix of one tile gives clusters of two, which merge half of the rows' columns each: above 64 rows longer than the
+  // merge kernel takes, unless the problems are many.  us per call, before clusters / split / cluster, 100 tokens: 60 nodes
+  // 9.4 / 9.2 / 9.6, 100 nodes of 16 query / 2 KV heads 9.0 / 9.2 / 9.9, of 32 KV heads 12.4 / 10.0 / 10.5; but 60 nodes of
+  // 32 KV heads (60 rows) 10.5 / 9.0 / 8.9, 100 nodes of 64 query / 8 KV heads (56 problems) 14.5 / 12.6 / 11.5, of 64 KV
+  // heads 17.1 / 12.2 / 11.0.  (Between them 40 problems take 1.08 of the split form's time, 50 0.95.)
+  if (p.UPP == 2 && p.D == 128 && p.rows > 64 && np <= 40) return 0;
   const int tiles = (p.UPP + size - 1) / size;
   int split;
   if (pair) {

@@ -56,3 +56,12 @@ def test_small_chunks_stay_on_the_split_path(cuda_device, Hq, Hkv, D, T, L, C, w
 ])
 def test_many_tiles_go_to_the_pairs(cuda_device, Hq, Hkv, T, L, scored, want):
     assert launches(cuda_device, Hq, Hkv, 128, T, L, 32, scored) == want
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,L,want", [
+    (32, 8, 128, 60, 100, 2), (32, 8, 128, 60, 129, 1),      # one tile and the tree, two and the tree
+    (32, 8, 128, 16, 128, 1), (32, 8, 128, 17, 128, 2),      # 64 and 68 rows
+    (64, 64, 128, 100, 100, 1), (12, 12, 64, 100, 100, 1),   # many problems, head_dim 64
+])
+def test_prefix_of_one_tile(cuda_device, Hq, Hkv, D, T, L, want):
+    assert launches(cuda_device, Hq, Hkv, D, T, L) == want
