@@ -30,6 +30,7 @@
 // global memory is touched only after griddepcontrol.wait.
 #include "common.cuh"
 #include "pair.cuh"
+#include "tmap.h"
 
 using namespace sm100;
 using namespace pair;
@@ -798,49 +799,6 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn2() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(ptr);
-  }
-  return fn;
-}
-
-// bf16 tensor [n2][n1][128] with element strides (s2, s1, 1); box = 64 x 1 x b2, 128-byte swizzle,
-// out-of-range elements read as zero.
-bool encode_map2(CUtensorMap* m, const void* ptr, long long n1, long long s1, long long n2, long long s2, int b2) {
-  EncodeTiledFn fn = encode_fn2();
-  if (!fn) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)n1, (cuuint64_t)n2};
-  const cuuint64_t strides[2] = {(cuuint64_t)s1 * 2, (cuuint64_t)s2 * 2};
-  const cuuint32_t box[3] = {64, 1, (cuuint32_t)b2};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Q [T][Hq][128] (element strides q_st, q_sh, 1) with boxes of 64 elements x G heads x 128/G nodes.
-bool encode_q_map(CUtensorMap* m, const void* ptr, int T, int Hq, int G, long long q_st, long long q_sh) {
-  EncodeTiledFn fn = encode_fn2();
-  if (!fn || G > 128 || 128 % G != 0) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)T};
-  const cuuint64_t strides[2] = {(cuuint64_t)q_sh * 2, (cuuint64_t)q_st * 2};
-  const cuuint32_t box[3] = {64, (cuuint32_t)G, (cuuint32_t)(128 / G)};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int SCORE, bool DEVLEN>
 cudaError_t launch2(const AttnArgs& a, const Tc2Maps& maps, cudaStream_t st) {
   static SpxOncePerDevice once;
@@ -870,16 +828,17 @@ cudaError_t spx_launch_attn_tc2(const AttnArgs& a, cudaStream_t st, int* n_launc
   const AttnPlan& p = a.plan;
   if (p.D != D || p.RB != 256) return cudaErrorInvalidValue;
   Tc2Maps maps;
-  bool ok = encode_map2(&maps.kt, a.Kt, p.Hkv, a.tkv_sh, p.T, a.tkv_st, 64);
-  ok = ok && encode_map2(&maps.vt, a.Vt, p.Hkv, a.tkv_sh, p.T, a.tkv_st, SPX_TILE_KEYS);
+  bool ok = spx_encode_map(&maps.kt, a.Kt, D, p.Hkv, a.tkv_sh, p.T, a.tkv_st, 1, 64);
+  ok = ok && spx_encode_map(&maps.vt, a.Vt, D, p.Hkv, a.tkv_sh, p.T, a.tkv_st, 1, SPX_TILE_KEYS);
   if (p.L > 0) {
-    ok = ok && encode_map2(&maps.kp, a.Kp, p.Hkv, a.kv_sh, p.L, a.kv_sl, 64);
-    ok = ok && encode_map2(&maps.vp, a.Vp, p.Hkv, a.kv_sh, p.L, a.kv_sl, SPX_TILE_KEYS);
+    ok = ok && spx_encode_map(&maps.kp, a.Kp, D, p.Hkv, a.kv_sh, p.L, a.kv_sl, 1, 64);
+    ok = ok && spx_encode_map(&maps.vp, a.Vp, D, p.Hkv, a.kv_sh, p.L, a.kv_sl, 1, SPX_TILE_KEYS);
   } else {
     maps.kp = maps.kt;
     maps.vp = maps.vt;
   }
-  ok = ok && encode_q_map(&maps.q, a.Q, p.T, p.Hq, p.G, a.q_st, a.q_sh);
+  // Q [T][Hq][128]: boxes of 64 elements x G heads x 128/G nodes, the 128 stacked rows of one CTA
+  ok = ok && spx_encode_map(&maps.q, a.Q, D, p.Hq, a.q_sh, p.T, a.q_st, p.G, 128 / p.G);
   if (!ok) return cudaErrorInvalidValue;
   const cudaError_t e = a.L_dev       ? launch2<0, true>(a, maps, st)       // never with chunk sums
                         : !p.want_score ? launch2<0, false>(a, maps, st)

@@ -2,6 +2,8 @@
 #ifndef SPECEXT_TMAP_H_
 #define SPECEXT_TMAP_H_
 
+#include <atomic>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -9,15 +11,18 @@ typedef CUresult (*SpxEncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32
                                      const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// The driver's encoder, looked up until it is found (several threads may do so at once); null when there is no driver.
 inline SpxEncodeTiledFn spx_encode_fn() {
-  static const SpxEncodeTiledFn fn = [] {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess)
-      ptr = nullptr;
-    return reinterpret_cast<SpxEncodeTiledFn>(ptr);
-  }();
+  static std::atomic<SpxEncodeTiledFn> known{nullptr};
+  SpxEncodeTiledFn fn = known.load();
+  if (fn) return fn;
+  void* ptr = nullptr;
+  cudaDriverEntryPointQueryResult qres;
+  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) != cudaSuccess ||
+      qres != cudaDriverEntryPointSuccess)
+    return nullptr;
+  fn = reinterpret_cast<SpxEncodeTiledFn>(ptr);
+  known.store(fn);
   return fn;
 }
 
