@@ -294,7 +294,8 @@ __global__ void __launch_bounds__(kSelThreads) select_gather_kernel(const __grid
   __shared__ int32_t s_idx[kFusedMaxK];
   sm100::pdl_launch_dependents();
   const int keff = min(g.k, g.NC);
-  // (an index stays -1 only when the scores change while they are ranked; the copy skips it)
+  // (the selection fills all of them; should a caller rewrite the scores meanwhile and a key be read twice, one left over is
+  // skipped by the copy instead of becoming an address)
   for (int j = threadIdx.x; j < keff; j += kSelThreads) s_idx[j] = -1;
   const SelShape sh = {g.NC, g.L, g.C, g.n_sink, g.n_recent};
   sm100::pdl_wait();                                 // the scores are complete
