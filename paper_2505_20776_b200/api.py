@@ -1,6 +1,7 @@
 """Thin binding of the C ABI declared in include/specext.h.
 
-The functions here carry the same names as the C entry points and only marshal arguments
+The functions here carry the names of the C entry points (select_gather_flat is specext_select_gather for scores that are
+part of a larger buffer) and only marshal arguments
 (device pointers, strides, the current CUDA stream; the calls of a decoding step through the extension
 module built from csrc/binding.cpp, the others through ctypes); every step of the path runs in the
 library's kernels.  There is no CPU fallback: if the shared library is missing or a tensor is not on a CUDA
@@ -84,6 +85,8 @@ def _binding():
         path = _build.BINDING_PATH
         if not os.path.exists(path):
             raise RuntimeError(f"{path} is missing: run `python -m paper_2505_20776_b200.build`")
+        if not _build.binding_fits(path):
+            raise RuntimeError(f"{path} was built for another torch or Python: run `python -m paper_2505_20776_b200.build`")
         spec = importlib.util.spec_from_file_location(__package__ + "._binding", path)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)

@@ -60,16 +60,28 @@ def _compile(lib: str, sources, defines, verbose: bool) -> str:
     return _run(cmd, lib, verbose)
 
 
+def binding_tag() -> str:
+    """What the extension module is compiled against: its code depends on the layout of torch's and Python's objects."""
+    import torch
+    return f"specext binding for torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def binding_fits(path: str = BINDING_PATH) -> bool:
+    """Whether the module at `path` was built against the torch and the Python that run now (it carries its tag)."""
+    with open(path, "rb") as f:
+        return (binding_tag() + "\0").encode() in f.read()
+
+
 def build_binding(force: bool = False, verbose: bool = False) -> str:
     """Builds the extension module against the installed torch and returns its path."""
     src = os.path.join(CSRC, "binding.cpp")
-    if not force and not _stale(BINDING_PATH, [src]):
+    if not force and not _stale(BINDING_PATH, [src]) and binding_fits():
         return BINDING_PATH
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(nvcc_path())) if os.path.isabs(nvcc_path()) else "/usr/local/cuda"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-o", BINDING_PATH, src,
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DSPX_BUILT_FOR="{binding_tag()}"',
            "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(root, "include"),
            "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"), "-I" + os.path.join(cuda, "include"),
            "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
@@ -77,11 +89,11 @@ def build_binding(force: bool = False, verbose: bool = False) -> str:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Builds libspecext.so (and the extension module) next to this file and returns its path."""
+    """Builds libspecext.so, then the extension module, next to this file and returns the library's path."""
+    if force or needs_build():
+        _compile(LIB_PATH, SOURCES, [], verbose)
     build_binding(force, verbose)
-    if not force and not needs_build():
-        return LIB_PATH
-    return _compile(LIB_PATH, SOURCES, [], verbose)
+    return LIB_PATH
 
 
 def build_testing(force: bool = False, verbose: bool = False) -> str:

@@ -300,4 +300,12 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, kMethods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding() { return PyModule_Create(&kModule); }
+// (SPX_BUILT_FOR: the torch and the Python whose headers this was compiled with; the module is loaded by no other)
+PyMODINIT_FUNC PyInit__binding() {
+  PyObject* m = PyModule_Create(&kModule);
+  if (m && PyModule_AddStringConstant(m, "built_for", SPX_BUILT_FOR) != 0) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}
