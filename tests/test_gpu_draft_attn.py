@@ -12,7 +12,9 @@ import torch
 from oracle import specext_oracle as orc
 from paper_2505_20776_b200 import api
 from tests.guards import GuardedHotPath
+from tests.test_gpu_dispatch import launches
 from tests.test_gpu_parity import LSE_ATOL, O_ATOL, RECORD
+from tests.testing_lib import tuned
 from tests.util import bf16_bits, f64
 from workloads import synth
 
@@ -49,9 +51,14 @@ SHAPES = [
     (12, 12, 64, 1, "chain", 1024),            # 68M-class heads, plain decode step, 1K working cache
     (12, 12, 64, 8, "uniform", 1024),          # 68M-class, a small tree
     (32, 8, 128, 1, "chain", 2048),            # EAGLE-class single layer (the target's layer shape), decode
-    (32, 8, 128, 12, "uniform", 2048),         # EAGLE-class, small tree: 48 stacked rows -> one-CTA kernel
-    (32, 8, 128, 60, "levels", 2048),          # EAGLE-class, a full 60-node tree: 240 rows -> paired kernel
-    (32, 8, 128, 100, "uniform", 1024),        # a tree of more than 64 nodes: two row blocks
+    (32, 8, 128, 12, "uniform", 2048),         # EAGLE-class, small tree: 48 stacked rows
+    (32, 8, 128, 60, "levels", 2048),          # EAGLE-class, a full 60-node tree: 240 rows, two row blocks
+    (32, 8, 128, 100, "uniform", 1024),        # a tree of more than 64 nodes: four row blocks
+]
+# (all of these are clusters that merge by themselves; the forms with a merge kernel below)
+SPLIT_SHAPES = [
+    (32, 8, 128, 60, "levels", 8192),          # paired kernel: both CTAs clear the tail of a ragged tile, runs without a tile
+    (32, 8, 128, 1, "chain", 16384),           # one-CTA kernel, workers across problems
 ]
 
 
@@ -87,6 +94,21 @@ def test_draft_attn_lengths_on_device(cuda_device, Hq, Hkv, D, T, tree, cap):
     assert side.hp.read_status() == 0
     O_ref, _, _ = _oracle(t_cpu, t_cpu["K_prefix"], t_cpu["V_prefix"], cap, parent)
     assert np.abs(f64(side.hp.O) - O_ref).max() <= O_ATOL
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,tree,cap", SPLIT_SHAPES)
+def test_draft_attn_lengths_on_device_with_a_merge_kernel(cuda_device, Hq, Hkv, D, T, tree, cap):
+    assert launches(cuda_device, Hq, Hkv, D, T, cap, n_tokens=cap) == 2
+    test_draft_attn_lengths_on_device(cuda_device, Hq, Hkv, D, T, tree, cap)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,tree,cap", SHAPES)
+def test_draft_attn_lengths_on_device_without_clusters(cuda_device, Hq, Hkv, D, T, tree, cap):
+    """The same shapes as workers that leave partial results (the device may hold no clusters), and as one launch."""
+    assert launches(cuda_device, Hq, Hkv, D, T, cap, n_tokens=cap) == 1
+    with tuned(3, 0):
+        assert launches(cuda_device, Hq, Hkv, D, T, cap, n_tokens=cap) == 2
+        test_draft_attn_lengths_on_device(cuda_device, Hq, Hkv, D, T, tree, cap)
 
 
 def test_select_gather_draft_attn_chain_in_one_graph(cuda_device):

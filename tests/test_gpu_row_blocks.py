@@ -4,6 +4,7 @@ import pytest
 
 from tests.test_gpu_parity import check_attn, make_hp
 from tests.test_gpu_prefill import _compare, _inputs, _run
+from tests.testing_lib import tuned
 from workloads import synth
 
 pytestmark = pytest.mark.gpu
@@ -46,3 +47,18 @@ def test_prefill_wide_groups(cuda_device, G):
 def test_chunk_scores_in_groups_of_eight(cuda_device, Hq, Hkv, D, T, L, C):
     w = synth.Workload("score8", Hq, Hkv, D, L, T, C, 4, "uniform", "needle", seed=T + C)
     check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, C)
+
+
+@pytest.mark.parametrize("C", [8, 16, 64, 128])
+@pytest.mark.parametrize("kernel,Hq,Hkv,D,T,L", [
+    (0, 2, 2, 128, 64, 700),       # one cluster per problem
+    (2, 2, 2, 128, 64, 700),       # workers that leave partial results
+    (2, 8, 2, 128, 60, 1000),      # two row blocks of the one-CTA kernel
+    (0, 160, 160, 64, 5, 515),     # several segments per worker
+    (0, 32, 8, 128, 60, 3001),     # paired kernel
+])
+def test_chunk_sums_of_every_class(cuda_device, kernel, Hq, Hkv, D, T, L, C):
+    """Chunks of fewer than 32 keys, of 64 and of 128, whose sums the kernels store in three ways."""
+    w = synth.Workload("chunks", Hq, Hkv, D, L, T, C, 4, "uniform", "needle", seed=C + L)
+    with tuned(kernel, 0):
+        check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, C)
