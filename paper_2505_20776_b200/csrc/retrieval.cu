@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
 __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32_t* s_idx, int keff) {
   const int vpr = g.D / 8, vpt = g.H * vpr;                        // vectors per head row, token
   const long long vpc = (long long)g.C * vpt;                      // per chunk of the compact cache
-  // segments per chunk (which may be longer than the prefix)
-  const uint32_t spc = (uint32_t)(((long long)min(g.C, g.L) * vpt + 63) / 64);
+  // segments per chunk, which may be longer than the prefix (the vectors that exist in a layer fit 32 bits: 64 GB)
+  const uint32_t spc = ((uint32_t)min(g.C, g.L) * (uint32_t)vpt + 63) / 64;
   const uint32_t n_seg = 2u * g.n_layers * keff * spc;
   const bool contiguous = g.s_h == g.D && g.s_l == (long long)g.H * g.D;
   const int lane = threadIdx.x & 31;
@@ -256,7 +256,10 @@ __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32
         const uint32_t which = part / (uint32_t)g.n_layers, layer = part - which * g.n_layers;
         const int c = s_idx[i];
         // vectors of the chunk from here on, as far as this segment goes
-        if (c >= 0 && c < g.NC) lim[q] = (int)max(0ll, min((long long)min(g.C, g.L - c * g.C) * vpt - w0, 64ll));
+        if (c >= 0 && c < g.NC) {
+          const uint32_t total = (uint32_t)min(g.C, g.L - c * g.C) * (uint32_t)vpt;
+          lim[q] = w0 < total ? (int)min(total - w0, 64u) : 0;
+        }
         const __nv_bfloat16* base = g.src[which] + (long long)layer * g.s_layer + (long long)c * g.C * g.s_l;
         dst[q] = reinterpret_cast<uint4*>(g.dst[which]) + ((long long)layer * g.max_selected + i) * vpc + w0 + lane;
         if (contiguous) {
