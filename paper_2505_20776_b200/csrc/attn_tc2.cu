@@ -151,7 +151,8 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
   // come by plain loads like those of every later segment.)
   constexpr bool dev_len = DEVLEN;
   // With many tiles per worker a second tile is asked for in L2 and four instead of two tiles are requested at the start:
-  // 8K 16.7 -> 16.5 us a call, 16K 22.5 -> 22.3, 32K 33.7 -> 33.4; with three or four tiles 0.1 us slower.
+  // 8K 16.7 -> 16.5 us a call replayed, 16K 22.5 -> 22.3, 32K 35.3 -> 35.1; launched one by one within what runs
+  // differ; with three or four tiles 0.1 us slower.
   const bool many = unit_hi - unit_lo >= 6;
   if (warp == kProducerWarp && lane == 0 && unit_lo < unit_hi && !dev_len) {
     const int prob = unit_lo / p.UPP;

@@ -14,6 +14,11 @@
 // range that lies inside one problem is a "segment" and yields one partial result (unnormalised
 // output, running maximum, row sum) in slot c + problem.  Slots are unique because both c and the
 // problem index are non-decreasing along the line.
+//
+// With cluster > 0 the cpp = cluster workers of a problem (CTAs, one segment each) are one thread-block
+// cluster that merges its results itself: through shared memory, or through the same part of the
+// workspace, where CTA k of problem b then owns entry b * cluster + k ([D/4][128 rows] of float4, and
+// (maximum, row sum) pairs): n_cta entries, no merge kernel.
 #ifndef SPECEXT_PLAN_H_
 #define SPECEXT_PLAN_H_
 
@@ -42,7 +47,7 @@ struct AttnPlan {
   int cluster;     // > 0: the cpp workers of a problem are one cluster of this many CTAs and merge among themselves
   int cpp;         // workers per problem, or 0 when the line of units is cut without regard to problems
   int q, rem;      // cpp > 0: UPP = q*cpp + rem;  cpp == 0: U = q*n_cta + rem
-  int n_slots;     // n_cta + NP - 1 partial slots
+  int n_slots;     // partial slots: n_cta + NP - 1, or n_cta with clusters
   int max_segs;    // upper bound on segments per problem
   int CPT;         // chunks per key tile = 128 / C
   int NC;          // ceil(L/C)

@@ -1,7 +1,8 @@
 // Hybrid Tree Attention with one CTA per worker, on the pipeline of core.cuh: split-over-KV partial attention of the
 // stacked (query head x tree node) rows of one KV head, in row blocks of 128, against 128-key tiles of the prefix and the
-// tree.  Taken for head_dim 64 and for at most 128 stacked rows: targets without grouped heads, single-token steps, draft
-// models.  (More rows with head_dim 128 go to the pairs of attn_tc2.cu.)
+// tree.  Taken for head_dim 64, for at most 128 stacked rows (targets without grouped heads, single-token steps, draft models)
+// and, in clusters, for more rows on short prefixes.  (Longer ones with head_dim 128 and more than 128 rows go to the pairs of
+// attn_tc2.cu; the line is drawn at cluster_size in api.cu.)
 //
 // A worker owns a range of (problem, key tile) units; the part of the range inside one problem is a segment and ends with
 // one partial result (unnormalised O, reference maximum, row sum) in the workspace.
@@ -77,8 +78,11 @@ struct VerifyWork {
 // another CTA takes stores at ~20 GB/s, 64 KB of 128 rows in 3 us, and shared-memory room needs the second meeting; L2
 // costs two of its latencies.  us per call, by shared memory / by L2: 4 rows on 2K 8.0 / 8.5, 12 x 64 heads with 8 rows
 // 7.4 / 7.6, 10 rows of 32 KV heads 10.2 / 10.1, 40 rows 8.3 / 7.6, 120 rows at 8K 17.2 / 15.9, 240 rows at 1K 10.6 / 9.7.
-// (Bulk copies between the CTAs instead of stores were slower than either: 8.8, 7.7, 10.5, 8.1, 17.7, 11.2.)  Each is an
-// instantiation of its own: with both in one kernel a call was 0.1 to 0.3 us longer.
+// (Bulk copies between the CTAs instead of stores were slower than either: 8.8, 7.7, 10.5, 8.1, 17.7, 11.2.)  The other way
+// round where the tiles are many: 60 rows of 32 KV heads at 8K are 0.5 us shorter through shared memory.  Each is an
+// instantiation of its own: with both in one kernel a call was 0.1 to 0.3 us longer.  The forms through shared memory spill
+// for head_dim 128 and for the device-side length (8 to 16 bytes of stack, 312 to 348 bytes of reloads), in the exchange; those
+// through L2 do not.
 struct MergeCtx {
   int cs, rank;            // CTAs of the cluster, this one
   int prob, g, rblk;       // the problem

@@ -253,9 +253,9 @@ def test_edge_shapes(cuda_device, Hq, Hkv, D, L, T, C):
 
 
 @pytest.mark.parametrize("Hq,Hkv,D,L,T,C,tree", [
-    (32, 8, 128, 1000, 100, 32, "uniform"),   # 400 stacked rows: two row blocks on the paired kernel
+    (32, 8, 128, 1000, 100, 32, "uniform"),   # 400 stacked rows
     (32, 8, 128, 700, 128, 32, "levels"),     # the largest tree
-    (4, 4, 128, 300, 128, 32, "chain"),       # one query head per KV head, head_dim 128: 256-row blocks, a 128-deep chain
+    (4, 4, 128, 300, 128, 32, "chain"),       # one query head per KV head, head_dim 128: a 128-deep chain
     (4, 4, 64, 300, 128, 16, "chain"),        # head_dim 64: the one-CTA kernel with two mask words per node
     (8, 2, 64, 200, 65, 32, "uniform"),
     (8, 2, 128, 0, 90, 32, "chain"),          # tree only: node i sees exactly nodes 0..i, across both mask words
