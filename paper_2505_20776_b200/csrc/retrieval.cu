@@ -233,19 +233,19 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Gat
 // longer than the copy.
 __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32_t* s_idx, int keff) {
   const int vpr = g.D / 8, vpt = g.H * vpr;                        // vectors per head row, token
-  const long long vpc = (long long)g.C * vpt;                      // per chunk of the compact cache
+  const unsigned long long vpc = (unsigned long long)g.C * vpt;    // per chunk of the compact cache
   // segments per chunk, which may be longer than the prefix (the vectors that exist in a layer fit 32 bits: 64 GB)
   const uint32_t spc = ((uint32_t)min(g.C, g.L) * (uint32_t)vpt + 63) / 64;
   const uint32_t n_seg = 2u * g.n_layers * keff * spc;
   const bool contiguous = g.s_h == g.D && g.s_l == (long long)g.H * g.D;
-  const int lane = threadIdx.x & 31;
+  const uint32_t lane = threadIdx.x & 31;
   const uint32_t n_warps = gridDim.x * (blockDim.x / 32);
   // warps of different blocks next to each other in the line, so that a short line keeps every SM busy
   const uint32_t first = (threadIdx.x / 32) * gridDim.x + blockIdx.x;
   for (uint32_t s0 = first; s0 < n_seg; s0 += 4 * n_warps) {
     uint4 x[4][2];
     uint4* dst[4];
-    int lim[4];
+    uint32_t lim[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint32_t s = s0 + q * n_warps;
@@ -255,13 +255,14 @@ __device__ __forceinline__ void gather_segments(const GatherArgs& g, const int32
         const uint32_t part = chunk / (uint32_t)keff, i = chunk - part * keff;
         const uint32_t which = part / (uint32_t)g.n_layers, layer = part - which * g.n_layers;
         const int c = s_idx[i];
-        // vectors of the chunk from here on, as far as this segment goes
+        // vectors of the chunk from here on
         if (c >= 0 && c < g.NC) {
           const uint32_t total = (uint32_t)min(g.C, g.L - c * g.C) * (uint32_t)vpt;
-          lim[q] = w0 < total ? (int)min(total - w0, 64u) : 0;
+          lim[q] = total - min(total, w0);
         }
         const __nv_bfloat16* base = g.src[which] + (long long)layer * g.s_layer + (long long)c * g.C * g.s_l;
-        dst[q] = reinterpret_cast<uint4*>(g.dst[which]) + ((long long)layer * g.max_selected + i) * vpc + w0 + lane;
+        const uint32_t row = layer * g.max_selected + i;             // (at most 65535 layers x 1024 chunks)
+        dst[q] = reinterpret_cast<uint4*>(g.dst[which]) + row * vpc + w0 + lane;
         if (contiguous) {
           const uint4* src = reinterpret_cast<const uint4*>(base) + w0 + lane;
 #pragma unroll
