@@ -128,8 +128,8 @@ int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
 }
 
 // Size of the cluster whose CTAs share the key tiles of a problem and merge among themselves, or 0 for workers that leave
-// partial results to the merge kernel.
-int cluster_size(const AttnPlan& p, bool pair) {
+// partial results to the merge kernel.  dev_len: the prefix length is on the device (a draft call).
+int cluster_size(const AttnPlan& p, bool pair, bool dev_len) {
   const long long np = (long long)p.Hkv * ((p.rows + 127) / 128);
   int dev = -1, size = 0;
   if (np > sm_count() / 2) return 0;
@@ -147,7 +147,7 @@ int cluster_size(const AttnPlan& p, bool pair) {
   // 9.4 / 9.2 / 9.6, 100 nodes of 16 query / 2 KV heads 9.0 / 9.2 / 9.9, of 32 KV heads 12.4 / 10.0 / 10.5; but 60 nodes of
   // 32 KV heads (60 rows) 10.5 / 9.0 / 8.9, 100 nodes of 64 query / 8 KV heads (56 problems) 14.5 / 12.6 / 11.5, of 64 KV
   // heads 17.1 / 12.2 / 11.0.  (Between them 40 problems take 1.08 of the split form's time, 50 0.95.)
-  if (p.UPP == 2 && p.D == 128 && p.rows > 64 && np <= 40) return 0;
+  if (p.UPP == 2 && p.D == 128 && p.rows > 64 && np <= 40 && !dev_len) return 0;
   const int tiles = (p.UPP + size - 1) / size;
   int split;
   if (pair) {
@@ -173,13 +173,15 @@ int cluster_size(const AttnPlan& p, bool pair) {
   //   their merge takes a second wave of blocks (256 threads: 32 query / 4 KV heads, 80 nodes at 5K 17.1 / 14.9, scored
   //   20.5 / 18.2; 512 threads: 64 query / 8 KV heads, 80 nodes at 5K 22.2 / 21.6, scored 26.8 / 25.9), which two segments a
   //   row make up for sooner (100 nodes at 2K 18.0 / 17.6 with 9 tiles, 3K 21.0 / 21.2 with 13);
+  //   a draft call goes there (the pairs' form with the length on the device is another 2 us longer: 60 nodes of 64 query
+  //   heads in a cache of 4096 19.1 / 17.0 with 9 tiles, 100 nodes of 16 / 2 heads in 16384 24.6 / 21.6 with 15);
   //   without scores also a cluster of more than 8 CTAs (100 nodes of 16 query / 2 KV heads at 8K 15.8 / 15.1 with 8 tiles,
   //   scored 19.5 / 20.3).
   int limit = 0;
   if (pair) {
     const int np2 = p.Hkv * ((p.rows + 255) / 256), per = sm_count() / 2 / np2;      // (np2 <= np <= half of the SMs)
     const bool second_wave = 8 * np2 * (per > 4 ? 2 : 1) > sm_count();
-    limit = tiles < split || (second_wave && per > 2) ? 16 : second_wave || (!p.want_score && size > 8) ? 11 : 6;
+    limit = dev_len || tiles < split || (second_wave && per > 2) ? 16 : second_wave || (!p.want_score && size > 8) ? 11 : 6;
     if (p.want_score && p.C < 32) limit = 16;                                         // (see below)
   }
   int most = pair ? (tiles <= limit ? (split > 3 ? split : 3) : 0)
@@ -201,7 +203,8 @@ int cluster_size(const AttnPlan& p, bool pair) {
   return size;
 }
 
-int build_plan(const specext_attn_desc* d, AttnPlan* out) {
+// (The workspace is that of the split form whatever dev_len is: the clusters' is never larger.)
+int build_plan(const specext_attn_desc* d, AttnPlan* out, bool dev_len = false) {
   if (!d) return SPECEXT_ERR_INVALID_ARG;
   if (d->n_q_heads < 1 || d->n_kv_heads < 1 || d->n_q_heads % d->n_kv_heads != 0) return SPECEXT_ERR_INVALID_ARG;
   if (d->prefix_len < 0 || d->prefix_len > (1 << 24)) return SPECEXT_ERR_INVALID_ARG;
@@ -234,7 +237,7 @@ int build_plan(const specext_attn_desc* d, AttnPlan* out) {
   const bool pair = p.D == 128 && p.rows > 128 && want != 2;
   int rc = lay_out(&p, want == 1 ? 1 : (pair ? 3 : 2), pair ? 256 : 128, 0);
   if (rc != SPECEXT_OK) return rc;
-  const int size = want == 0 && tuning_min_units() == 1 ? cluster_size(p, pair) : 0;
+  const int size = want == 0 && tuning_min_units() == 1 ? cluster_size(p, pair, dev_len) : 0;
   if (size > 0) {
     // (the workspace keeps its size: it does not depend on what clusters the device holds)
     const long long split_floats = p.total_floats;
@@ -284,7 +287,7 @@ int run_attn(const specext_attn_desc* desc, const void* Q, const void* K_prefix,
              void* O, float* lse, float* chunk_score, void* workspace, size_t workspace_bytes,
              int32_t* device_status, void* cuda_stream) {
   AttnArgs a;
-  const int rc = build_plan(desc, &a.plan);
+  const int rc = build_plan(desc, &a.plan, prefix_len_dev != nullptr);
   if (rc != SPECEXT_OK) return rc;
   const AttnPlan& p = a.plan;
   if (prefix_len_dev && (p.want_score || p.kernel == 1 || (reinterpret_cast<uintptr_t>(prefix_len_dev) & 3u) != 0))

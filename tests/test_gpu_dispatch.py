@@ -65,3 +65,10 @@ def test_many_tiles_go_to_the_pairs(cuda_device, Hq, Hkv, T, L, scored, want):
 ])
 def test_prefix_of_one_tile(cuda_device, Hq, Hkv, D, T, L, want):
     assert launches(cuda_device, Hq, Hkv, D, T, L) == want
+
+
+@pytest.mark.parametrize("Hq,Hkv,T,cap", [(64, 8, 60, 4096), (32, 8, 100, 4096), (16, 2, 100, 16384), (32, 8, 60, 128)])
+def test_draft_calls_stay_in_clusters(cuda_device, Hq, Hkv, T, cap):
+    """Shapes that verification takes to the pairs; the workspace is the same for both."""
+    assert launches(cuda_device, Hq, Hkv, 128, T, cap) == 2
+    assert launches(cuda_device, Hq, Hkv, 128, T, cap, n_tokens=cap) == 1
