@@ -146,7 +146,8 @@ int cluster_size(const AttnPlan& p, bool pair, bool dev_len) {
   // merge kernel takes, unless the problems are many.  us per call, before clusters / split / cluster, 100 tokens: 60 nodes
   // 9.4 / 9.2 / 9.6, 100 nodes of 16 query / 2 KV heads 9.0 / 9.2 / 9.9, of 32 KV heads 12.4 / 10.0 / 10.5; but 60 nodes of
   // 32 KV heads (60 rows) 10.5 / 9.0 / 8.9, 100 nodes of 64 query / 8 KV heads (56 problems) 14.5 / 12.6 / 11.5, of 64 KV
-  // heads 17.1 / 12.2 / 11.0.  (Between them 40 problems take 1.08 of the split form's time, 50 0.95.)
+  // heads 17.1 / 12.2 / 11.0.  (Between them 40 problems take 1.08 of the split form's time, 50 0.95.  Draft calls stay: their
+  // split form is longer, see below.)
   if (p.UPP == 2 && p.D == 128 && p.rows > 64 && np <= 40 && !dev_len) return 0;
   const int tiles = (p.UPP + size - 1) / size;
   int split;
@@ -195,7 +196,7 @@ int cluster_size(const AttnPlan& p, bool pair, bool dev_len) {
     int most_small;
     if (pair) most_small = tiles <= (p.C == 16 ? 12 : 5) ? split : 0;    // 4 keys: 7 against 7 0.3 to 9 % slower, 12 1 to 11 %
     else most_small = tiles <= 4 && (size > 8 || split >= 3) ? 4 : p.D == 64 ? split : split * 6 / 5;
-    if (most_small < 2 && p.C >= 4) most_small = 2;      // (a key or two: 60 nodes at 1K 36.2 before, 43.9 in clusters with two)
+    if (most_small < 2 && p.C >= 4) most_small = 2;      // (a key or two: 60 nodes at 1K 35.4 before, 43.2 in clusters)
     if (most > most_small) most = most_small;
   }
   if (tiles > most) return 0;
