@@ -26,8 +26,10 @@
 // always reach the final cluster barrier before tensor memory is freed.
 //
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory
-// allocation and the start-up cluster barrier run while the kernel before it in the stream finishes;
-// global memory is touched only after griddepcontrol.wait.
+// allocation and the start-up cluster barrier run while the kernel before it in the stream finishes.  Each role waits for
+// that kernel just before its own first read or write of global memory; the first K/V tiles are asked for in L2 ahead of the
+// wait (one scored call with its retrieval at 50K 49.9 -> 48.9 us, at 4K 23.7 -> 23.5; no change where the power limit sets
+// the pace).
 #include "common.cuh"
 #include "pair.cuh"
 #include "tmap.h"
@@ -130,66 +132,24 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     fence_mbar_init();
   }
   cluster_arrive();
-  // The kernel after this one (the merge) may be set up while this one runs; this one touches global
-  // memory only once the kernel before it has completed (its set-up so far has used none).
+  // The kernel after this one (the merge) may be set up while this one runs; this one reads and writes global
+  // memory only once the kernel before it has completed: each role that does waits for that itself.
   pdl_launch_dependents();
-  if (warp != kMmaWarp) pdl_wait();
 
   const uint32_t rank = cluster_rank();
   const int cl = blockIdx.x >> 1;                        // the plan's "CTA" index is the cluster index
   const int unit_lo = spx_unit_start(p, cl), unit_hi = spx_unit_start(p, cl + 1);
-
-  // The first segment's Q rows are requested before anything else, into a shared-memory scratch, so
-  // that their latency runs under the set-up instead of delaying the first S MMA.  The scratch holds
-  // the CTA's 128 rows twice 64 elements (warpgroup 0 reads the first 64 elements of a row, warpgroup
-  // 1 the rest), 128 bytes per row with the 16-byte chunks XOR-swizzled by the row (the TMA 128-byte
-  // swizzle), so that the per-row reads are conflict-free.  It is the tail of the V ring, which the
-  // producer leaves alone until the first S MMA is done.  One thread fetches it with two TMA boxes
-  // of 64 elements x G heads x 128/G nodes: exactly the stacked rows (G is a power of two), rows
-  // past the tree zero-filled.
-  // (With a device-side prefix length the first segment may turn out to be empty; its Q rows then
-  // come by plain loads like those of every later segment.)
   constexpr bool dev_len = DEVLEN;
   // With many tiles per worker a second tile is asked for in L2 and four instead of two tiles are requested at the start:
   // 8K 16.7 -> 16.5 us a call replayed, 16K 22.5 -> 22.3, 32K 35.3 -> 35.1; launched one by one within what runs
   // differ; with three or four tiles 0.1 us slower.
   const bool many = unit_hi - unit_lo >= 6;
-  if (warp == kProducerWarp && lane == 0 && unit_lo < unit_hi && !dev_len) {
-    const int prob = unit_lo / p.UPP;
-    const int g = prob / p.n_rblk, rblk = prob - g * p.n_rblk;
-    const int t0 = (rblk * p.RB + (int)rank * 128) / p.G;
-    unsigned char* scratch = ring + (2 * kStages - 2) * kStageBytes;
-    mbar_arrive_expect_tx(&ctl->q_land, 2 * kStageBytes);
-    tma_load_3d(scratch, &maps.q, &ctl->q_land, 0, g * p.G, t0);
-    tma_load_3d(scratch + kStageBytes, &maps.q, &ctl->q_land, 64, g * p.G, t0);
-    // The first K/V tiles can only be loaded once the pair's barriers are known to exist (a cluster
-    // barrier away); until then their halves are at least pulled into L2.
-    for (int i = 0; i < (many ? 2 : 1); ++i) {
-      const int tile = unit_lo - prob * p.UPP + i;
-      if (tile > p.TPH) break;
-      const bool is_tree = tile == p.TPH;
-      const int key0 = is_tree ? 0 : tile * SPX_TILE_KEYS;
-      const CUtensorMap* mk = is_tree ? &maps.kt : &maps.kp;
-      tma_prefetch_3d(mk, 0, g, key0 + 64 * rank);
-      tma_prefetch_3d(mk, 64, g, key0 + 64 * rank);
-      tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * rank, g, key0);
-    }
-  }
-
-  if (warp == kProducerWarp && lane == 0) {
-    prefetch_tensormap(&maps.q);
-    prefetch_tensormap(&maps.kp);
-    prefetch_tensormap(&maps.vp);
-    prefetch_tensormap(&maps.kt);
-    prefetch_tensormap(&maps.vt);
-  }
   if (warp == kMmaWarp) {
     // tensor memory for the pair: both CTAs' warps with this index allocate all 512 columns
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                  "r"(512u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    pdl_wait();
   }
   bool ok = true;
 
@@ -197,6 +157,25 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     // ================================ TMA producer (each CTA loads its halves) ===============
     setmaxnreg_dec<kRegsOther>();
     cluster_wait();                        // both CTAs' barriers exist
+    pdl_wait();
+    if (lane == 0 && unit_lo < unit_hi && !dev_len) {
+      // The first segment's Q rows are requested before anything else, into a shared-memory scratch.  It holds
+      // the CTA's 128 rows twice 64 elements (warpgroup 0 reads the first 64 elements of a row, warpgroup
+      // 1 the rest), 128 bytes per row with the 16-byte chunks XOR-swizzled by the row (the TMA 128-byte
+      // swizzle), so that the per-row reads are conflict-free.  It is the tail of the V ring, which the
+      // producer leaves alone until the first S MMA is done.  One thread fetches it with two TMA boxes
+      // of 64 elements x G heads x 128/G nodes: exactly the stacked rows (G is a power of two), rows
+      // past the tree zero-filled.
+      // (With a device-side prefix length the first segment may turn out to be empty; its Q rows then
+      // come by plain loads like those of every later segment.)
+      const int prob = unit_lo / p.UPP;
+      const int g = prob / p.n_rblk, rblk = prob - g * p.n_rblk;
+      const int t0 = (rblk * p.RB + (int)rank * 128) / p.G;
+      unsigned char* scratch = ring + (2 * kStages - 2) * kStageBytes;
+      mbar_arrive_expect_tx(&ctl->q_land, 2 * kStageBytes);
+      tma_load_3d(scratch, &maps.q, &ctl->q_land, 0, g * p.G, t0);
+      tma_load_3d(scratch + kStageBytes, &maps.q, &ctl->q_land, 64, g * p.G, t0);
+    }
     if (lane == 0) {
       uint32_t kp = 0, vp = 0;
       const uint64_t stream_once = policy_evict_first();
@@ -367,6 +346,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     if (warp == kTreeWarp) {
       // registers first: the softmax warpgroups cannot grow until every warp of this warpgroup has shrunk
       setmaxnreg_dec<kRegsOther>();
+      pdl_wait();
 #pragma unroll
       for (int q = 0; q < kSpxMaxTree / 32; ++q) ctl->parent[lane + 32 * q] = lane + 32 * q < p.T ? a.parent[lane + 32 * q] : -1;
       __syncwarp();
@@ -395,6 +375,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     if (warp == kMmaWarp) {
       // ================================ issuer of S = Q K^T (leader CTA) =====================
       setmaxnreg_dec<kRegsOther>();
+      if (DEVLEN) pdl_wait();
       if (lane == 0 && rank == 0) {
         const uint32_t idesc_s = idesc_bf16_f32(256, SPX_TILE_KEYS, false, false);
         constexpr uint32_t hi = desc_hi(1024);
@@ -435,6 +416,23 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     } else if (warp == kPvWarp) {
       // ================================ issuer of O += P V (leader CTA) ======================
       setmaxnreg_dec<kRegsOther>();
+      if (lane == 0 && unit_lo < unit_hi && !dev_len) {
+        // The first K/V tiles are asked for in L2 ahead of the dependency wait, by a thread that has nothing else to do.  A
+        // prefetch changes no result: what the kernel before may still write to these lines goes through L2 as well.
+        const int prob = unit_lo / p.UPP;
+        const int g = prob / p.n_rblk;
+        for (int i = 0; i < (many ? 2 : 1); ++i) {
+          const int tile = unit_lo - prob * p.UPP + i;
+          if (tile > p.TPH) break;
+          const bool is_tree = tile == p.TPH;
+          const int key0 = is_tree ? 0 : tile * SPX_TILE_KEYS;
+          const CUtensorMap* mk = is_tree ? &maps.kt : &maps.kp;
+          tma_prefetch_3d(mk, 0, g, key0 + 64 * rank);
+          tma_prefetch_3d(mk, 64, g, key0 + 64 * rank);
+          tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * rank, g, key0);
+        }
+      }
+      if (DEVLEN) pdl_wait();
       if (lane == 0 && rank == 0) {
         const uint32_t idesc_o = idesc_bf16_f32(256, D, false, true);
         constexpr uint32_t hi = desc_hi(1024);
@@ -496,6 +494,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
       uint32_t n_oth = 0;        // tiles the other warpgroup had been given before the current segment
       int seg = 0;
       bool anc_seen = false;
+      pdl_wait();
       const int L_eff = DEVLEN ? spx_prefix_len(a) : p.L;
       const int tph_eff = DEVLEN ? (L_eff + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS : p.TPH;
       for (int u = unit_lo; u < unit_hi && ok;) {

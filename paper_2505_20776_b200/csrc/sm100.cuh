@@ -73,9 +73,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 // ---- TMA ----------------------------------------------------------------------------------
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
-}
 // 3-D tiled load global -> shared of this CTA, completion counted in bytes on `bar`.
 // Coordinate c0 (innermost) times the element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1,

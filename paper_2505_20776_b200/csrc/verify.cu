@@ -23,8 +23,12 @@
 // threads reach the final barrier before tensor memory is freed.
 //
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory allocation and the
-// start-up barrier run while the kernel before it in the stream finishes; global memory is touched only after
-// griddepcontrol.wait.
+// start-up barrier run while the kernel before it in the stream finishes.  Each role waits for that kernel just before its own
+// first read or write of global memory, with the place of its first tile worked out, and the first tiles are asked for in L2
+// ahead of the wait.  Between the release and the request for the first K tile 1.2 to 2.0 us went by when all threads waited
+// at one place and the producer asked for L2 itself, now 0.5; us per pass, launched one by one: four layers at 1K with scores
+// and retrieval 53.0 -> 50.0, two layers of 12 x 64 heads on a 1K cache 16.4 -> 15.8, four layers of 32 KV heads at 8K
+// 137.3 -> 135.0, eight layers of 64 query heads at 1.4K 111.1 -> 106.9.
 #include <atomic>
 
 #include "common.cuh"
@@ -304,33 +308,21 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const G geo(p.q_rows);
 
-  setup<1>(ctl, warp, lane);
   const int worker = blockIdx.x;
   const int unit_lo = spx_unit_start(p, worker), unit_hi = spx_unit_start(p, worker + 1);
-  // The kernel after this one may be set up while this one runs; this one touches global memory only once the kernel
-  // before it has completed.
+  setup<1>(ctl, warp, lane);
+  // The kernel after this one may be set up while this one runs; this one reads and writes global memory only once the kernel
+  // before it has completed: each role that does waits for that itself.
   pdl_launch_dependents();
-  pdl_wait();
-  if (warp == kProducerWarp && lane == 0 && unit_lo < unit_hi && !DEVLEN) {
-    // The first tile is asked for in L2 as well, in one piece for K and V ahead of the ring's loads: 8K prefix with 32 KV
-    // heads 28.5 -> 27.3 us, one node on 16K 20.5 -> 19.6.  The second one too where a worker has several: 16K 19.6 ->
-    // 19.3, 128K 88.3 -> 87.5, but 2K 8.1 -> 8.4.
-    const int prob = unit_lo / p.UPP, tile = unit_lo - prob * p.UPP, g = prob / p.n_rblk;
-    for (int i = 0; i < (unit_hi - unit_lo >= 6 ? 2 : 1); ++i) {
-      if (tile + i > p.TPH) break;
-      const bool is_tree = tile + i == p.TPH;
-      const int key0 = is_tree ? 0 : (tile + i) * SPX_TILE_KEYS;
-#pragma unroll
-      for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.kt : &maps.kp, 64 * ds, g, key0);
-#pragma unroll
-      for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * ds, g, key0);
-    }
-  }
-
-  const int L_eff = DEVLEN ? spx_prefix_len(a) : p.L;
-  const int tph_eff = DEVLEN ? (L_eff + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS : p.TPH;
-  VerifyWork<DEVLEN> work(p, unit_lo, unit_hi, tph_eff);
   bool ok = true;
+  int L_eff = p.L;
+  VerifyWork<DEVLEN> work(p, unit_lo, unit_hi, p.TPH);
+  auto read_length = [&]() {
+    if (DEVLEN) {
+      L_eff = spx_prefix_len(a);
+      work.tph_eff = (L_eff + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS;
+    }
+  };
 
   if (warp == kProducerWarp) {
     // ================================ TMA producer of K and V ================================
@@ -342,7 +334,14 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       unsigned char* vring = base + geo.v_off;
       int kst = 0, vst = 0;
       uint32_t kph = 1, vph = 1, n_rag = 0;
-      while (ok && work.next()) {
+      bool more = false;
+      if (!DEVLEN) more = work.next();                   // (worked out ahead of the wait)
+      pdl_wait();
+      if (DEVLEN) {
+        read_length();
+        more = work.next();
+      }
+      for (; ok && more; more = work.next()) {
         const int g = work.prob / p.n_rblk;
         for (int j = 0; j < work.n && ok; ++j) {
           const int tile = work.tile(j);
@@ -407,9 +406,32 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     }
   } else if (warp == kMmaWarp) {
     setmaxnreg_dec<kRegsOther>();
+    if (DEVLEN) {
+      pdl_wait();
+      read_length();
+    }
     if (lane == 0) ok = issue_s<1, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kPvWarp) {
     setmaxnreg_dec<kRegsOther>();
+    if (lane == 0 && unit_lo < unit_hi) {
+      // The first tile is asked for in L2 ahead of the dependency wait, by a thread that has nothing else to do yet; the second one
+      // too where a worker has several: 16K 19.6 -> 19.3, 128K 88.3 -> 87.5, but 2K 8.1 -> 8.4.  A prefetch changes no result:
+      // what the kernel before may still write to these lines goes through L2 as well.
+      const int prob = unit_lo / p.UPP, tile = unit_lo - prob * p.UPP, g = prob / p.n_rblk;
+      for (int i = 0; i < (unit_hi - unit_lo >= 6 ? 2 : 1); ++i) {
+        if (tile + i > p.TPH) break;
+        const bool is_tree = tile + i == p.TPH;
+        const int key0 = is_tree ? 0 : (tile + i) * SPX_TILE_KEYS;
+#pragma unroll
+        for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.kt : &maps.kp, 64 * ds, g, key0);
+#pragma unroll
+        for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * ds, g, key0);
+      }
+    }
+    if (DEVLEN) {
+      pdl_wait();
+      read_length();
+    }
     if (lane == 0) ok = issue_pv<1, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kTreeWarp) {
     // ================================ ancestor masks, TMA producer of Q =======================
@@ -417,14 +439,22 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     // boxes of 64 elements x G heads x q_rows/G nodes: exactly the stacked rows (G is a power of two), rows past the
     // tree zero-filled
     const uint32_t q_bar = smem_u32(&ctl->q_full);
-    auto load_q = [&]() {
-      const int g = work.prob / p.n_rblk, rblk = work.prob - g * p.n_rblk;
+    auto load_q = [&](int prob) {
+      const int g = prob / p.n_rblk, rblk = prob - g * p.n_rblk;
       arrive_expect_tx_cluster(q_bar, geo.q_blk * G::kBlocks);
 #pragma unroll
       for (int ds = 0; ds < G::kBlocks; ++ds)
         tma_load<1>(smem_u32(base + ds * geo.q_blk), &maps.q, q_bar, 64 * ds, g * p.G, rblk * p.RB / p.G);
     };
-    if (lane == 0 && work.next()) load_q();              // the first segment's; later ones below
+    // the first segment's; later ones below
+    bool any = false;
+    if (!DEVLEN) any = work.next();
+    pdl_wait();
+    if (DEVLEN) {
+      read_length();
+      any = work.next();
+    }
+    if (lane == 0 && any) load_q(work.prob);
     __syncwarp();
 #pragma unroll
     for (int q = 0; q < kSpxMaxTree / 32; ++q) ctl->parent[lane + 32 * q] = lane + 32 * q < p.T ? a.parent[lane + 32 * q] : -1;
@@ -443,7 +473,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     if (lane == 0) {
       for (uint32_t seg = 0; ok && work.next(); ++seg) {
         ok = wait_c(&ctl->q_empty, seg & 1, abort_flag);
-        if (ok) load_q();
+        if (ok) load_q(work.prob);
       }
     }
   } else {
@@ -464,6 +494,8 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     uint32_t t0 = 0, seg = 0;                            // tiles and segments before the current segment
     bool anc_seen = false;
     float m_loc, l;                                      // l is relative to m_loc
+    pdl_wait();
+    read_length();
     while (ok && work.next_any()) {
       const int prob = work.prob, g = prob / p.n_rblk, rblk = prob - g * p.n_rblk, n = work.n;
       const int r = rblk * p.RB + rr;
