@@ -71,7 +71,7 @@ int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
   p.kernel = kernel;
   p.cluster = cluster;
   p.RB = row_block;
-  p.q_rows = kernel == 2 && p.D == 128 && p.rows <= 64 ? 64 : 128;
+  p.q_rows = kernel != 2 || p.D != 128 || p.rows > 64 ? 128 : cluster > 0 && p.rows <= kSpxClusterRowsBySmem ? 32 : 64;
   p.n_rblk = (p.rows + p.RB - 1) / p.RB;
   p.NP = p.Hkv * p.n_rblk;
   const long long U = (long long)p.NP * p.UPP;

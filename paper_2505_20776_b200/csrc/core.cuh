@@ -51,11 +51,11 @@ struct Geo {
   static constexpr int kCtrlOffset = kWide ? 16384 + 6 * 32768 : kQBytes + 11 * 16384;
   int q_blk, nk, nv;
   uint32_t k_off, v_off;
-  // rows = 64 (only with one CTA, head_dim 128 and at most 64 stacked rows): Q takes half the room, which is one more
-  // stage.  The MMA still reads 128 rows; what lies behind the 64 is multiplied into rows nobody looks at.
+  // rows = 64 or 32 (only with one CTA, head_dim 128 and at most that many stacked rows): Q takes half the room or less, which
+  // is one more stage.  The MMA still reads 128 rows; what lies behind Q is multiplied into rows nobody looks at.
   __device__ __forceinline__ explicit Geo(int rows) {
     q_blk = rows * 128;
-    nk = kWide ? (rows == 64 ? 3 : 2) : 5;
+    nk = kWide ? (rows <= 64 ? 3 : 2) : 5;
     nv = kWide ? 3 : 6;
     k_off = q_blk * kBlocks;
     v_off = k_off + nk * kKStage;

@@ -77,12 +77,16 @@ struct VerifyWork {
 // for the same rows.  Each CTA passes its part on, the cluster meets, and each CTA adds up and writes its share of O.  How
 // depends on the number of rows of the call.
 //
-// Up to 32: through the other CTAs' shared memory (where Q and the rings were, so the CTAs meet before as well), the rows
-// dealt in equal runs.  More: through the workspace, that is through L2, the columns dealt in units of 8.  Shared memory of
-// another CTA takes stores at ~20 GB/s, 64 KB of 128 rows in 3 us, and shared-memory room needs the second meeting; L2
-// costs two of its latencies.  us per call, by shared memory / by L2: 4 rows on 2K 8.0 / 8.5, 12 x 64 heads with 8 rows
-// 7.4 / 7.6, 10 rows of 32 KV heads 10.2 / 10.1, 40 rows 8.3 / 7.6, 120 rows at 8K 17.2 / 15.9, 240 rows at 1K 10.6 / 9.7.
-// (Bulk copies between the CTAs instead of stores were slower than either: 8.8, 7.7, 10.5, 8.1, 17.7, 11.2.)  The other way
+// Up to 32: through the other CTAs' shared memory, the rows dealt in equal runs.  More: through the workspace, that is through
+// L2, the columns dealt in units of 8.  Shared memory of another CTA takes stores at ~20 GB/s, 64 KB of 128 rows in 3 us; L2
+// costs two of its latencies.  us per call, by shared memory / by L2, when the parts still went where Q and the rings had been
+// and the CTAs therefore met twice: 4 rows on 2K 8.0 / 8.5, 12 x 64 heads with 8 rows 7.4 / 7.6, 10 rows of 32 KV heads
+// 10.2 / 10.1, 40 rows 8.3 / 7.6, 120 rows at 8K 17.2 / 15.9, 240 rows at 1K 10.6 / 9.7.  Room of its own for the parts (see
+// Layout) saves the first meeting, 0.5 to 0.9 us; launched one by one, us per pass: two draft layers of 12 x 64 heads, 8 rows
+// 15.8 -> 15.0, one with 1 row 7.3 -> 6.8, 1 row of 32 KV heads on a 1K cache 10.3 -> 9.8, 4 rows 9.6 -> 9.1.
+// (Bulk copies between the CTAs instead of stores were slower than either: 8.8, 7.7, 10.5, 8.1, 17.7, 11.2.  Through L2, (m, l)
+// passed through shared memory and a CTA's own part of its share kept in tensor memory instead of going through L2 too: 240
+// rows at 1K 12.5 -> 13.2 us a call, 60 rows of 32 KV heads at 8K 33.8 -> 34.6.)  The other way
 // round where the tiles are many: 60 rows of 32 KV heads at 8K are 0.5 us shorter through shared memory.  Each is an
 // instantiation of its own: with both in one kernel a call was 0.1 to 0.3 us longer.  The forms through shared memory spill
 // for head_dim 128 and for the device-side length (8 to 16 bytes of stack, 312 to 348 bytes of reloads), in the exchange; those
@@ -96,6 +100,18 @@ struct MergeCtx {
 };
 constexpr int kMaxCluster = 16;
 constexpr int kRowsBySmem = kSpxClusterRowsBySmem;
+
+// Shared memory of an instantiation: the pipeline's (core.cuh) and, behind its control block, what the CTAs of a cluster write
+// into each other (MERGE 1): c CTAs x ceil(rows / c) parts of rows, at most 36 for up to 32 rows and 8 CTAs, of D floats and
+// (m, l).  With head_dim 128 the room comes from Q, which has at most 32 rows there (AttnPlan::q_rows).
+template <int D, int MERGE>
+struct Layout {
+  static constexpr int kCtrl = Geo<1, D>::kCtrlOffset - (MERGE == 1 && D == 128 ? 8192 : 0);
+  static constexpr int kExchange = kCtrl + kCtrlBytes;
+  static constexpr int kBytes = kExchange + (MERGE == 1 ? 36 * (D * 4 + 8) : 0) + 1024;
+  static_assert(kBytes <= 232448, "more shared memory than a CTA can have");
+};
+static_assert(kRowsBySmem <= 32, "Layout has room for 36 parts");
 constexpr float kLn2 = 0.693147180559945309417f;
 
 // This thread's half row of O.
@@ -113,14 +129,14 @@ __device__ __forceinline__ void own_half_row(const RowCtx& rc, bool any, uint32_
 }
 
 template <int D>
-__device__ __forceinline__ void merge_by_smem(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const MergeCtx& mc,
+__device__ __forceinline__ void merge_by_smem(const AttnArgs& a, const RowCtx& rc, unsigned char* room, const MergeCtx& mc,
                                               bool ok) {
-  cluster_sync();                                                  // the rings are free everywhere
+  cluster_wait();                                                  // every CTA of the cluster has started
   constexpr int kCols = D / 4;                                     // 16-byte columns of a row
   const AttnPlan& p = a.plan;
   const int cs = mc.cs, run = (mc.n_rows + cs - 1) / cs;           // rows of a CTA
   // received: [source CTA][row of the run][column, swizzled by the row so that a warp's rows use all banks]
-  float4* part = reinterpret_cast<float4*>(base);
+  float4* part = reinterpret_cast<float4*>(room);
   float2* ml = reinterpret_cast<float2*>(part + cs * run * kCols);
   if (ok && rc.row_t - rc.lane < mc.n_rows) {
     uint32_t v[D / 64][32];
@@ -270,7 +286,7 @@ __device__ __forceinline__ void merge_by_l2(const AttnArgs& a, const RowCtx& rc,
 }
 
 template <int D, int MERGE, class Work>
-__device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx& rc, unsigned char* base, const Work& work,
+__device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx& rc, unsigned char* room, const Work& work,
                                                  bool ok, float m_loc, float l) {
   const AttnPlan& p = a.plan;
   MergeCtx mc;
@@ -286,7 +302,7 @@ __device__ __forceinline__ bool merge_in_cluster(const AttnArgs& a, const RowCtx
   mc.l = 0.f;
   if (ok && mc.any) ok = segment_end(rc, work.n - 1, 0, m_loc, l, mc.m, mc.l);
   __syncwarp();
-  if constexpr (MERGE == 1) merge_by_smem<D>(a, rc, base, mc, ok);
+  if constexpr (MERGE == 1) merge_by_smem<D>(a, rc, room, mc, ok);
   else merge_by_l2<D, MERGE == 2 ? 8 : 16>(a, rc, mc, ok);
   return ok;
 }
@@ -303,7 +319,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                          ~static_cast<uintptr_t>(1023));
-  Ctrl* ctl = reinterpret_cast<Ctrl*>(base + G::kCtrlOffset);
+  Ctrl* ctl = reinterpret_cast<Ctrl*>(base + Layout<D, MERGE>::kCtrl);
   volatile int* abort_flag = &ctl->abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const G geo(p.q_rows);
@@ -311,6 +327,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
   const int worker = blockIdx.x;
   const int unit_lo = spx_unit_start(p, worker), unit_hi = spx_unit_start(p, worker + 1);
   setup<1>(ctl, warp, lane);
+  if constexpr (MERGE == 1) cluster_arrive_relaxed();    // (waited for before the first write to another CTA)
   // The kernel after this one may be set up while this one runs; this one reads and writes global memory only once the kernel
   // before it has completed: each role that does waits for that itself.
   pdl_launch_dependents();
@@ -614,12 +631,12 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       t0 += n;
       ++seg;
     }
-    if constexpr (MERGE != 0) ok = merge_in_cluster<D, MERGE>(a, rc, base, work, ok, m_loc, l);
+    if constexpr (MERGE != 0) ok = merge_in_cluster<D, MERGE>(a, rc, base + Layout<D, MERGE>::kExchange, work, ok, m_loc, l);
   }
   if constexpr (MERGE != 0) {
     if (warp >= kProducerWarp) {                         // the meetings of merge_in_cluster
       __syncwarp();
-      if (MERGE == 1) cluster_sync();
+      if (MERGE == 1) cluster_wait();
       cluster_sync();
     }
   }
@@ -631,7 +648,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
 template <int D, int SCORE, bool DEVLEN, int MERGE>
 cudaError_t launch(const AttnArgs& a, const VerifyMaps& maps, cudaStream_t st) {
   static SpxOncePerDevice once;
-  constexpr int smem = smem_bytes<1, D>();
+  constexpr int smem = Layout<D, MERGE>::kBytes;
   const cudaError_t ec = spx_opt_in_smem(verify_kernel<D, SCORE, DEVLEN, MERGE>, smem, &once, MERGE != 0);
   if (ec != cudaSuccess) return ec;
   cudaLaunchConfig_t cfg = {};
@@ -677,7 +694,7 @@ int spx_verify_max_clusters(int dev, int size) {
   if (n > 0) return n - 1;
   auto* kernel = verify_kernel<128, 0, false, 3>;
   static SpxOncePerDevice once;
-  constexpr int smem = smem_bytes<1, 128>();
+  constexpr int smem = Layout<128, 3>::kBytes;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(size);
   cfg.blockDim = dim3(kThreads);

@@ -31,6 +31,16 @@ def test_one_cta_row_blocks(cuda_device, Hq, Hkv, D, T, L):
     check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, 32)
 
 
+@pytest.mark.parametrize("Hq,Hkv,D,T,L", [
+    (12, 12, 128, 31, 600), (12, 12, 128, 32, 600), (12, 12, 64, 32, 600),     # 6 CTAs: 36 parts, all the room there is
+    (4, 4, 128, 29, 800), (8, 1, 128, 4, 900), (2, 1, 64, 16, 250),            # 7 and 8 CTAs, 35 and 32 parts; 3 CTAs, 33
+])
+def test_parts_in_shared_memory(cuda_device, Hq, Hkv, D, T, L):
+    """Clusters of few rows write their parts into each other's shared memory: as many parts as it has room for."""
+    w = synth.Workload("parts", Hq, Hkv, D, L, T, 32, 4, "uniform", "needle", seed=Hq + T + L)
+    check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, 32)
+
+
 @pytest.mark.parametrize("G", [64, 128, 256])
 def test_prefill_wide_groups(cuda_device, G):
     """Blocks of 4, 2 and 1 tokens: more problems than clusters, and (G = 256) one token's heads on two CTAs."""
