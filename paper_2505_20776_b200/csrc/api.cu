@@ -71,7 +71,6 @@ int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
   p.kernel = kernel;
   p.cluster = cluster;
   p.RB = row_block;
-  p.q_rows = kernel != 2 || p.D != 128 || p.rows > 64 ? 128 : cluster > 0 && p.rows <= kSpxClusterRowsBySmem ? 32 : 64;
   p.n_rblk = (p.rows + p.RB - 1) / p.RB;
   p.NP = p.Hkv * p.n_rblk;
   const long long U = (long long)p.NP * p.UPP;
@@ -114,6 +113,15 @@ int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
     p.max_segs = (p.UPP + p.q - 1) / p.q + 1;
   }
   if (p.max_segs > p.n_cta) p.max_segs = p.n_cta;
+  // Rows of Q a CTA of the one-CTA kernel keeps.  Its MMAs read 128 rows whatever there are, and what lies behind Q is K: at
+  // the power limit, where long passes run, multiplying it costs more than the stage of the K ring that 128 rows of Q (zeros
+  // behind the last) take up.  60 rows of 32 KV heads, one by one for seconds, 64 / 128 rows kept: four layers at 8K (16 tiles a
+  // CTA) 138.2 / 133.5 us, at 17K 247 / 235; 4 rows of 8 KV heads at 16K (7 tiles) the same, short calls up to 1 % longer.
+  p.q_rows = 128;
+  if (p.kernel == 2 && p.D == 128) {
+    if (p.cluster > 0 && p.rows <= kSpxClusterRowsBySmem) p.q_rows = 32;       // (the exchange needs the room, see Layout)
+    else if (p.rows <= 64 && p.U / p.n_cta < 12) p.q_rows = 64;
+  }
   p.n_slots = p.cluster > 0 ? p.n_cta : p.n_cta + p.NP - 1;
   long long off = 0;
   p.off_part_o = off; off += (long long)p.n_slots * p.D * p.RB;

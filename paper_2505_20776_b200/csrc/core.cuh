@@ -302,6 +302,7 @@ struct RowCtx {
   int w, row_t, lane;      // warpgroup, row inside the CTA's 128 rows
   uint32_t s_free, p_full; // cluster addresses of the leader's s_free[w] and p_full[w]
   float scale2;
+  bool pad;                // a row behind the last stacked one: its probabilities are zeros
   volatile int* abort_flag;
 };
 
@@ -393,7 +394,7 @@ __device__ __forceinline__ bool softmax_tile(const RowCtx& rc, uint32_t t, bool 
   }
   tc_fence_after();
 
-  const float neg_m = -m_new;
+  const float neg_m = rc.pad ? -INFINITY : -m_new;
   const uint64_t scale2x2 = pack_f32x2(rc.scale2, rc.scale2), neg_mx2 = pack_f32x2(neg_m, neg_m);
   auto exp_chunk = [&](uint32_t (&v)[32], int c) {
     // two elements per fma and per add (packed fp32 pairs); the exponential itself is per element

@@ -159,6 +159,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
       const int n = work.n;
       const int tok = work.b * a.tb + rr / a.G;          // this row's token
       const bool valid = tok < a.L;
+      rc.pad = !valid;
       const int head = work.g * a.G + rr % a.G;
       const int tok_eff = valid ? tok : a.L - 1;         // a padding row sees what the last token sees; it is not stored
       const int block_lo = work.b * a.tb;                // tiles that end at or before this key are fully visible

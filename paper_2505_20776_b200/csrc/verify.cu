@@ -511,6 +511,17 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     uint32_t t0 = 0, seg = 0;                            // tiles and segments before the current segment
     bool anc_seen = false;
     float m_loc, l;                                      // l is relative to m_loc
+    if (rr - lane >= p.rows) {
+      // No row block reaches this warp's rows: zeros for the PV MMAs to read there, once.  (Rows of zeros cost the tensor cores
+      // next to no power, see lay_out in api.cu.)
+      uint32_t z[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) z[k] = 0u;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tmem_st16(rc.lane_tmem + kColP + rc.w * 64 + c * 16, z);
+      tmem_wait_st();
+      tc_fence_before();
+    }
     pdl_wait();
     read_length();
     while (ok && work.next_any()) {
@@ -518,6 +529,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       const int r = rblk * p.RB + rr;
       const bool valid = r < p.rows;
       const bool warp_valid = r - lane < p.rows;
+      rc.pad = !valid;
       const int slot = worker + prob;
       float* po = a.ws + p.off_part_o + (long long)slot * (D / 4) * p.RB * 4;
       // this warpgroup's half of the output columns, in groups of 16
