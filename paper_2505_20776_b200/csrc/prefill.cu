@@ -14,7 +14,9 @@
 // segment_handover).  us per call, replayed, against the same loop with one P buffer, Q in tensor memory by plain loads and a
 // stop between problems / with both warpgroups ending a problem (32 query / 8 KV heads): 1K tokens 22.6 / 20.5 -> 18.4,
 // 2K 52.5 / 45.0 -> 40.6, 4K 135 / 121 -> 115, 16K 1655 / 1628 -> 1600 (1374 TFLOP/s; under the power cap 1825 -> 1720
-// before the last step).  Prefetching the tensor maps at the start costs 0.4 us at 2K and helps nowhere.  Slower than that
+// before the last step).  Each role waits for the kernel before just ahead of its own first access, with its first problem
+// worked out, and an idle thread asks for the first tile in L2 ahead of the wait: one by one 2K 43.6 -> 42.9, 1.8K with 64 query
+// heads 66.0 -> 65.4; 16K the same.  Prefetching the tensor maps by the producer costs 0.4 us at 2K and helps nowhere.  Slower than that
 // loop are prompts of at most 16 tokens with many KV heads, a single tile on every cluster: 48 heads of their own with 8 tokens
 // 5.6 -> 6.2, 32 5.4 -> 5.9, 12 5.3 -> 5.5; 33 tokens 6.4 -> 6.3, 6.1 -> 5.8, 6.3 -> 5.7.
 #include "common.cuh"
@@ -80,8 +82,8 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
   setup<2, true>(ctl, warp, lane);
   const uint32_t rank = cluster_rank();
   PrefillWork work(a, blockIdx.x >> 1);
+  // Global memory is read and written only once the kernel before has completed: each role that does waits for that itself.
   pdl_launch_dependents();
-  pdl_wait();
   bool ok = true;
 
   if (warp == kProducerWarp) {
@@ -91,7 +93,9 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
       const uint32_t kfull0 = leader_addr<2>(&ctl->k_full[0]), vfull0 = leader_addr<2>(&ctl->v_full[0]);
       int kst = 0, vst = 0;
       uint32_t kph = 1, vph = 1;
-      while (ok && work.next()) {
+      bool more = work.next();                           // (worked out ahead of the wait)
+      pdl_wait();
+      for (; ok && more; more = work.next()) {
         for (int tile = 0; tile < work.n && ok; ++tile) {
           const int key0 = tile * SPX_TILE_KEYS;
           ok = wait_c(&ctl->k_empty[kst], kph, abort_flag);
@@ -121,13 +125,25 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
     if (lane == 0 && rank == 0) ok = issue_s<2, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kPvWarp) {
     setmaxnreg_dec<kRegsOther>();
+    if (lane == 0) {
+      // The first tile is asked for in L2 ahead of the dependency wait, by a thread that has nothing else to do yet.  (A prefetch
+      // changes no result: what the kernel before may still write to these lines goes through L2 as well.)
+      PrefillWork first = work;
+      if (first.next()) {
+        tma_prefetch_3d(&maps.k, 0, first.g, 64 * rank);
+        tma_prefetch_3d(&maps.k, 64, first.g, 64 * rank);
+        tma_prefetch_3d(&maps.v, 64 * rank, first.g, 0);
+      }
+    }
     if (lane == 0 && rank == 0) ok = issue_pv<2, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kTreeWarp) {
     // ================================ TMA producer of Q =======================================
     setmaxnreg_dec<kRegsOther>();
     if (lane == 0) {
       const uint32_t bar = leader_addr<2>(&ctl->q_full);
-      for (uint32_t seg = 0; ok && work.next(); ++seg) {
+      bool more = work.next();
+      pdl_wait();
+      for (uint32_t seg = 0; ok && more; ++seg, more = work.next()) {
         if (seg > 0) ok = wait_c(&ctl->q_empty, (seg - 1) & 1, abort_flag);
         if (!ok) break;
         // rows rank*128.. of the block: 128/G tokens of all G heads, or half of the heads of the one token (G = 256)
@@ -155,6 +171,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
     const uint32_t o_free_l = leader_addr<2>(&ctl->o_free);
     const int rr = (int)rank * 128 + rc.row_t;           // row inside the 256-row block
     uint32_t t0 = 0, seg = 0;                            // tiles and problems before the current problem
+    pdl_wait();
     while (ok && work.next()) {
       const int n = work.n;
       const int tok = work.b * a.tb + rr / a.G;          // this row's token
