@@ -61,8 +61,12 @@ __device__ __forceinline__ void merge_batch(const float* __restrict__ pm, const 
   }
 }
 
+// (One block per SM, see launch_merge: told so, the compiler takes 242 and 107 registers a thread instead of 134 and 64 and keeps
+// more of a batch in flight.  us per pass, one by one: one scored call and its retrieval at 12K with 4 rows and chunks of 16
+// 35.5 -> 34.3, at 10K with 92 rows 37.2 -> 35.9, two layers at 27K with 8 rows 68.6 -> 66.9, at 36K with 4 rows 74.8 -> 73.0,
+// four layers at 5K with chunks of 16 81.9 -> 80.7; no change where the power limit sets the pace.)
 template <int B, int NT>
-__global__ void __launch_bounds__(NT) merge_kernel(const __grid_constant__ AttnArgs a) {
+__global__ void __launch_bounds__(NT, 1) merge_kernel(const __grid_constant__ AttnArgs a) {
   const AttnPlan& p = a.plan;
   sm100::pdl_launch_dependents();
   // everything that needs no global memory (indices, addresses, the output position) comes before the wait
