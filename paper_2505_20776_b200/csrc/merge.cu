@@ -4,7 +4,7 @@
 // merge_kernel: for each query row: M = max_s m_s,
 // Z = sum_s l_s 2^(m_s - M), lse = (M + log2 Z) ln 2, O = sum_s O~_s 2^(m_s - M) / Z.
 //
-// score_kernel: for every (tree node, chunk) sums over all query heads the chunk's exponential sum
+// score_kernel (and score_beside, in the merge's launch): for every (tree node, chunk) sums over all query heads the chunk's exponential sum
 // rescaled from its tile's reference maximum to the row's final lse, i.e. the exactly normalised
 // probability mass, and divides by Hq.
 #include "common.cuh"
@@ -15,6 +15,7 @@ namespace {
 constexpr float kLn2 = 0.693147180559945309417f;
 constexpr int kMergeSmemCap = 200 * 1024;          // bytes of dynamic shared memory requested only to limit residency
 constexpr float kLog2e = 1.44269504088896340736f;
+constexpr int kOneWave = 148;                      // blocks, one per SM
 
 // Block = NT / 32 warps; warp w handles two 16-byte column groups (d4, d4 + 1) for 32 consecutive rows of
 // one problem, so every partial read is a 512-byte coalesced segment, all reads of a thread are
@@ -61,24 +62,8 @@ __device__ __forceinline__ void merge_batch(const float* __restrict__ pm, const 
   }
 }
 
-// (One block per SM, see launch_merge: told so, the compiler takes 242 and 107 registers a thread instead of 134 and 64 and keeps
-// more of a batch in flight.  us per pass, one by one: one scored call and its retrieval at 12K with 4 rows and chunks of 16
-// 35.5 -> 34.3, at 10K with 92 rows 37.2 -> 35.9, two layers at 27K with 8 rows 68.6 -> 66.9, at 36K with 4 rows 74.8 -> 73.0,
-// four layers at 5K with chunks of 16 81.9 -> 80.7; no change where the power limit sets the pace.)
-template <int B, int NT>
-__global__ void __launch_bounds__(NT, 1) merge_kernel(const __grid_constant__ AttnArgs a) {
-  const AttnPlan& p = a.plan;
-  sm100::pdl_launch_dependents();
-  // everything that needs no global memory (indices, addresses, the output position) comes before the wait
-  const int blocks_per_prob = p.RB / 32;
-  const int prob = blockIdx.x / blocks_per_prob;
-  const int rr0 = (blockIdx.x - prob * blocks_per_prob) * 32;
-  const int g = prob / p.n_rblk;
-  const int rblk = prob - g * p.n_rblk;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rr = rr0 + lane;
-  const int r = rblk * p.RB + rr;
-  if (r >= p.rows) return;
+// The partial results of a problem: slot of the first one, and how many.
+__device__ __forceinline__ int segments_of(const AttnPlan& p, int prob, int& slot0) {
   int c_first, c_last;
   if (p.cpp > 0 && p.UPP >= p.cpp) {               // every one of the problem's cpp workers has a segment
     c_first = prob * p.cpp;
@@ -87,10 +72,139 @@ __global__ void __launch_bounds__(NT, 1) merge_kernel(const __grid_constant__ At
     c_first = spx_unit_owner(p, prob * p.UPP);
     c_last = spx_unit_owner(p, (prob + 1) * p.UPP - 1);
   }
-  const int nseg = c_last - c_first + 1;
-  const int slot0 = c_first + prob;
+  slot0 = c_first + prob;
+  return c_last - c_first + 1;
+}
+
+// Chunk scores beside the merge: 256 threads of a block that merges with its others.  A task is 64 rows of one key tile (VW
+// chunks); a block keeps to one group of 64 rows, whose statistics it takes from the partial results, once, instead of waiting
+// for the lse that the merge writes.  All sums have a fixed order, as in score_kernel.
+constexpr int kScoreRows = 64;
+constexpr int kScoreMaxKv = 64;                    // KV heads whose statistics have room
+template <int VW>
+struct ScoreRoom {
+  float part[4][kScoreRows][VW];
+  float lse2[kScoreMaxKv][kScoreRows];             // log2 of a row's sum, its maximum included
+};
+template <int VW>
+__device__ __forceinline__ void score_beside(const AttnArgs& a, ScoreRoom<VW>& sm, int tid) {
+  const AttnPlan& p = a.plan;
+  const int rr = tid & (kScoreRows - 1), slice = tid / kScoreRows;
+  const int n_groups = (p.rows + kScoreRows - 1) / kScoreRows;     // (gridDim.x is a multiple of it)
+  const int group = blockIdx.x % n_groups, r = group * kScoreRows + rr;
+  const int nodes = kScoreRows / p.G, t0 = group * nodes;          // nodes of the group
+  const float inv = 1.f / (float)p.Hq;
+  sm100::pdl_wait();                               // the attention kernel's results are complete
+  if (r < p.rows) {
+    for (int g = slice; g < p.Hkv; g += 4) {
+      int slot0;
+      const int nseg = segments_of(p, g, slot0);
+      const float* pm = a.ws + p.off_part_m + (long long)slot0 * p.RB + r;
+      const float* pl = a.ws + p.off_part_l + (long long)slot0 * p.RB + r;
+      float M = -INFINITY, Z = 0.f;
+      for (int s0 = 0; s0 < nseg; s0 += 12) {
+        float ms[12], ls[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+          ms[k] = s0 + k < nseg ? __ldcg(pm + (s0 + k) * p.RB) : -INFINITY;
+          ls[k] = s0 + k < nseg ? __ldcg(pl + (s0 + k) * p.RB) : 0.f;
+        }
+        float Mb = M;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) Mb = fmaxf(Mb, ms[k]);
+        Z *= sm100::ex2_approx(M - Mb);            // (0 on the first batch)
+        M = Mb;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) Z = fmaf(ls[k], sm100::ex2_approx(ms[k] - M), Z);
+      }
+      sm.lse2[g][rr] = M + log2f(Z);                  // (read by this thread only)
+    }
+  }
+  for (int tile = blockIdx.x / n_groups; tile < p.TPH; tile += gridDim.x / n_groups) {
+    float acc[VW];
+#pragma unroll
+    for (int k = 0; k < VW; ++k) acc[k] = 0.f;
+    if (r < p.rows) {
+      for (int g0 = slice; g0 < p.Hkv; g0 += 16) {
+        float m[4][VW], ref[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int g = g0 + q * 4;
+          if (g < p.Hkv) {
+            const long long base = ((long long)g * p.TPH + tile) * p.RB + r;
+            const float* src = a.ws + p.off_mass + base * VW;
+            if constexpr (VW == 4) {
+              const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+              m[q][0] = v.x; m[q][1] = v.y; m[q][2] = v.z; m[q][3] = v.w;
+            } else if constexpr (VW == 2) {
+              const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
+              m[q][0] = v.x; m[q][1] = v.y;
+            } else {
+              m[q][0] = __ldcg(src);
+            }
+            ref[q] = __ldcg(a.ws + p.off_mref + base);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int g = g0 + q * 4;
+          if (g < p.Hkv) {
+            const float f = exp2f(ref[q] - sm.lse2[g][rr]);
+#pragma unroll
+            for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[q][k], f, acc[k]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < VW; ++k) sm.part[slice][rr][k] = acc[k];
+    sm100::named_bar_sync(1, 256);
+    for (int o = tid; o < nodes * VW; o += 256) {
+      const int tt = o / VW, k = o - tt * VW, node = t0 + tt, c = tile * VW + k;
+      if (node < p.T && c < p.NC) {
+        float sum = 0.f;
+        for (int s = 0; s < 4; ++s)
+          for (int j = 0; j < p.G; ++j) sum += sm.part[s][tt * p.G + j][k];
+        a.chunk_score[(long long)node * p.NC + c] = sum * inv;
+      }
+    }
+    sm100::named_bar_sync(1, 256);
+  }
+}
+
+// VW > 0: blocks of NT + 256 threads in one line, of which the first n_merge (merge_x groups of rows times the blocks that share a
+// group's columns) merge with their first NT threads, and all add up chunk scores with the others.
+// (One block per SM, see launch_merge: told so, the compiler takes 242 and 107 registers a thread instead of 134 and 64 and keeps
+// more of a batch in flight.  us per pass, one by one: one scored call and its retrieval at 12K with 4 rows and chunks of 16
+// 35.5 -> 34.3, at 10K with 92 rows 37.2 -> 35.9, two layers at 27K with 8 rows 68.6 -> 66.9, at 36K with 4 rows 74.8 -> 73.0,
+// four layers at 5K with chunks of 16 81.9 -> 80.7; no change where the power limit sets the pace.)
+template <int B, int NT, int VW>
+__global__ void __launch_bounds__(NT + (VW > 0 ? 256 : 0), 1) merge_kernel(const __grid_constant__ AttnArgs a, int merge_x, int n_merge) {
+  const AttnPlan& p = a.plan;
+  sm100::pdl_launch_dependents();
+  if constexpr (VW > 0) {
+    __shared__ __align__(16) ScoreRoom<VW> room;
+    if (threadIdx.x >= NT) {
+      score_beside<VW>(a, room, threadIdx.x - NT);
+      return;
+    }
+    if ((int)blockIdx.x >= n_merge) return;
+  }
+  const int bx = VW > 0 ? (int)blockIdx.x % merge_x : (int)blockIdx.x, by = VW > 0 ? (int)blockIdx.x / merge_x : (int)blockIdx.y;
+  // everything that needs no global memory (indices, addresses, the output position) comes before the wait
+  const int blocks_per_prob = p.RB / 32;
+  const int prob = bx / blocks_per_prob;
+  const int rr0 = (bx - prob * blocks_per_prob) * 32;
+  const int g = prob / p.n_rblk;
+  const int rblk = prob - g * p.n_rblk;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rr = rr0 + lane;
+  const int r = rblk * p.RB + rr;
+  if (r >= p.rows) return;
+  int slot0;
+  const int nseg = segments_of(p, prob, slot0);
   const int nd4 = p.D / 4;
-  const int d4 = (blockIdx.y * (NT / 32) + warp) * 2;
+  const int d4 = (by * (NT / 32) + warp) * 2;
 
   const float* pm = a.ws + p.off_part_m + (long long)slot0 * p.RB + rr;
   const float* pl = a.ws + p.off_part_l + (long long)slot0 * p.RB + rr;
@@ -215,20 +329,43 @@ cudaError_t launch_score(const AttnArgs& a, cudaStream_t st) {
 
 namespace {
 
+int score_groups(const AttnPlan& p) { return (p.rows + kScoreRows - 1) / kScoreRows; }
+
+// Whether the chunk scores are added up beside the merge, in one launch, or by a launch of their own that waits for it.
+// Beside, the scores wait for the attention kernel only, which saves a launch that waits for another (3 us with its own chain of
+// latencies), but a block has its tasks one after another and works out its rows' statistics from all their segments: as long as
+// every block has one task.  One scored call and its retrieval, one by one, own launch / beside, 32 query / 8 KV heads: 60 nodes at
+// 4K (128 tasks) 23.4 / 21.9 us, one node at 16K (129) 29.9 / 29.7, one node of 64 heads at 18K (147) 34.6 / 34.6; four tasks a
+// block and more: 60 nodes at 16K 4 us longer.  (Started beside the merge as a launch of its own, by the merge once the attention
+// kernel was complete: 4K 23.6 -> 27.6.  A launch that was not set up ahead comes 4 us after it is asked for.)
+bool scores_beside_merge(const AttnPlan& p) {
+  return p.cluster == 0 && p.C >= 32 && p.n_rblk == 1 && p.Hkv <= kScoreMaxKv &&
+         p.NP * (p.RB / 32) * (p.D / 64) <= kOneWave && p.TPH * score_groups(p) <= kOneWave;
+}
+
 // Launched so that its blocks may be resident (waiting) before the attention kernel has finished.
 // Blocks become resident wherever an SM has room, so without a limit the SMs that the attention
 // kernel leaves first would take eight blocks each and a fraction of the SMs would do all the work:
 // an (unused) dynamic shared-memory request caps residency at one block per SM (measured: 1.1 us
 // per call faster than two per SM, which in turn was 2 us faster than no cap).
-template <int B, int NT>
+template <int B, int NT, int VW = 0>
 cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st) {
   const AttnPlan& p = a.plan;
   static SpxOncePerDevice once;
-  const cudaError_t ec = spx_opt_in_smem(merge_kernel<B, NT>, kMergeSmemCap, &once);
+  const cudaError_t ec = spx_opt_in_smem(merge_kernel<B, NT, VW>, kMergeSmemCap, &once);
   if (ec != cudaSuccess) return ec;
+  const int merge_x = p.NP * (p.RB / 32), merge_y = p.D * 4 / NT;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.NP * (p.RB / 32), p.D * 4 / NT);
-  cfg.blockDim = dim3(NT);
+  cfg.gridDim = dim3(merge_x, merge_y);
+  cfg.blockDim = dim3(NT + (VW > 0 ? 256 : 0));
+  if (VW > 0) {
+    // as many blocks as there are tasks, one per SM at most but at least the merge's, and a multiple of the groups of rows
+    const int n_groups = score_groups(p), tasks = p.TPH * n_groups, n_merge = merge_x * merge_y;
+    int blocks = kOneWave / n_groups * n_groups;
+    if (blocks > tasks) blocks = tasks;
+    if (blocks < n_merge) blocks = (n_merge + n_groups - 1) / n_groups * n_groups;
+    cfg.gridDim = dim3(blocks);
+  }
   cfg.dynamicSmemBytes = kMergeSmemCap;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -236,7 +373,7 @@ cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_kernel<B, NT>, a);
+  return cudaLaunchKernelEx(&cfg, merge_kernel<B, NT, VW>, a, merge_x, merge_x * merge_y);
 }
 
 }  // namespace
@@ -246,6 +383,13 @@ cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st) {
 cudaError_t spx_launch_merge(const AttnArgs& a, cudaStream_t st, int* n_launches) {
   const AttnPlan& p = a.plan;
   cudaError_t e = cudaSuccess;
+  if (p.want_score && p.NC > 0 && scores_beside_merge(p)) {
+    e = p.C == 32   ? launch_merge<12, 256, 4>(a, st)
+        : p.C == 64 ? launch_merge<12, 256, 2>(a, st)
+                    : launch_merge<12, 256, 1>(a, st);
+    *n_launches += 1;
+    return e;
+  }
   if (p.cluster == 0) {
     // With few segments per row the problems are many (64 query heads: 16 problems of 4 segments, 256 blocks of 256 threads):
     // blocks of 512 threads, all columns of 32 rows, keep the grid to one wave.  64 query heads at 16K 36.5 -> 34.8 us a

@@ -72,3 +72,15 @@ def test_chunk_sums_of_every_class(cuda_device, kernel, Hq, Hkv, D, T, L, C):
     w = synth.Workload("chunks", Hq, Hkv, D, L, T, C, 4, "uniform", "needle", seed=C + L)
     with tuned(kernel, 0):
         check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, C)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,T,L,C", [
+    (32, 8, 128, 60, 4096, 64), (32, 8, 128, 60, 4700, 128),     # pairs; 37 tiles x 4 groups of 64 rows: all the blocks there are
+    (32, 8, 128, 60, 4737, 32),                                  # one tile more: a launch of its own
+    (32, 8, 128, 37, 4000, 32),                                  # 148 rows: two and a third groups
+    (32, 8, 128, 1, 16383, 32), (16, 2, 64, 3, 16000, 128),      # one-CTA kernel, fewer rows than a group
+    (32, 1, 128, 2, 14000, 32),                                  # one KV head, 16 and more segments a row, blocks without a merge
+])
+def test_chunk_scores_beside_the_merge(cuda_device, Hq, Hkv, D, T, L, C):
+    w = synth.Workload("beside", Hq, Hkv, D, L, T, C, 4, "uniform", "needle", seed=T + C)
+    check_attn(make_hp(w, cuda_device), synth.make_layer(w), synth.make_tree(w), L, C)
