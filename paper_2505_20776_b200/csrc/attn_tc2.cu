@@ -662,7 +662,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
             }
           }
 
-          const float neg_m = valid ? -m_new : -INFINITY;    // (probabilities of a padding row: zeros)
+          const float neg_m = -m_new;
           const uint64_t scale2x2 = pack_f32x2(scale2, scale2), neg_mx2 = pack_f32x2(neg_m, neg_m);
           const bool score = SCORE != 0 && !is_tree;
           float* mass = nullptr;

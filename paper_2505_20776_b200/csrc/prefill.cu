@@ -168,6 +168,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
     rc.p_full = leader_addr<2>(&ctl->p_full[rc.w]);
     rc.scale2 = a.scale2;
     rc.abort_flag = abort_flag;
+    rc.pad = false;                                      // (only the last block has rows behind the last one)
     const uint32_t o_free_l = leader_addr<2>(&ctl->o_free);
     const int rr = (int)rank * 128 + rc.row_t;           // row inside the 256-row block
     uint32_t t0 = 0, seg = 0;                            // tiles and problems before the current problem
@@ -176,7 +177,6 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
       const int n = work.n;
       const int tok = work.b * a.tb + rr / a.G;          // this row's token
       const bool valid = tok < a.L;
-      rc.pad = !valid;
       const int head = work.g * a.G + rr % a.G;
       const int tok_eff = valid ? tok : a.L - 1;         // a padding row sees what the last token sees; it is not stored
       const int block_lo = work.b * a.tb;                // tiles that end at or before this key are fully visible
