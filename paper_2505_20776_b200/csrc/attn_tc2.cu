@@ -27,8 +27,8 @@
 //
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory
 // allocation and the start-up cluster barrier run while the kernel before it in the stream finishes.  Each role waits for
-// that kernel just before its own first read or write of global memory; the first K/V tiles are asked for in L2 ahead of the
-// wait (one scored call with its retrieval at 50K 49.9 -> 48.9 us, at 4K 23.7 -> 23.5; no change where the power limit sets
+// that kernel just before its own first read or write of global memory or, if that comes earlier, its first bounded wait; the
+// first K/V tiles are asked for in L2 ahead of that (one scored call with its retrieval at 50K 49.9 -> 48.9 us, at 4K 23.7 -> 23.5; no change where the power limit sets
 // the pace).
 #include "common.cuh"
 #include "pair.cuh"
@@ -133,7 +133,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
   }
   cluster_arrive();
   // The kernel after this one (the merge) may be set up while this one runs; this one reads and writes global
-  // memory only once the kernel before it has completed: each role that does waits for that itself.
+  // memory, and begins a bounded wait, only once the kernel before it has completed: each role waits for that itself.
   pdl_launch_dependents();
 
   const uint32_t rank = cluster_rank();
@@ -375,7 +375,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     if (warp == kMmaWarp) {
       // ================================ issuer of S = Q K^T (leader CTA) =====================
       setmaxnreg_dec<kRegsOther>();
-      if (DEVLEN) pdl_wait();
+      pdl_wait();                          // (a bounded wait must not count the time of the kernel before)
       if (lane == 0 && rank == 0) {
         const uint32_t idesc_s = idesc_bf16_f32(256, SPX_TILE_KEYS, false, false);
         constexpr uint32_t hi = desc_hi(1024);
@@ -432,7 +432,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
           tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * rank, g, key0);
         }
       }
-      if (DEVLEN) pdl_wait();
+      pdl_wait();
       if (lane == 0 && rank == 0) {
         const uint32_t idesc_o = idesc_bf16_f32(256, D, false, true);
         constexpr uint32_t hi = desc_hi(1024);

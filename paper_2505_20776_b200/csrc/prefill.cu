@@ -14,8 +14,8 @@
 // segment_handover).  us per call, replayed, against the same loop with one P buffer, Q in tensor memory by plain loads and a
 // stop between problems / with both warpgroups ending a problem (32 query / 8 KV heads): 1K tokens 22.6 / 20.5 -> 18.4,
 // 2K 52.5 / 45.0 -> 40.6, 4K 135 / 121 -> 115, 16K 1655 / 1628 -> 1600 (1374 TFLOP/s; under the power cap 1825 -> 1720
-// before the last step).  Each role waits for the kernel before just ahead of its own first access, with its first problem
-// worked out, and an idle thread asks for the first tile in L2 ahead of the wait: one by one 2K 43.6 -> 42.9, 1.8K with 64 query
+// before the last step).  Each role waits for the kernel before just ahead of its own first access or bounded wait, with
+// its first problem worked out, and an idle thread asks for the first tile in L2 ahead of the wait: one by one 2K 43.6 -> 42.9, 1.8K with 64 query
 // heads 66.0 -> 65.4; 16K the same.  Prefetching the tensor maps by the producer costs 0.4 us at 2K and helps nowhere.  Slower than that
 // loop are prompts of at most 16 tokens with many KV heads, a single tile on every cluster: 48 heads of their own with 8 tokens
 // 5.6 -> 6.2, 32 5.4 -> 5.9, 12 5.3 -> 5.5; 33 tokens 6.4 -> 6.3, 6.1 -> 5.8, 6.3 -> 5.7.
@@ -82,7 +82,8 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
   setup<2, true>(ctl, warp, lane);
   const uint32_t rank = cluster_rank();
   PrefillWork work(a, blockIdx.x >> 1);
-  // Global memory is read and written only once the kernel before has completed: each role that does waits for that itself.
+  // Global memory is read and written, and a bounded wait begun, only once the kernel before has completed: each role waits for
+  // that itself.
   pdl_launch_dependents();
   bool ok = true;
 
@@ -122,6 +123,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
     }
   } else if (warp == kMmaWarp) {
     setmaxnreg_dec<kRegsOther>();
+    pdl_wait();                                          // (a bounded wait must not count the time of the kernel before)
     if (lane == 0 && rank == 0) ok = issue_s<2, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kPvWarp) {
     setmaxnreg_dec<kRegsOther>();
@@ -135,6 +137,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
         tma_prefetch_3d(&maps.v, 64 * rank, first.g, 0);
       }
     }
+    pdl_wait();
     if (lane == 0 && rank == 0) ok = issue_pv<2, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kTreeWarp) {
     // ================================ TMA producer of Q =======================================

@@ -23,7 +23,26 @@ __global__ void __launch_bounds__(32) wait_timeout_kernel(long long limit_cycles
   if (!ok && threadIdx.x == 0) spx_raise(status, SPECEXT_ERR_TIMEOUT);
 }
 
+// A kernel that lets its dependents be set up at once and then takes its time, as one of another library may: at its end it
+// writes `value` to *dst.  It ends by itself after `cycles`.
+__global__ void __launch_bounds__(32) slow_kernel(long long cycles, int32_t* dst, int32_t value) {
+  sm100::pdl_launch_dependents();
+  if (threadIdx.x != 0) return;
+  const long long t0 = clock64();
+  while (clock64() - t0 < cycles) __nanosleep(1000);
+  *dst = value;
+}
+
 }  // namespace
+
+extern "C" int specext_test_slow_kernel(int64_t cycles, int32_t* dst, int32_t value, void* cuda_stream) {
+  if (!dst || cycles < 1 || cycles > 4000000000ll) return SPECEXT_ERR_INVALID_ARG;
+  slow_kernel<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>((long long)cycles, dst, value);
+  if (cudaGetLastError() != cudaSuccess) return SPECEXT_ERR_CUDA;
+  return SPECEXT_OK;
+}
+
+extern "C" int64_t specext_test_wait_limit(void) { return sm100::kWaitLimitCycles; }
 
 extern "C" int specext_test_wait_timeout(int64_t limit_cycles, int32_t* device_status, void* cuda_stream) {
   if (!device_status || limit_cycles < 1 || limit_cycles > 4000000000ll) return SPECEXT_ERR_INVALID_ARG;

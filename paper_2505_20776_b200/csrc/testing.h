@@ -30,6 +30,15 @@ int specext_test_set_tuning(int32_t attn_kernel, int32_t min_tiles_per_cta);
  */
 int specext_test_wait_timeout(int64_t limit_cycles, int32_t* device_status, void* cuda_stream);
 
+/*
+ * Launches a kernel of one CTA that lets the kernels behind it be set up at once, runs for `cycles` SM
+ * cycles (1 .. 4e9) and then stores `value` to *dst.  Returns a specext_status for the launch.
+ */
+int specext_test_slow_kernel(int64_t cycles, int32_t* dst, int32_t value, void* cuda_stream);
+
+/* The library's limit of a bounded wait, in SM cycles. */
+int64_t specext_test_wait_limit(void);
+
 #ifdef __cplusplus
 }
 #endif

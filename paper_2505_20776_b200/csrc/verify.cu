@@ -24,8 +24,8 @@
 //
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory allocation and the
 // start-up barrier run while the kernel before it in the stream finishes.  Each role waits for that kernel just before its own
-// first read or write of global memory, with the place of its first tile worked out, and the first tiles are asked for in L2
-// ahead of the wait.  Between the release and the request for the first K tile 1.2 to 2.0 us went by when all threads waited
+// first read or write of global memory or, if that comes earlier, its first bounded wait, with the place of its first tile
+// worked out, and the first tiles are asked for in L2 ahead of the wait.  Between the release and the request for the first K tile 1.2 to 2.0 us went by when all threads waited
 // at one place and the producer asked for L2 itself, now 0.5; us per pass, launched one by one: four layers at 1K with scores
 // and retrieval 53.0 -> 50.0, two layers of 12 x 64 heads on a 1K cache 16.4 -> 15.8, four layers of 32 KV heads at 8K
 // 137.3 -> 135.0, eight layers of 64 query heads at 1.4K 111.1 -> 106.9.
@@ -328,8 +328,8 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
   const int unit_lo = spx_unit_start(p, worker), unit_hi = spx_unit_start(p, worker + 1);
   setup<1>(ctl, warp, lane);
   if constexpr (MERGE == 1) cluster_arrive_relaxed();    // (waited for before the first write to another CTA)
-  // The kernel after this one may be set up while this one runs; this one reads and writes global memory only once the kernel
-  // before it has completed: each role that does waits for that itself.
+  // The kernel after this one may be set up while this one runs; this one reads and writes global memory, and begins a bounded
+  // wait, only once the kernel before it has completed: each role waits for that itself.
   pdl_launch_dependents();
   bool ok = true;
   int L_eff = p.L;
@@ -423,10 +423,8 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     }
   } else if (warp == kMmaWarp) {
     setmaxnreg_dec<kRegsOther>();
-    if (DEVLEN) {
-      pdl_wait();
-      read_length();
-    }
+    pdl_wait();                                          // (a bounded wait must not count the time of the kernel before)
+    read_length();
     if (lane == 0) ok = issue_s<1, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kPvWarp) {
     setmaxnreg_dec<kRegsOther>();
@@ -445,10 +443,8 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
         for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.vt : &maps.vp, 64 * ds, g, key0);
       }
     }
-    if (DEVLEN) {
-      pdl_wait();
-      read_length();
-    }
+    pdl_wait();
+    read_length();
     if (lane == 0) ok = issue_pv<1, D>(ctl, base, geo, work, abort_flag);
   } else if (warp == kTreeWarp) {
     // ================================ ancestor masks, TMA producer of Q =======================
