@@ -341,6 +341,7 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
           step(cv);
         }
       }
+      if (*abort_flag) ok = false;         // (see settle)
     }
   } else {
     if (warp == kTreeWarp) {
@@ -788,7 +789,10 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
     }
   }
 
-  if (!ok && lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+  if (!ok) {
+    if (lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+    settle();
+  }
   tc_fence_before();
   // The peer may still signal this CTA's barriers or read its halves, and tensor memory is freed by one
   // warp for all: everybody meets once more.  The partial results written above need no ordering here.

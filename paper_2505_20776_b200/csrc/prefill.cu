@@ -120,6 +120,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
           }
         }
       }
+      if (*abort_flag) ok = false;                       // (see settle)
     }
   } else if (warp == kMmaWarp) {
     setmaxnreg_dec<kRegsOther>();
@@ -156,6 +157,7 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
         tma_load<2>(smem_u32(base), &maps.q, bar, 0, head, tok);
         tma_load<2>(smem_u32(base + geo.q_blk), &maps.q, bar, 64, head, tok);
       }
+      if (*abort_flag) ok = false;
     }
   } else {
     // ================================ softmax warps ===========================================
@@ -234,7 +236,10 @@ prefill_kernel(const __grid_constant__ PrefillArgs a, const __grid_constant__ Pr
     }
   }
 
-  if (!ok && lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+  if (!ok) {
+    if (lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+    settle();
+  }
   finish<2>(ctl, warp);
 }
 

@@ -72,6 +72,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// When a role has given up, copies into shared memory may still be on their way, and that memory is another CTA's once this one
+// has ended.  A wait tests its barrier before the abort flag, so a producer may even issue some behind the abort, as far as its
+// ring has room.  So every thread that gave up, and a producer that finds that somebody did, lets kSettleCycles (a millisecond; a
+// copy takes microseconds) pass before it goes to the CTA's last barrier: the CTA ends that long after the last copy was issued.
+constexpr long long kSettleCycles = 2000000ll;
+__device__ __forceinline__ void settle() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < kSettleCycles) __nanosleep(100);
+}
+
 // ---- TMA ----------------------------------------------------------------------------------
 // 3-D tiled load global -> shared of this CTA, completion counted in bytes on `bar`.
 // Coordinate c0 (innermost) times the element size must be a multiple of 16 bytes.

@@ -36,6 +36,14 @@ int specext_test_wait_timeout(int64_t limit_cycles, int32_t* device_status, void
  */
 int specext_test_slow_kernel(int64_t cycles, int32_t* dst, int32_t value, void* cuda_stream);
 
+/*
+ * Launches a kernel of one warp that runs the end of a role that has given up (see settle in sm100.cuh)
+ * with a copy of 16 KB from `src` (16-byte aligned) on its way.  out[2] (device): the cycles it took,
+ * and whether the copy had landed then.
+ */
+int specext_test_settle(const void* src, int64_t* out, void* cuda_stream);
+int64_t specext_test_settle_cycles(void);
+
 /* The library's limit of a bounded wait, in SM cycles. */
 int64_t specext_test_wait_limit(void);
 

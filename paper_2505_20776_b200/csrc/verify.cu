@@ -420,6 +420,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
           }
         }
       }
+      if (*abort_flag) ok = false;                       // (see settle)
     }
   } else if (warp == kMmaWarp) {
     setmaxnreg_dec<kRegsOther>();
@@ -488,6 +489,7 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
         ok = wait_c(&ctl->q_empty, seg & 1, abort_flag);
         if (ok) load_q(work.prob);
       }
+      if (*abort_flag) ok = false;
     }
   } else {
     // ================================ softmax warps ===========================================
@@ -649,7 +651,10 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
     }
   }
 
-  if (!ok && lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+  if (!ok) {
+    if (lane == 0) spx_raise(a.status, SPECEXT_ERR_TIMEOUT);
+    settle();
+  }
   finish<1>(ctl, warp);
 }
 

@@ -22,6 +22,10 @@ def load_testing_lib() -> ctypes.CDLL:
         L.specext_test_slow_kernel.argtypes = [ctypes.c_int64, ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p]
         L.specext_test_wait_limit.restype = ctypes.c_int64
         L.specext_test_wait_limit.argtypes = []
+        L.specext_test_settle.restype = ctypes.c_int
+        L.specext_test_settle.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+        L.specext_test_settle_cycles.restype = ctypes.c_int64
+        L.specext_test_settle_cycles.argtypes = []
         _TLIB = L
     return _TLIB
 
