@@ -22,8 +22,10 @@
  *   - The kernels of these calls are launched with programmatic stream serialization, so
  *     that the set-up of one overlaps the tail of the one before it in the stream; each of them
  *     waits for that predecessor to complete (and its writes to be visible) before it reads or
- *     writes global memory, so the stream order the caller sees is the usual one.  The calls can
- *     be captured into CUDA graphs.
+ *     writes global memory, so the stream order the caller sees is the usual one.  (Ahead of that
+ *     wait the attention kernels only ask for K/V tiles to be brought into L2, a draft call for those
+ *     that *n_tokens counts at that moment; no result depends on it.)  The calls can be captured into
+ *     CUDA graphs.
  */
 #ifndef SPECEXT_H_
 #define SPECEXT_H_

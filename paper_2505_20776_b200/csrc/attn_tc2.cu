@@ -419,7 +419,9 @@ attn_tc2_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Tc2M
       setmaxnreg_dec<kRegsOther>();
       if (lane == 0 && unit_lo < unit_hi && !dev_len) {
         // The first K/V tiles are asked for in L2 ahead of the dependency wait, by a thread that has nothing else to do.  A
-        // prefetch changes no result: what the kernel before may still write to these lines goes through L2 as well.
+        // prefetch changes no result: what the kernel before may still write to these lines goes through L2 as well.  (Not with
+        // a device-side length: whether a tile exists is not known before the wait, and the draft calls that come here, 60
+        // nodes and more on long caches, have not been measured with a look at the length as it stands, see verify.cu.)
         const int prob = unit_lo / p.UPP;
         const int g = prob / p.n_rblk;
         for (int i = 0; i < (many ? 2 : 1); ++i) {

@@ -433,10 +433,16 @@ verify_kernel(const __grid_constant__ AttnArgs a, const __grid_constant__ Verify
       // The first tile is asked for in L2 ahead of the dependency wait, by a thread that has nothing else to do yet; the second one
       // too where a worker has several: 16K 19.6 -> 19.3, 128K 88.3 -> 87.5, but 2K 8.1 -> 8.4.  A prefetch changes no result:
       // what the kernel before may still write to these lines goes through L2 as well.
+      // A device-side length is looked at here as it stands (the kernel before may be about to change it, so it decides about
+      // this request and nothing else): a cache that is partly filled does not read the rest of its capacity.  us per pass of
+      // two calls, no request / asked for whatever the length / as it is, 10 nodes of 32 query / 8 KV heads: 2048 tokens of
+      // 8192 24.5 / 26.4 / 24.7, 4096 27.6 / 28.0 / 27.3, all 30.3 / 29.5 / 29.0, 16384 of 16384 46.6 / 42.7 / 42.5.
       const int prob = unit_lo / p.UPP, tile = unit_lo - prob * p.UPP, g = prob / p.n_rblk;
+      const int tph_now = DEVLEN ? (spx_prefix_len(a) + SPX_TILE_KEYS - 1) / SPX_TILE_KEYS : p.TPH;
       for (int i = 0; i < (unit_hi - unit_lo >= 6 ? 2 : 1); ++i) {
         if (tile + i > p.TPH) break;
         const bool is_tree = tile + i == p.TPH;
+        if (DEVLEN && !is_tree && tile + i >= tph_now) break;
         const int key0 = is_tree ? 0 : (tile + i) * SPX_TILE_KEYS;
 #pragma unroll
         for (int ds = 0; ds < G::kBlocks; ++ds) tma_prefetch_3d(is_tree ? &maps.kt : &maps.kp, 64 * ds, g, key0);
