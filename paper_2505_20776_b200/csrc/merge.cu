@@ -76,9 +76,9 @@ __device__ __forceinline__ int segments_of(const AttnPlan& p, int prob, int& slo
   return c_last - c_first + 1;
 }
 
-// Chunk scores beside the merge: 256 threads of a block that merges with its others.  A task is 64 rows of one key tile (VW
-// chunks); a block keeps to one group of 64 rows, whose statistics it takes from the partial results, once, instead of waiting
-// for the lse that the merge writes.  All sums have a fixed order, as in score_kernel.
+// Chunk scores beside the merge: 256 threads of a block that merges with its others.  A block has one task, 64 rows of one key
+// tile (VW chunks); it takes the rows' statistics from the partial results instead of waiting for the lse that the merge writes.
+// All sums have a fixed order, as in score_kernel.
 constexpr int kScoreRows = 64;
 constexpr int kScoreMaxKv = 64;                    // KV heads whose statistics have room
 template <int VW>
@@ -90,8 +90,9 @@ template <int VW>
 __device__ __forceinline__ void score_beside(const AttnArgs& a, ScoreRoom<VW>& sm, int tid) {
   const AttnPlan& p = a.plan;
   const int rr = tid & (kScoreRows - 1), slice = tid / kScoreRows;
-  const int n_groups = (p.rows + kScoreRows - 1) / kScoreRows;     // (gridDim.x is a multiple of it)
-  const int group = blockIdx.x % n_groups, r = group * kScoreRows + rr;
+  const int n_groups = (p.rows + kScoreRows - 1) / kScoreRows;
+  const int tile = blockIdx.x / n_groups, group = blockIdx.x - tile * n_groups, r = group * kScoreRows + rr;
+  if (tile >= p.TPH) return;                       // a block that only merges
   const int nodes = kScoreRows / p.G, t0 = group * nodes;          // nodes of the group
   const float inv = 1.f / (float)p.Hq;
   sm100::pdl_wait();                               // the attention kernel's results are complete
@@ -120,62 +121,62 @@ __device__ __forceinline__ void score_beside(const AttnArgs& a, ScoreRoom<VW>& s
       sm.lse2[g][rr] = M + log2f(Z);                  // (read by this thread only)
     }
   }
-  for (int tile = blockIdx.x / n_groups; tile < p.TPH; tile += gridDim.x / n_groups) {
-    float acc[VW];
+  float acc[VW];
 #pragma unroll
-    for (int k = 0; k < VW; ++k) acc[k] = 0.f;
-    if (r < p.rows) {
-      for (int g0 = slice; g0 < p.Hkv; g0 += 16) {
-        float m[4][VW], ref[4];
+  for (int k = 0; k < VW; ++k) acc[k] = 0.f;
+  if (r < p.rows) {
+    for (int g0 = slice; g0 < p.Hkv; g0 += 16) {
+      float m[4][VW], ref[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int g = g0 + q * 4;
-          if (g < p.Hkv) {
-            const long long base = ((long long)g * p.TPH + tile) * p.RB + r;
-            const float* src = a.ws + p.off_mass + base * VW;
-            if constexpr (VW == 4) {
-              const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
-              m[q][0] = v.x; m[q][1] = v.y; m[q][2] = v.z; m[q][3] = v.w;
-            } else if constexpr (VW == 2) {
-              const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
-              m[q][0] = v.x; m[q][1] = v.y;
-            } else {
-              m[q][0] = __ldcg(src);
-            }
-            ref[q] = __ldcg(a.ws + p.off_mref + base);
+      for (int q = 0; q < 4; ++q) {
+        const int g = g0 + q * 4;
+        if (g < p.Hkv) {
+          const long long base = ((long long)g * p.TPH + tile) * p.RB + r;
+          const float* src = a.ws + p.off_mass + base * VW;
+          if constexpr (VW == 4) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+            m[q][0] = v.x; m[q][1] = v.y; m[q][2] = v.z; m[q][3] = v.w;
+          } else if constexpr (VW == 2) {
+            const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
+            m[q][0] = v.x; m[q][1] = v.y;
+          } else {
+            m[q][0] = __ldcg(src);
           }
+          ref[q] = __ldcg(a.ws + p.off_mref + base);
         }
+      }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int g = g0 + q * 4;
-          if (g < p.Hkv) {
-            const float f = exp2f(ref[q] - sm.lse2[g][rr]);
+      for (int q = 0; q < 4; ++q) {
+        const int g = g0 + q * 4;
+        if (g < p.Hkv) {
+          const float f = exp2f(ref[q] - sm.lse2[g][rr]);
 #pragma unroll
-            for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[q][k], f, acc[k]);
-          }
+          for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[q][k], f, acc[k]);
         }
       }
     }
+  }
 #pragma unroll
-    for (int k = 0; k < VW; ++k) sm.part[slice][rr][k] = acc[k];
-    sm100::named_bar_sync(1, 256);
-    for (int o = tid; o < nodes * VW; o += 256) {
-      const int tt = o / VW, k = o - tt * VW, node = t0 + tt, c = tile * VW + k;
-      if (node < p.T && c < p.NC) {
-        float sum = 0.f;
-        for (int s = 0; s < 4; ++s)
-          for (int j = 0; j < p.G; ++j) sum += sm.part[s][tt * p.G + j][k];
-        a.chunk_score[(long long)node * p.NC + c] = sum * inv;
-      }
+  for (int k = 0; k < VW; ++k) sm.part[slice][rr][k] = acc[k];
+  sm100::named_bar_sync(1, 256);
+  for (int o = tid; o < nodes * VW; o += 256) {
+    const int tt = o / VW, k = o - tt * VW, node = t0 + tt, c = tile * VW + k;
+    if (node < p.T && c < p.NC) {
+      float sum = 0.f;
+      for (int s = 0; s < 4; ++s)
+        for (int j = 0; j < p.G; ++j) sum += sm.part[s][tt * p.G + j][k];
+      a.chunk_score[(long long)node * p.NC + c] = sum * inv;
     }
-    sm100::named_bar_sync(1, 256);
   }
 }
 
 // VW > 0: blocks of NT + 256 threads in one line, of which the first n_merge (merge_x groups of rows times the blocks that share a
-// group's columns) merge with their first NT threads, and all add up chunk scores with the others.
-// (One block per SM, see launch_merge: told so, the compiler takes 242 and 107 registers a thread instead of 134 and 64 and keeps
-// more of a batch in flight.  us per pass, one by one: one scored call and its retrieval at 12K with 4 rows and chunks of 16
+// group's columns) merge with their first NT threads; the other 256 threads add up the chunk scores of task blockIdx.x, if there
+// is one.  Those 512 threads have 128 registers each and the merge spills 16 bytes (with 192 for the merge and 64 for the scores,
+// setmaxnreg, nothing spills, but a pass with 64 rows and 140 tiles takes 32.7 instead of 32.3 us, 240 rows at 4K 21.2 instead of
+// 21.1).
+// VW = 0 (one block per SM, see launch_merge: told so, the compiler takes 242 and 107 registers a thread instead of 134 and 64 and
+// keeps more of a batch in flight.  us per pass, one by one: one scored call and its retrieval at 12K with 4 rows and chunks of 16
 // 35.5 -> 34.3, at 10K with 92 rows 37.2 -> 35.9, two layers at 27K with 8 rows 68.6 -> 66.9, at 36K with 4 rows 74.8 -> 73.0,
 // four layers at 5K with chunks of 16 81.9 -> 80.7; no change where the power limit sets the pace.)
 template <int B, int NT, int VW>
@@ -333,11 +334,13 @@ int score_groups(const AttnPlan& p) { return (p.rows + kScoreRows - 1) / kScoreR
 
 // Whether the chunk scores are added up beside the merge, in one launch, or by a launch of their own that waits for it.
 // Beside, the scores wait for the attention kernel only, which saves a launch that waits for another (3 us with its own chain of
-// latencies), but a block has its tasks one after another and works out its rows' statistics from all their segments: as long as
-// every block has one task.  One scored call and its retrieval, one by one, own launch / beside, 32 query / 8 KV heads: 60 nodes at
-// 4K (128 tasks) 23.4 / 21.9 us, one node at 16K (129) 29.9 / 29.7, one node of 64 heads at 18K (147) 34.6 / 34.6; four tasks a
-// block and more: 60 nodes at 16K 4 us longer.  (Started beside the merge as a launch of its own, by the merge once the attention
-// kernel was complete: 4K 23.6 -> 27.6.  A launch that was not set up ahead comes 4 us after it is asked for.)
+// latencies), but a block works out its rows' statistics from all their segments: as long as every block has one task.  One scored
+// call and its retrieval, one by one, own launch / beside, 32 query / 8 KV heads: 60 nodes at 4K (128 tasks) 23.4 / 21.9 us, one
+// node at 16K (129) 29.9 / 29.7, one node of 64 heads at 18K (147) 34.6 / 34.6.  Two tasks a block, in a loop: 60 nodes at 6K
+// 24.9 / 24.1, at 8K 26.9 / 26.3, but one node at 32K 38.4 / 40.3, 16 at 30K 39.4 / 40.4; three: 60 nodes at 12K 30.3 / 30.8, one
+// at 50K 49.6 / 51.3; four and more: 60 nodes at 16K 4 us longer.  (The loop for several tasks, where every block has one: 60 nodes
+// at 4K 21.13 -> 21.05 without it, one at 16K 28.5 -> 28.0.  Started beside the merge as a launch of its own, by the merge once the
+// attention kernel was complete: 4K 23.6 -> 27.6.  A launch that was not set up ahead comes 4 us after it is asked for.)
 bool scores_beside_merge(const AttnPlan& p) {
   return p.cluster == 0 && p.C >= 32 && p.n_rblk == 1 && p.Hkv <= kScoreMaxKv &&
          p.NP * (p.RB / 32) * (p.D / 64) <= kOneWave && p.TPH * score_groups(p) <= kOneWave;
@@ -359,12 +362,8 @@ cudaError_t launch_merge(const AttnArgs& a, cudaStream_t st) {
   cfg.gridDim = dim3(merge_x, merge_y);
   cfg.blockDim = dim3(NT + (VW > 0 ? 256 : 0));
   if (VW > 0) {
-    // as many blocks as there are tasks, one per SM at most but at least the merge's, and a multiple of the groups of rows
-    const int n_groups = score_groups(p), tasks = p.TPH * n_groups, n_merge = merge_x * merge_y;
-    int blocks = kOneWave / n_groups * n_groups;
-    if (blocks > tasks) blocks = tasks;
-    if (blocks < n_merge) blocks = (n_merge + n_groups - 1) / n_groups * n_groups;
-    cfg.gridDim = dim3(blocks);
+    const int tasks = p.TPH * score_groups(p), n_merge = merge_x * merge_y;
+    cfg.gridDim = dim3(tasks > n_merge ? tasks : n_merge);
   }
   cfg.dynamicSmemBytes = kMergeSmemCap;
   cfg.stream = st;
