@@ -547,6 +547,18 @@ int specext_test_set_tuning(int32_t attn_kernel, int32_t min_tiles_per_cta) {
   if (min_tiles_per_cta > 0) g_min_units.store(min_tiles_per_cta);
   return SPECEXT_OK;
 }
+
+// Test library only: the form that a call with this descriptor takes (see testing.h).
+int specext_test_plan(const specext_attn_desc* desc, int32_t length_on_device, int32_t* out) {
+  AttnPlan p;
+  const int rc = build_plan(desc, &p, length_on_device != 0);
+  if (rc != SPECEXT_OK) return rc;
+  out[0] = p.kernel;
+  out[1] = p.cluster;
+  out[2] = p.q_rows;
+  out[3] = p.U / p.n_cta;
+  return SPECEXT_OK;
+}
 #endif
 
 }  // extern "C"

@@ -7,6 +7,8 @@
 
 #include <stdint.h>
 
+#include "../../include/specext.h"
+
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -21,6 +23,13 @@ extern "C" {
  * Both change the workspace size: query specext_verify_attn_workspace after setting them.
  */
 int specext_test_set_tuning(int32_t attn_kernel, int32_t min_tiles_per_cta);
+
+/*
+ * The form that a call takes (length_on_device: a draft call), without running it.  out[4]: the kernel
+ * (2 / 3 as above), the size of its clusters or 0, the rows of Q that a CTA keeps (one-CTA kernel), the
+ * key tiles per worker, rounded down.  Returns a specext_status.
+ */
+int specext_test_plan(const specext_attn_desc* desc, int32_t length_on_device, int32_t* out);
 
 /*
  * Launches a one-CTA kernel that waits, with the library's bounded mbarrier wait and the given limit

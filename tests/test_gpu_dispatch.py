@@ -1,5 +1,6 @@
 """Which form a call takes, seen by the kernels it launches: one whose clusters merge by themselves is one launch, one that
-leaves partial results two, and the chunk scores are one more.  On the B200 (clusters of up to 16 of its CTAs)."""
+leaves partial results two, and the chunk scores are one more, unless they are added up beside the merge (chunks of 32 keys and
+more on up to 148 tiles of 64 rows).  On the B200 (clusters of up to 16 of its CTAs)."""
 import pytest
 import torch
 

@@ -33,7 +33,8 @@ def test_one_cta_row_blocks(cuda_device, Hq, Hkv, D, T, L):
 
 @pytest.mark.parametrize("Hq,Hkv,D,T,L", [
     (12, 12, 128, 31, 600), (12, 12, 128, 32, 600), (12, 12, 64, 32, 600),     # 6 CTAs: 36 parts, all the room there is
-    (4, 4, 128, 29, 800), (8, 1, 128, 4, 900), (2, 1, 64, 16, 250),            # 7 and 8 CTAs, 35 and 32 parts; 3 CTAs, 33
+    (4, 4, 128, 29, 800), (8, 1, 128, 4, 900), (2, 1, 64, 16, 250),            # 8, 5 and 3 CTAs: 32, 35 and 33 parts
+    (4, 4, 128, 32, 700),                                                      # 7 CTAs, 35 parts
 ])
 def test_parts_in_shared_memory(cuda_device, Hq, Hkv, D, T, L):
     """Clusters of few rows write their parts into each other's shared memory: as many parts as it has room for."""

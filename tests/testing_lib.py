@@ -26,8 +26,23 @@ def load_testing_lib() -> ctypes.CDLL:
         L.specext_test_settle.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
         L.specext_test_settle_cycles.restype = ctypes.c_int64
         L.specext_test_settle_cycles.argtypes = []
+        L.specext_test_plan.restype = ctypes.c_int
+        L.specext_test_plan.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p]
         _TLIB = L
     return _TLIB
+
+
+def plan(Hq, Hkv, D, T, L, C=32, scored=False, length_on_device=False):
+    """(kernel, size of its clusters, rows of Q per CTA, key tiles per worker) of a call on contiguous tensors."""
+    d = api.AttnDesc()
+    d.n_q_heads, d.n_kv_heads, d.head_dim = Hq, Hkv, D
+    d.prefix_len, d.n_tree, d.chunk_size = L, T, C
+    d.softmax_scale, d.want_chunk_score = 0.0, int(scored)
+    d.q_stride_t, d.kv_stride_l, d.tkv_stride_t, d.o_stride_t = Hq * D, Hkv * D, Hkv * D, Hq * D
+    d.q_stride_h = d.kv_stride_h = d.tkv_stride_h = d.o_stride_h = D
+    out = (ctypes.c_int32 * 4)()
+    assert load_testing_lib().specext_test_plan(ctypes.byref(d), int(length_on_device), out) == 0
+    return tuple(out)
 
 
 @contextlib.contextmanager
