@@ -115,8 +115,12 @@ int lay_out(AttnPlan* plan, int kernel, int row_block, int cluster) {
   if (p.max_segs > p.n_cta) p.max_segs = p.n_cta;
   // Rows of Q a CTA of the one-CTA kernel keeps.  Its MMAs read 128 rows whatever there are, and what lies behind Q is K: at
   // the power limit, where long passes run, multiplying it costs more than the stage of the K ring that 128 rows of Q (zeros
-  // behind the last) take up.  60 rows of 32 KV heads, one by one for seconds, 64 / 128 rows kept: four layers at 8K (16 tiles a
-  // CTA) 138.2 / 133.5 us, at 17K 247 / 235; 4 rows of 8 KV heads at 16K (7 tiles) the same, short calls up to 1 % longer.
+  // behind the last) take up.  us per pass, one by one, 64 / 128 rows kept: 60 rows of 32 KV heads, two layers at 8K (16 tiles a
+  // CTA) 73.9 / 72.8, at 16K 122.9 / 120.6; of 8 KV heads, 4 rows, two layers at 32K (13 tiles) 71.9 / 70.4, 32 rows at 48K
+  // 97.7 / 95.0, 64 rows at 32K 77.5 / 75.3, one layer of 64 rows at 128K (55 tiles) 120.2 / 119.0; one row of 32 KV heads at 16K
+  // and 40K the same.  Below the line: 4 rows of 8 KV heads at 16K (7 tiles) the same, short calls up to 1 % longer with 128.
+  // (The cleared rows of P in verify.cu are the other half: without them 60 rows of 32 KV heads, four layers, take 134.8 instead
+  // of 133.3 at 8K and 229.0 instead of 225.9 at 16K, 64 rows of 8 at 128K 119.7 instead of 118.5, 16 rows and fewer the same.)
   p.q_rows = 128;
   if (p.kernel == 2 && p.D == 128) {
     if (p.cluster > 0 && p.rows <= kSpxClusterRowsBySmem) p.q_rows = 32;       // (the exchange needs the room, see Layout)

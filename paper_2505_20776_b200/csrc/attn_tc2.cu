@@ -28,8 +28,8 @@
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory
 // allocation and the start-up cluster barrier run while the kernel before it in the stream finishes.  Each role waits for
 // that kernel just before its own first read or write of global memory or, if that comes earlier, its first bounded wait; the
-// first K/V tiles are asked for in L2 ahead of that (one scored call with its retrieval at 50K 49.9 -> 48.9 us, at 4K 23.7 -> 23.5; no change where the power limit sets
-// the pace).
+// first K/V tiles are asked for in L2 ahead of that (one scored call with its retrieval at 50K 49.9 -> 48.9 us, at 4K
+// 23.7 -> 23.5; no change where the power limit sets the pace).
 #include "common.cuh"
 #include "pair.cuh"
 #include "tmap.h"

@@ -47,12 +47,13 @@ struct Geo {
   static constexpr int kVStage = PAIR == 2 ? kVBlk : kVBlk * kBlocks;
   static constexpr int kQBytes = 128 * 128 * kBlocks;
   static constexpr bool kWide = kKStage == 32768;            // one CTA with head_dim 128: stages of 32 KB
-  // (wide: 16 KB of Q and six stages with q_rows = 64, or 32 KB of Q and five stages)
+  // (wide: 16 KB of Q and six stages with 64 rows, 8 KB and six with 32, or 32 KB and five with 128)
   static constexpr int kCtrlOffset = kWide ? 16384 + 6 * 32768 : kQBytes + 11 * 16384;
   int q_blk, nk, nv;
   uint32_t k_off, v_off;
-  // rows = 64 or 32 (only with one CTA, head_dim 128 and at most that many stacked rows): Q takes half the room or less, which
-  // is one more stage.  The MMA still reads 128 rows; what lies behind Q is multiplied into rows nobody looks at.
+  // rows = AttnPlan::q_rows.  64 or 32 (one CTA, head_dim 128 and at most that many stacked rows): Q takes half the room or less,
+  // which is one more stage.  The MMA still reads 128 rows; what lies behind Q is multiplied into rows nobody looks at.  Calls
+  // with as few rows may keep 128 all the same, zeros behind the last (see lay_out in api.cu).
   __device__ __forceinline__ explicit Geo(int rows) {
     q_blk = rows * 128;
     nk = kWide ? (rows <= 64 ? 3 : 2) : 5;

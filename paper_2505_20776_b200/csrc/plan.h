@@ -37,7 +37,8 @@ struct AttnPlan {
   int rows;        // G*T query rows per KV head
   int RB;          // rows per row block (128 or 256)
   int n_rblk;      // row blocks per KV head
-  int q_rows;      // query rows a CTA keeps in shared memory: 128, or 64 or 32 when no row block has more (one-CTA kernel)
+  int q_rows;      // query rows a CTA keeps in shared memory: 128, or 64 or 32 in some calls where no row block has more (one-CTA
+                   // kernel, head_dim 128; the rule is in lay_out, api.cu)
   int NP;          // problems = Hkv * n_rblk
   int TPH;         // prefix key tiles per problem = ceil(L/128)
   int UPP;         // units per problem = TPH + 1 (tree tile last)

@@ -15,10 +15,10 @@
 // stop between problems / with both warpgroups ending a problem (32 query / 8 KV heads): 1K tokens 22.6 / 20.5 -> 18.4,
 // 2K 52.5 / 45.0 -> 40.6, 4K 135 / 121 -> 115, 16K 1655 / 1628 -> 1600 (1374 TFLOP/s; under the power cap 1825 -> 1720
 // before the last step).  Each role waits for the kernel before just ahead of its own first access or bounded wait, with
-// its first problem worked out, and an idle thread asks for the first tile in L2 ahead of the wait: one by one 2K 43.6 -> 42.9, 1.8K with 64 query
-// heads 66.0 -> 65.4; 16K the same.  Prefetching the tensor maps by the producer costs 0.4 us at 2K and helps nowhere.  Slower than that
-// loop are prompts of at most 16 tokens with many KV heads, a single tile on every cluster: 48 heads of their own with 8 tokens
-// 5.6 -> 6.2, 32 5.4 -> 5.9, 12 5.3 -> 5.5; 33 tokens 6.4 -> 6.3, 6.1 -> 5.8, 6.3 -> 5.7.
+// its first problem worked out, and an idle thread asks for the first tile in L2 ahead of the wait: one by one 2K 43.6 -> 42.9,
+// 1.8K with 64 query heads 66.0 -> 65.4; 16K the same.  Prefetching the tensor maps by the producer costs 0.4 us at 2K and helps
+// nowhere.  Slower than that loop are prompts of at most 16 tokens with many KV heads, a single tile on every cluster: 48 heads of
+// their own with 8 tokens 5.6 -> 6.2, 32 5.4 -> 5.9, 12 5.3 -> 5.5; 33 tokens 6.4 -> 6.3, 6.1 -> 5.8, 6.3 -> 5.7.
 #include "common.cuh"
 #include "core.cuh"
 #include "tmap.h"

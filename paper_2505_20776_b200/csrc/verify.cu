@@ -25,10 +25,12 @@
 // The kernel is launched with programmatic stream serialization: barrier set-up, tensor-memory allocation and the
 // start-up barrier run while the kernel before it in the stream finishes.  Each role waits for that kernel just before its own
 // first read or write of global memory or, if that comes earlier, its first bounded wait, with the place of its first tile
-// worked out, and the first tiles are asked for in L2 ahead of the wait.  Between the release and the request for the first K tile 1.2 to 2.0 us went by when all threads waited
-// at one place and the producer asked for L2 itself, now 0.5; us per pass, launched one by one: four layers at 1K with scores
-// and retrieval 53.0 -> 50.0, two layers of 12 x 64 heads on a 1K cache 16.4 -> 15.8, four layers of 32 KV heads at 8K
-// 137.3 -> 135.0, eight layers of 64 query heads at 1.4K 111.1 -> 106.9.
+// worked out, and the first tiles are asked for in L2 ahead of the wait.  Between the release and the request for the first K
+// tile 1.2 to 2.0 us went by when all threads waited at one place and the producer asked for L2 itself, now 0.5; us per pass,
+// launched one by one: four layers at 1K with scores and retrieval 53.0 -> 50.0, two layers of 12 x 64 heads on a 1K cache
+// 16.4 -> 15.8, four layers of 32 KV heads at 8K 137.3 -> 135.0, eight layers of 64 query heads at 1.4K 111.1 -> 106.9.  (The
+// issuers without that wait, ahead of the release in a wait of about a second at most: 0.1 us a call less with 240 rows at 1K,
+// nothing elsewhere; with a limit that starts at the release, a state word of the CTA that every wait looks at, 0.2 us more.)
 #include <atomic>
 
 #include "common.cuh"
@@ -86,11 +88,12 @@ struct VerifyWork {
 // 15.8 -> 15.0, one with 1 row 7.3 -> 6.8, 1 row of 32 KV heads on a 1K cache 10.3 -> 9.8, 4 rows 9.6 -> 9.1.
 // (Bulk copies between the CTAs instead of stores were slower than either: 8.8, 7.7, 10.5, 8.1, 17.7, 11.2.  Through L2, (m, l)
 // passed through shared memory and a CTA's own part of its share kept in tensor memory instead of going through L2 too: 240
-// rows at 1K 12.5 -> 13.2 us a call, 60 rows of 32 KV heads at 8K 33.8 -> 34.6.)  The other way
-// round where the tiles are many: 60 rows of 32 KV heads at 8K are 0.5 us shorter through shared memory.  Each is an
-// instantiation of its own: with both in one kernel a call was 0.1 to 0.3 us longer.  The forms through shared memory spill
-// for head_dim 128 and for the device-side length (8 to 16 bytes of stack, 312 to 348 bytes of reloads), in the exchange; those
-// through L2 do not.
+// rows at 1K 12.5 -> 13.2 us a call, 60 rows of 32 KV heads at 8K 33.8 -> 34.6.)  The line at 32 rows stands where it was with two
+// meetings: more rows need more room than Q gives up.  The other way round where the tiles are many: 60 rows of 32 KV heads at 8K
+// are 0.5 us shorter through shared memory.  Each is an instantiation of its own: with both in one kernel a call was 0.1 to 0.3 us
+// longer.  The forms through shared memory spill for head_dim 128 and for the device-side length (8 bytes of stack, 328 to 352
+// bytes of reloads), in the exchange; those through L2 do not.  (Without clusters the forms without scores spill: 16 bytes of stack
+// and 180 of reloads, 8 and 48 with the device-side length.)
 struct MergeCtx {
   int cs, rank;            // CTAs of the cluster, this one
   int prob, g, rblk;       // the problem
