@@ -78,16 +78,11 @@ __device__ __forceinline__ int segments_of(const AttnPlan& p, int prob, int& slo
 
 // Chunk scores beside the merge: 256 threads of a block that merges with its others.  A block has one task, 64 rows of one key
 // tile (VW chunks); it takes the rows' statistics from the partial results instead of waiting for the lse that the merge writes.
-// All sums have a fixed order, as in score_kernel.
+// A thread has one row of every fourth KV head, of two at most.  All sums have a fixed order, as in score_kernel.
 constexpr int kScoreRows = 64;
-constexpr int kScoreMaxKv = 64;                    // KV heads whose statistics have room
+constexpr int kScoreSlices = 256 / kScoreRows, kScoreHeads = 2;
 template <int VW>
-struct ScoreRoom {
-  float part[4][kScoreRows][VW];
-  float lse2[kScoreMaxKv][kScoreRows];             // log2 of a row's sum, its maximum included
-};
-template <int VW>
-__device__ __forceinline__ void score_beside(const AttnArgs& a, ScoreRoom<VW>& sm, int tid) {
+__device__ __forceinline__ void score_beside(const AttnArgs& a, float (&part)[kScoreSlices][kScoreRows][VW], int tid) {
   const AttnPlan& p = a.plan;
   const int rr = tid & (kScoreRows - 1), slice = tid / kScoreRows;
   const int n_groups = (p.rows + kScoreRows - 1) / kScoreRows;
@@ -95,11 +90,15 @@ __device__ __forceinline__ void score_beside(const AttnArgs& a, ScoreRoom<VW>& s
   if (tile >= p.TPH) return;                       // a block that only merges
   const int nodes = kScoreRows / p.G, t0 = group * nodes;          // nodes of the group
   const float inv = 1.f / (float)p.Hq;
+  const int n_heads = r < p.rows ? (p.Hkv - slice + kScoreSlices - 1) / kScoreSlices : 0;      // heads slice, slice + 4
   sm100::pdl_wait();                               // the attention kernel's results are complete
-  if (r < p.rows) {
-    for (int g = slice; g < p.Hkv; g += 4) {
+  float lse2[kScoreHeads];                         // log2 of the row's sum, its maximum included
+#pragma unroll
+  for (int q = 0; q < kScoreHeads; ++q) {
+    lse2[q] = 0.f;
+    if (q < n_heads) {
       int slot0;
-      const int nseg = segments_of(p, g, slot0);
+      const int nseg = segments_of(p, slice + q * kScoreSlices, slot0);
       const float* pm = a.ws + p.off_part_m + (long long)slot0 * p.RB + r;
       const float* pl = a.ws + p.off_part_l + (long long)slot0 * p.RB + r;
       float M = -INFINITY, Z = 0.f;
@@ -118,53 +117,47 @@ __device__ __forceinline__ void score_beside(const AttnArgs& a, ScoreRoom<VW>& s
 #pragma unroll
         for (int k = 0; k < 12; ++k) Z = fmaf(ls[k], sm100::ex2_approx(ms[k] - M), Z);
       }
-      sm.lse2[g][rr] = M + log2f(Z);                  // (read by this thread only)
+      lse2[q] = M + log2f(Z);
+    }
+  }
+  float m[kScoreHeads][VW], ref[kScoreHeads];
+#pragma unroll
+  for (int q = 0; q < kScoreHeads; ++q) {
+    if (q < n_heads) {
+      const long long base = ((long long)(slice + q * kScoreSlices) * p.TPH + tile) * p.RB + r;
+      const float* src = a.ws + p.off_mass + base * VW;
+      if constexpr (VW == 4) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+        m[q][0] = v.x; m[q][1] = v.y; m[q][2] = v.z; m[q][3] = v.w;
+      } else if constexpr (VW == 2) {
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
+        m[q][0] = v.x; m[q][1] = v.y;
+      } else {
+        m[q][0] = __ldcg(src);
+      }
+      ref[q] = __ldcg(a.ws + p.off_mref + base);
     }
   }
   float acc[VW];
 #pragma unroll
   for (int k = 0; k < VW; ++k) acc[k] = 0.f;
-  if (r < p.rows) {
-    for (int g0 = slice; g0 < p.Hkv; g0 += 16) {
-      float m[4][VW], ref[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int g = g0 + q * 4;
-        if (g < p.Hkv) {
-          const long long base = ((long long)g * p.TPH + tile) * p.RB + r;
-          const float* src = a.ws + p.off_mass + base * VW;
-          if constexpr (VW == 4) {
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
-            m[q][0] = v.x; m[q][1] = v.y; m[q][2] = v.z; m[q][3] = v.w;
-          } else if constexpr (VW == 2) {
-            const float2 v = __ldcg(reinterpret_cast<const float2*>(src));
-            m[q][0] = v.x; m[q][1] = v.y;
-          } else {
-            m[q][0] = __ldcg(src);
-          }
-          ref[q] = __ldcg(a.ws + p.off_mref + base);
-        }
-      }
+  for (int q = 0; q < kScoreHeads; ++q) {
+    if (q < n_heads) {
+      const float f = exp2f(ref[q] - lse2[q]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int g = g0 + q * 4;
-        if (g < p.Hkv) {
-          const float f = exp2f(ref[q] - sm.lse2[g][rr]);
-#pragma unroll
-          for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[q][k], f, acc[k]);
-        }
-      }
+      for (int k = 0; k < VW; ++k) acc[k] = fmaf(m[q][k], f, acc[k]);
     }
   }
 #pragma unroll
-  for (int k = 0; k < VW; ++k) sm.part[slice][rr][k] = acc[k];
+  for (int k = 0; k < VW; ++k) part[slice][rr][k] = acc[k];
   sm100::named_bar_sync(1, 256);
   for (int o = tid; o < nodes * VW; o += 256) {
     const int tt = o / VW, k = o - tt * VW, node = t0 + tt, c = tile * VW + k;
     if (node < p.T && c < p.NC) {
       float sum = 0.f;
-      for (int s = 0; s < 4; ++s)
-        for (int j = 0; j < p.G; ++j) sum += sm.part[s][tt * p.G + j][k];
+      for (int s = 0; s < kScoreSlices; ++s)
+        for (int j = 0; j < p.G; ++j) sum += part[s][tt * p.G + j][k];
       a.chunk_score[(long long)node * p.NC + c] = sum * inv;
     }
   }
@@ -184,9 +177,9 @@ __global__ void __launch_bounds__(NT + (VW > 0 ? 256 : 0), 1) merge_kernel(const
   const AttnPlan& p = a.plan;
   sm100::pdl_launch_dependents();
   if constexpr (VW > 0) {
-    __shared__ __align__(16) ScoreRoom<VW> room;
+    __shared__ float part[kScoreSlices][kScoreRows][VW];
     if (threadIdx.x >= NT) {
-      score_beside<VW>(a, room, threadIdx.x - NT);
+      score_beside<VW>(a, part, threadIdx.x - NT);
       return;
     }
     if ((int)blockIdx.x >= n_merge) return;
@@ -334,15 +327,21 @@ int score_groups(const AttnPlan& p) { return (p.rows + kScoreRows - 1) / kScoreR
 
 // Whether the chunk scores are added up beside the merge, in one launch, or by a launch of their own that waits for it.
 // Beside, the scores wait for the attention kernel only, which saves a launch that waits for another (3 us with its own chain of
-// latencies), but a block works out its rows' statistics from all their segments: as long as every block has one task.  One scored
-// call and its retrieval, one by one, own launch / beside, 32 query / 8 KV heads: 60 nodes at 4K (128 tasks) 23.4 / 21.9 us, one
-// node at 16K (129) 29.9 / 29.7, one node of 64 heads at 18K (147) 34.6 / 34.6.  Two tasks a block, in a loop: 60 nodes at 6K
-// 24.9 / 24.1, at 8K 26.9 / 26.3, but one node at 32K 38.4 / 40.3, 16 at 30K 39.4 / 40.4; three: 60 nodes at 12K 30.3 / 30.8, one
-// at 50K 49.6 / 51.3; four and more: 60 nodes at 16K 4 us longer.  (The loop for several tasks, where every block has one: 60 nodes
-// at 4K 21.13 -> 21.05 without it, one at 16K 28.5 -> 28.0.  Started beside the merge as a launch of its own, by the merge once the
-// attention kernel was complete: 4K 23.6 -> 27.6.  A launch that was not set up ahead comes 4 us after it is asked for.)
+// latencies), but a block works out its rows' statistics from all their segments, twelve at a time and one KV head after another:
+// as long as every block has one task, a thread has two heads and a head has at most 48 segments.
+// Tasks.  One scored call and its retrieval, one by one, own launch / beside, 32 query / 8 KV heads: 60 nodes at 4K (128 tasks)
+// 23.4 / 21.9 us, one node at 16K (129) 29.9 / 29.7.  Two tasks a block, in a loop: 60 nodes at 6K 24.9 / 24.1, at 8K 26.9 / 26.3,
+// but one node at 32K 38.4 / 40.3, 16 at 30K 39.4 / 40.4; three: 60 nodes at 12K 30.3 / 30.8, one at 50K 49.6 / 51.3; four and more:
+// 60 nodes at 16K 4 us longer.  (The loop for several tasks, where every block has one: 60 nodes at 4K 21.13 -> 21.05 without it,
+// one at 16K 28.5 -> 28.0.)
+// Heads and segments.  Beside over own launch, calls of random shapes back to back, median (tenth, ninetieth percentile): 8 KV
+// heads 0.93 (0.89, 1.00) with head_dim 128, 0.99 (0.96, 1.01) with 64; up to 12 segments and 4 heads 0.88, 36 to 48 segments 1.00
+// (0.96, 1.03).  Any number of both, in a loop over the heads: 12 KV heads 1.08 (1.05, 1.09), 16 1.07 (1.04, 1.16), 32 1.12; 1 to 4
+// with 48 to 59 segments 1.02, 60 and more 1.03 to 1.13.
+// (Started beside the merge as a launch of its own, by the merge once the attention kernel was complete: 4K 23.6 -> 27.6.  A launch
+// that was not set up ahead comes 4 us after it is asked for.)
 bool scores_beside_merge(const AttnPlan& p) {
-  return p.cluster == 0 && p.C >= 32 && p.n_rblk == 1 && p.Hkv <= kScoreMaxKv &&
+  return p.cluster == 0 && p.C >= 32 && p.n_rblk == 1 && p.Hkv <= kScoreSlices * kScoreHeads && p.max_segs <= 48 &&
          p.NP * (p.RB / 32) * (p.D / 64) <= kOneWave && p.TPH * score_groups(p) <= kOneWave;
 }
 

@@ -60,8 +60,11 @@ def test_clusters_that_exchange_through_shared_memory(cuda_device, Hq, Hkv, D, T
 
 @pytest.mark.parametrize("Hq,Hkv,D,T,L,C,want", [
     (32, 8, 128, 60, 4096, 64, 2), (32, 8, 128, 60, 4700, 128, 2), (32, 8, 128, 60, 4737, 32, 3), (32, 8, 128, 37, 4000, 32, 2),
-    (32, 8, 128, 1, 16383, 32, 2), (16, 2, 64, 3, 16000, 128, 2), (32, 1, 128, 2, 14000, 32, 2),
-    (32, 8, 128, 60, 4096, 16, 3),       # chunks of fewer than 32 keys: a launch of their own
+    (32, 8, 128, 1, 16383, 32, 2), (16, 4, 128, 8, 16000, 32, 2), (32, 8, 128, 43, 78, 32, 2), (24, 6, 128, 8, 9000, 64, 2),
+    (48, 3, 128, 16, 126, 128, 2),
+    # a launch of their own: chunks of fewer than 32 keys, more than 8 KV heads, more than 48 segments
+    (32, 8, 128, 60, 4096, 16, 3), (48, 12, 128, 43, 78, 32, 3), (12, 12, 64, 9, 15607, 32, 3),
+    (16, 4, 128, 8, 18000, 32, 3), (16, 2, 64, 3, 16000, 128, 3), (32, 1, 128, 2, 14000, 32, 3),
 ])
 def test_scores_beside_the_merge(cuda_device, Hq, Hkv, D, T, L, C, want):
     assert plan(Hq, Hkv, D, T, L, C, scored=True)[1] == 0

@@ -79,8 +79,11 @@ def test_chunk_sums_of_every_class(cuda_device, kernel, Hq, Hkv, D, T, L, C):
     (32, 8, 128, 60, 4096, 64), (32, 8, 128, 60, 4700, 128),     # pairs; 37 tiles x 4 groups of 64 rows: all the blocks there are
     (32, 8, 128, 60, 4737, 32),                                  # one tile more: a launch of its own
     (32, 8, 128, 37, 4000, 32),                                  # 148 rows: two and a third groups
-    (32, 8, 128, 1, 16383, 32), (16, 2, 64, 3, 16000, 128),      # one-CTA kernel, fewer rows than a group
-    (32, 1, 128, 2, 14000, 32),                                  # one KV head, 16 and more segments a row, blocks without a merge
+    (32, 8, 128, 1, 16383, 32),                                  # one-CTA kernel, fewer rows than a group
+    (16, 4, 128, 8, 16000, 32),                                  # one head a thread, 43 segments, blocks without a merge
+    (24, 6, 128, 8, 9000, 64),                                   # two heads for two of the four slices
+    (48, 3, 128, 16, 126, 128),                                  # no head for the last slice
+    (16, 2, 64, 3, 16000, 128), (32, 1, 128, 2, 14000, 32),      # more than 48 segments: a launch of their own
 ])
 def test_chunk_scores_beside_the_merge(cuda_device, Hq, Hkv, D, T, L, C):
     w = synth.Workload("beside", Hq, Hkv, D, L, T, C, 4, "uniform", "needle", seed=T + C)
